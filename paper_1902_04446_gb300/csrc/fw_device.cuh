@@ -22,6 +22,9 @@ struct OpI32 {
   __device__ __forceinline__ static uint32_t addmin(uint32_t a, uint32_t b, uint32_t c) {
     return (uint32_t)__viaddmin_s32((int)a, (int)b, (int)c);
   }
+  __device__ __forceinline__ static uint32_t min3(uint32_t a, uint32_t b, uint32_t c) {
+    return (uint32_t)__vimin3_s32((int)a, (int)b, (int)c);
+  }
   // A-operand word for one element (same value in every lane of the word)
   __device__ __forceinline__ static uint32_t dup(elem e) { return (uint32_t)e; }
   __device__ __forceinline__ static elem inf_elem() { return (elem)1073741823; }
@@ -39,6 +42,9 @@ struct OpU16 {
   static constexpr int DTYPE = 1;
   __device__ __forceinline__ static uint32_t addmin(uint32_t a, uint32_t b, uint32_t c) {
     return __viaddmin_u16x2(a, b, c);
+  }
+  __device__ __forceinline__ static uint32_t min3(uint32_t a, uint32_t b, uint32_t c) {
+    return __vimin3_u16x2(a, b, c);
   }
   __device__ __forceinline__ static uint32_t dup(elem e) { return (uint32_t)e | ((uint32_t)e << 16); }
   __device__ __forceinline__ static elem inf_elem() { return (elem)0x7FFF; }
@@ -285,100 +291,217 @@ __device__ __forceinline__ float fmin3(float a, float b, float c) {
   asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+// How a kernel's k-loop is scheduled (chosen per kernel and element type; the
+// loops run the same operations in a different order, and ptxas's schedule and
+// register use differ with the surrounding kernel):
+//   PREFETCH  the operands of the next two k-steps are loaded into a second set
+//             of registers while the current two are computed (about 40 more
+//             registers; without it the loads wait on shared memory at the top
+//             of each pair);
+//   UNROLL    loop trips unrolled (a trip is two k-steps, or four with PREFETCH);
+//   COLS      the thread's 8 x TN block is walked column by column (one B value
+//             against all rows) instead of row by row;
+//   MIX       which outputs take the FMA-pipe form (integer ops, see
+//             tile_minplus): 0 checkerboard, 1 alternate pairs of columns,
+//             2 alternate rows, 3 alternate columns.  Always half of them.
+//             fp32: 0 A values as scalars, 1 as the loaded pairs.
+// Measured on GB300 (n = 16384, symmetric, ms per solve, best and worst of the
+// 64 combinations): int32 every round in one launch 110.0 / 132.6, per round
+// 115.4 / 130.5, packed 16-bit 63.0 / 82.5 and 72.7 / 81.0.
+template <bool PREFETCH_, int UNROLL_, bool COLS_, int MIX_>
+struct KLoop {
+  static constexpr bool PREFETCH = PREFETCH_, COLS = COLS_;
+  static constexpr int UNROLL = UNROLL_, MIX = MIX_;
+  static_assert(MIX >= 0 && MIX <= 3, "mix pattern");
+  __host__ __device__ static constexpr bool fma_form(int r, int c) {
+    return (MIX == 0 ? (r + c) & 1 : MIX == 1 ? (c >> 1) & 1 : MIX == 2 ? r & 1 : c & 1) != 0;
+  }
+};
+// Kernels with at most 128 registers a thread (Phase 2, one CTA per tile, batched).
+using KLoopSmall = KLoop<false, 1, false, 1>;
+
+// Runs compute(a, b) on every pair of k-steps: load(t, a, b) fetches the
+// operands of k-steps t and t + 1.
+template <class KL, int BK, class RegA, class RegB, class Load, class Compute>
+__device__ __forceinline__ void k_pairs(const Load &load, const Compute &compute) {
+  if constexpr (KL::PREFETCH) {
+    static_assert(BK % 4 == 0 && (BK & (BK - 1)) == 0, "k-steps in pairs of pairs");
+    RegA a0, a1;
+    RegB b0, b1;
+    load(0, a0, b0);
+    constexpr int U = KL::UNROLL;
+#pragma unroll U
+    for (int t = 0; t < BK; t += 4) {
+      load(t + 2, a1, b1);
+      compute(a0, b0);
+      load((t + 4) & (BK - 1), a0, b0);  // the last trip re-reads k-step 0: in bounds, unused
+      compute(a1, b1);
+    }
+  } else {
+    static_assert(BK % 2 == 0, "k-steps in pairs");
+    constexpr int U = KL::UNROLL;
+#pragma unroll U
+    for (int t = 0; t < BK; t += 2) {
+      RegA a;
+      RegB b;
+      load(t, a, b);
+      compute(a, b);
+    }
+  }
+}
+
 // fp32 min-plus tile, two k-steps at a time: acc = min(acc, a_t + b_t,
 // a_t+1 + b_t+1) with one three-input minimum, the sums for two neighbouring
 // columns formed by one packed pair add -- the same sums (each rounded to
 // nearest) and the same minimum as one add and one minimum per relaxation,
 // in fewer instructions.
-// U = k-step pairs per unrolled loop trip, chosen per kernel (measured on
-// GB300: every round in one launch 4, the per-round Phase 3 2, the min-plus
-// product 1; their register use and schedules differ).
-template <int BM, int BNW, int BK, int TN, int U>
+// The A values of two k-steps, as scalars or as the pairs they were loaded in
+// (the same values; the register allocation differs).
+template <bool PAIRS>
+struct RegsF32A {
+  float v[2][8];
+  __device__ __forceinline__ float at(int k, int r) const { return v[k][r]; }
+  __device__ __forceinline__ void set(int k, int h, const uint32_t *p) {
+    const float4 x = *reinterpret_cast<const float4 *>(p);
+    v[k][4 * h + 0] = x.x; v[k][4 * h + 1] = x.y; v[k][4 * h + 2] = x.z; v[k][4 * h + 3] = x.w;
+  }
+};
+template <>
+struct RegsF32A<true> {
+  uint64_t v[2][4];
+  __device__ __forceinline__ float at(int k, int r) const {
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v[k][r / 2]));
+    return (r & 1) ? y : x;
+  }
+  __device__ __forceinline__ void set(int k, int h, const uint32_t *p) {
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(p);
+    v[k][2 * h] = x.x;
+    v[k][2 * h + 1] = x.y;
+  }
+};
+template <int TN>
+struct RegsF32B {
+  uint64_t v[2][TN / 2];  // neighbouring columns (c, c + 1) as one packed pair
+};
+template <class KL, int BM, int BNW, int BK, int TN>
 __device__ __forceinline__ void tile_minplus_f32(const uint32_t *__restrict__ As, const uint32_t *__restrict__ Bs,
                                                  uint32_t (&acc)[8][TN], int ty, int tx) {
-  static_assert(BK % 2 == 0, "k-steps in pairs");
   float f[8][TN];
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
     for (int c = 0; c < TN; ++c) f[r][c] = __uint_as_float(acc[r][c]);
-  constexpr int UNROLL = TN == 8 ? U : 2;
-#pragma unroll UNROLL
-  for (int t = 0; t < BK; t += 2) {
-    float a[2][8];
-    uint64_t b[2][TN / 2];  // neighbouring columns (c, c + 1) as one packed pair
+  using RA = RegsF32A<KL::MIX == 1>;
+  auto load = [&](int t, RA &ra, RegsF32B<TN> &rb) {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const uint4 a0 = *reinterpret_cast<const uint4 *>(As + (t + k) * BM + ty * 4);
-      const uint4 a1 = *reinterpret_cast<const uint4 *>(As + (t + k) * BM + BM / 2 + ty * 4);
-      a[k][0] = __uint_as_float(a0.x); a[k][1] = __uint_as_float(a0.y);
-      a[k][2] = __uint_as_float(a0.z); a[k][3] = __uint_as_float(a0.w);
-      a[k][4] = __uint_as_float(a1.x); a[k][5] = __uint_as_float(a1.y);
-      a[k][6] = __uint_as_float(a1.z); a[k][7] = __uint_as_float(a1.w);
+      ra.set(k, 0, As + (t + k) * BM + ty * 4);
+      ra.set(k, 1, As + (t + k) * BM + BM / 2 + ty * 4);
 #pragma unroll
       for (int h = 0; h < TN / 4; ++h) {
         const ulonglong2 bv =
             *reinterpret_cast<const ulonglong2 *>(Bs + (t + k) * BNW + (h == 0 ? tx * 4 : BNW / 2 + tx * 4));
-        b[k][2 * h + 0] = bv.x;
-        b[k][2 * h + 1] = bv.y;
+        rb.v[k][2 * h + 0] = bv.x;
+        rb.v[k][2 * h + 1] = bv.y;
       }
     }
+  };
+  auto compute = [&](const RA &ra, const RegsF32B<TN> &rb) {
+    uint64_t ad[2][8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      uint64_t ad[2];
+    for (int r = 0; r < 8; ++r)
 #pragma unroll
-      for (int k = 0; k < 2; ++k) asm("mov.b64 %0, {%1, %1};" : "=l"(ad[k]) : "f"(a[k][r]));
+      for (int k = 0; k < 2; ++k) asm("mov.b64 %0, {%1, %1};" : "=l"(ad[k][r]) : "f"(ra.at(k, r)));
+    constexpr int NI = KL::COLS ? TN / 2 : 8, NJ = KL::COLS ? 8 : TN / 2;
 #pragma unroll
-      for (int p = 0; p < TN / 2; ++p) {
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const int r = KL::COLS ? j : i, p = KL::COLS ? i : j;
         uint64_t s0, s1;
-        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s0) : "l"(ad[0]), "l"(b[0][p]));
-        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s1) : "l"(ad[1]), "l"(b[1][p]));
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s0) : "l"(ad[0][r]), "l"(rb.v[0][p]));
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s1) : "l"(ad[1][r]), "l"(rb.v[1][p]));
         float x0, y0, x1, y1;
         asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(y0) : "l"(s0));
         asm("mov.b64 {%0, %1}, %2;" : "=f"(x1), "=f"(y1) : "l"(s1));
         f[r][2 * p] = fmin3(f[r][2 * p], x0, x1);
         f[r][2 * p + 1] = fmin3(f[r][2 * p + 1], y0, y1);
       }
-    }
-  }
+  };
+  k_pairs<KL, BK, RA, RegsF32B<TN>>(load, compute);
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
     for (int c = 0; c < TN; ++c) acc[r][c] = __float_as_uint(f[r][c]);
 }
 
-template <class Op, int BM, int BNW, int BK, int TN = 8, int F32U = 2>
+// 1, in a form the compiler cannot fold: a + b as a * kOne + b then stays an
+// integer multiply-add, which runs on the FMA pipe.
+__constant__ uint32_t kOne = 1;
+__device__ __forceinline__ uint32_t add_fma_pipe(uint32_t a, uint32_t b, uint32_t one) {
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(one), "r"(b));
+  return d;
+}
+
+template <int N>
+struct RegsU32 {
+  uint32_t v[2][N];
+};
+// Integer min-plus tile, two k-steps at a time.  The add-min instruction
+// (c = min(a + b, c)) issues at 64 lanes per clock per SM on the ALU pipe, and
+// with it alone the loop is bound there (measured 63.2 relaxations per clock
+// per SM) while the FMA pipe is idle.  So half of the outputs take the add-min
+// twice, and the other half form their two sums on the FMA pipe (integer
+// multiply-add by one) and take one three-input minimum: 1.5 ALU instructions
+// per output and pair of k-steps on average instead of 2 -- the same sums and
+// the same minimum.  Half is where the ALU pipe and the register-file reads
+// balance: a three-input minimum reads three fresh registers and holds the
+// issue port two cycles.  Measured with operands in shared memory and no
+// epilogue (relaxations per clock per SM, 32-bit words): no output in the FMA
+// form 63.2, a quarter 67, half 70 - 73, three quarters 65, all 53.
+// Packed 16-bit words add as plain 32-bit integers: every stored value is
+// <= 0x7FFF, so the low lane's sum never carries into the high lane.
+template <class Op, int BM, int BNW, int BK, int TN = 8, class KL = KLoopSmall>
 __device__ __forceinline__ void tile_minplus(const uint32_t *__restrict__ As, const uint32_t *__restrict__ Bs,
                                              uint32_t (&acc)[8][TN], int ty, int tx) {
   if constexpr (Op::DTYPE == 2) {
-    tile_minplus_f32<BM, BNW, BK, TN, F32U>(As, Bs, acc, ty, tx);
-    return;
-  }
-  // deeper unrolling for the 8 x 8 block (fewer loop instructions on the
-  // add-min pipe): for the integer ops 16 k-steps per loop trip measured
-  // fastest (8: 1.1 % slower on an n = 16384 int32 solve; 32 and 64: 1.5 % and
-  // 4.7 % slower, the longer bodies costing instruction fetch); fp32, two
-  // instructions per relaxation, was 2.7 % slower at 16 than at 8; the 8 x 4
-  // block of the 512-thread kernel must stay within 128 registers
-  constexpr int UNROLL = TN == 8 ? (Op::DTYPE == 2 ? 8 : 16) : 4;
-#pragma unroll UNROLL
-  for (int t = 0; t < BK; ++t) {
-    const uint4 a0 = *reinterpret_cast<const uint4 *>(As + t * BM + ty * 4);
-    const uint4 a1 = *reinterpret_cast<const uint4 *>(As + t * BM + BM / 2 + ty * 4);
-    const uint32_t a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-    uint32_t b[TN];
+    tile_minplus_f32<KL, BM, BNW, BK, TN>(As, Bs, acc, ty, tx);
+  } else {
+    const uint32_t one = kOne;
+    auto load = [&](int t, RegsU32<8> &ra, RegsU32<TN> &rb) {
 #pragma unroll
-    for (int h = 0; h < TN / 4; ++h) {
-      const uint4 bv = *reinterpret_cast<const uint4 *>(Bs + t * BNW + (h == 0 ? tx * 4 : BNW / 2 + tx * 4));
-      b[4 * h + 0] = bv.x;
-      b[4 * h + 1] = bv.y;
-      b[4 * h + 2] = bv.z;
-      b[4 * h + 3] = bv.w;
-    }
+      for (int k = 0; k < 2; ++k) {
+        const uint4 a0 = *reinterpret_cast<const uint4 *>(As + (t + k) * BM + ty * 4);
+        const uint4 a1 = *reinterpret_cast<const uint4 *>(As + (t + k) * BM + BM / 2 + ty * 4);
+        ra.v[k][0] = a0.x; ra.v[k][1] = a0.y; ra.v[k][2] = a0.z; ra.v[k][3] = a0.w;
+        ra.v[k][4] = a1.x; ra.v[k][5] = a1.y; ra.v[k][6] = a1.z; ra.v[k][7] = a1.w;
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+        for (int h = 0; h < TN / 4; ++h) {
+          const uint4 bv = *reinterpret_cast<const uint4 *>(Bs + (t + k) * BNW + (h == 0 ? tx * 4 : BNW / 2 + tx * 4));
+          rb.v[k][4 * h + 0] = bv.x;
+          rb.v[k][4 * h + 1] = bv.y;
+          rb.v[k][4 * h + 2] = bv.z;
+          rb.v[k][4 * h + 3] = bv.w;
+        }
+      }
+    };
+    auto compute = [&](const RegsU32<8> &ra, const RegsU32<TN> &rb) {
+      constexpr int NI = KL::COLS ? TN : 8, NJ = KL::COLS ? 8 : TN;
 #pragma unroll
-      for (int c = 0; c < TN; ++c) acc[r][c] = Op::addmin(a[r], b[c], acc[r][c]);
+      for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          const int r = KL::COLS ? j : i, c = KL::COLS ? i : j;
+          if (KL::fma_form(r, c))
+            acc[r][c] = Op::min3(add_fma_pipe(ra.v[0][r], rb.v[0][c], one), add_fma_pipe(ra.v[1][r], rb.v[1][c], one),
+                                 acc[r][c]);
+          else
+            acc[r][c] = Op::addmin(ra.v[1][r], rb.v[1][c], Op::addmin(ra.v[0][r], rb.v[0][c], acc[r][c]));
+        }
+    };
+    k_pairs<KL, BK, RegsU32<8>, RegsU32<TN>>(load, compute);
   }
 }
 

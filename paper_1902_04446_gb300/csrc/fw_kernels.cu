@@ -326,6 +326,13 @@ struct P3T {
   static constexpr int SMEM = 2 * STAGE_BYTES + P3T_C_BYTES + 1024;
 };
 
+// The first 1024-byte boundary of the dynamic shared memory.  Written as an
+// offset added to the array, so that the compiler still knows the pointer is in
+// shared memory: rounding the address as an integer made every operand fetch
+// of the k-loops a generic load (n = 16384 int32 per round with the loop of
+// tile_minplus: 129.9 ms generic, 118.6 - 124.6 ms shared).
+__device__ __forceinline__ uint8_t *align_smem(uint8_t *raw) { return raw + ((0u - smem_addr(raw)) & 1023u); }
+
 // TN = 8: 256 threads with 8 x 8 words each; TN = 4: 512 threads with 8 x 4
 // words each (twice the warps per SM to hide instruction latency).
 // Symmetric mode (sym = 1): only tiles (ty, tx) with tx >= ty / EPW -- the
@@ -356,7 +363,7 @@ __global__ void __launch_bounds__(TileMap<128, 128, TN>::THREADS, 1)
   __shared__ __align__(8) uint64_t bar_ab[2];
   __shared__ __align__(8) uint64_t bar_c;
   __shared__ int abort_flag;
-  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
   // stage s: A at base + s * STAGE, B right after it; C after both stages
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * P3T_STAGE_BYTES); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * P3T_STAGE_BYTES) + BK * BM; };
@@ -534,6 +541,29 @@ __device__ __forceinline__ void red_tail_store(int32_t *D, int64_t ld, int64_t n
   }
 }
 
+// Schedules of the warp-specialized kernels' k-loops (KLoop, fw_device.cuh).
+// Per element type the fastest measured of prefetch x unroll x walk x mix on
+// n = 16384 solves (one launch per round at widths 64 and 128, every round in
+// one launch) and on a 4096-cubed product; fp32 has no mix.
+template <class Op, int BK>
+struct P3Loop {
+  using Round = KLoop<true, 1, true, 1>;
+  using Solve = KLoop<true, 2, true, 0>;
+  using Product = KLoop<true, 2, true, 0>;
+};
+template <int BK>
+struct P3Loop<OpU16, BK> {
+  using Round = KLoop<true, 1, false, 2>;
+  using Solve = KLoop<false, 1, false, 1>;
+  using Product = KLoop<false, 1, false, 3>;
+};
+template <int BK>
+struct P3Loop<OpF32, BK> {
+  using Round = KLoop<true, 1, true, 0>;
+  using Solve = KLoop<false, 2, true, 0>;
+  using Product = KLoop<false, 4, true, 1>;
+};
+
 template <class Op, int BK, bool RED>
 __global__ void __launch_bounds__(P3W_THREADS, 1)
     fw_phase3_ws(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
@@ -548,7 +578,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_ab[2], empty_ab[2], full_c, cdone, cfree;
   __shared__ int abort_flag;
-  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE) + KS * BM; };
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
@@ -710,7 +740,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
         const int j = i * NSPLIT + h, s = j & 1;
         bad = !mbar_wait_bounded(&full_ab[s], (uint32_t)(j >> 1) & 1u, P3T_WAIT_LIMIT);
         if (__any_sync(0xffffffffu, bad)) break;
-        tile_minplus<Op, BM, BNW, KS, TN>(stA(s), stB(s), acc, ty, tx);
+        tile_minplus<Op, BM, BNW, KS, TN, typename P3Loop<Op, BK>::Round>(stA(s), stB(s), acc, ty, tx);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty_ab[s]);
       }
@@ -1033,7 +1063,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   __shared__ __align__(8) uint64_t full_ab[2], empty_ab[2], full_c, cdone, cfree;
   __shared__ int slot_kind[2], slot_info[2], slot_round[2];
   __shared__ int abort_flag;
-  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE) + BK * BM; };
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
@@ -1393,7 +1423,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
         for (int r = 0; r < 8; ++r)
 #pragma unroll
           for (int c = 0; c < TN; ++c) acc[r][c] = Op::INF_WORD;
-        tile_minplus<Op, BM, BNW, BK, TN, 4>(stA(s), stB(s), acc, ty, tx);
+        tile_minplus<Op, BM, BNW, BK, TN, typename P3Loop<Op, BK>::Solve>(stA(s), stB(s), acc, ty, tx);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty_ab[s]);
         const int64_t r0 = (int64_t)cty * BM, c0 = (int64_t)ctx * BNW * Op::EPW;
@@ -1581,7 +1611,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_ab[2], empty_ab[2], full_c, cdone, cfree;
   __shared__ int abort_flag;
-  uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE) + BK * BM; };
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
@@ -1685,7 +1715,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
         if (lane == 0) abort_flag = 1;
         break;
       }
-      tile_minplus<Op, BM, BNW, BK, TN, 1>(stA(s), stB(s), acc, ty, tx);
+      tile_minplus<Op, BM, BNW, BK, TN, typename P3Loop<Op, BK>::Product>(stA(s), stB(s), acc, ty, tx);
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty_ab[s]);
       if (c != nk - 1) continue;
