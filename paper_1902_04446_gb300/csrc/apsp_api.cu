@@ -272,8 +272,8 @@ apsp_status run_rounds_locked(apsp_handle *h, int dtype, void *D, int64_t n, int
   }
   if (h->cfg.symmetric == 1 || (h->cfg.symmetric == 0 && known_sym)) {
     rc.sym = true;
-  } else if (h->cfg.symmetric == 0 && n > 1 && apsp::single_launch(dtype, D, ld, n, rc)) {
-    // device check of W == W^T whose answer the single launch reads itself:
+  } else if (h->cfg.symmetric == 0 && n > 1 && apsp::device_sym(dtype, D, ld, n, rc)) {
+    // device check of W == W^T whose answer the kernels read themselves:
     // no host round trip before the rounds are enqueued
     int *flag = h->d_status + 1;
     e = cudaMemsetAsync(flag, 0, sizeof(int), s);
@@ -1353,8 +1353,8 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
     } else if (h->cfg.symmetric == 0) {
       int *dflag = g->status + 2;  // zeroed with the status words
       if (apsp::launch_symmetry_check(APSP_I32, rs[0]->D, rn, rn, dflag, s) != cudaSuccess) return APSP_E_CUDA;
-      if (apsp::single_launch(APSP_I32, rs[0]->D, rn, rn, rc)) {
-        rc.sym_flag = dflag;  // every round in one launch: the kernel reads the answer itself
+      if (apsp::device_sym(APSP_I32, rs[0]->D, rn, rn, rc)) {
+        rc.sym_flag = dflag;  // the kernels read the answer themselves
       } else {
         // one launch per round: the answer is read back before the rounds are enqueued
         int flag = 0;

@@ -445,6 +445,19 @@ __device__ __forceinline__ uint32_t add_fma_pipe(uint32_t a, uint32_t b, uint32_
   return d;
 }
 
+// One word of two relaxations: min(v, a0 + b0, a1 + b1), by the add-min twice
+// or (alt) in the form with half the ALU instructions (see tile_minplus).
+template <class Op>
+__device__ __forceinline__ uint32_t word_update2(uint32_t v, uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1,
+                                                 bool alt, uint32_t one) {
+  if constexpr (Op::DTYPE == 2)
+    return __float_as_uint(fmin3(__uint_as_float(v), __uint_as_float(a0) + __uint_as_float(b0),
+                                 __uint_as_float(a1) + __uint_as_float(b1)));
+  else
+    return alt ? Op::min3(add_fma_pipe(a0, b0, one), add_fma_pipe(a1, b1, one), v)
+               : Op::addmin(a1, b1, Op::addmin(a0, b0, v));
+}
+
 template <int N>
 struct RegsU32 {
   uint32_t v[2][N];
@@ -494,11 +507,8 @@ __device__ __forceinline__ void tile_minplus(const uint32_t *__restrict__ As, co
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
           const int r = KL::COLS ? j : i, c = KL::COLS ? i : j;
-          if (KL::fma_form(r, c))
-            acc[r][c] = Op::min3(add_fma_pipe(ra.v[0][r], rb.v[0][c], one), add_fma_pipe(ra.v[1][r], rb.v[1][c], one),
-                                 acc[r][c]);
-          else
-            acc[r][c] = Op::addmin(ra.v[1][r], rb.v[1][c], Op::addmin(ra.v[0][r], rb.v[0][c], acc[r][c]));
+          acc[r][c] = word_update2<Op>(acc[r][c], ra.v[0][r], rb.v[0][c], ra.v[1][r], rb.v[1][c], KL::fma_form(r, c),
+                                       one);
         }
     };
     k_pairs<KL, BK, RegsU32<8>, RegsU32<TN>>(load, compute);

@@ -28,12 +28,14 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include <cudaTypedefs.h>
 
 #include "fw_device.cuh"
 #include "fw_launch.h"
+#include "fw_panels.cuh"
 #include "fw_tasks.cuh"
 #include "tma.cuh"
 
@@ -564,11 +566,29 @@ struct P3Loop<OpF32, BK> {
   using Product = KLoop<false, 4, true, 1>;
 };
 
+// What a Phase-3 launch is told besides its tiles.
+template <class Op>
+struct P3Round {
+  int sym;                             // symmetric mode, unless sym_flag decides it on the device
+  const int *sym_flag;                 // nullable: symmetric when the int is 0
+  int tiles_x, tiles_y;                // the tile grid
+  int tiles_gen, tiles_sym;            // processed tiles without and with the symmetric mode
+  int64_t q0;                          // first row of the next round's diagonal block; < 0: no next_diag task
+  const uint32_t *colT;                // next_diag: the panels of this round
+  int64_t ldT;
+  const typename Op::elem *symB;
+  DiagBuf *diag;                       // next_diag: where the closed block goes
+};
+
+// With a next_diag task (round width 64), block 0 runs it before its tiles: the
+// task costs about as much as one tile, so it counts as one in the split of the
+// tiles over the CTAs.
 template <class Op, int BK, bool RED>
 __global__ void __launch_bounds__(P3W_THREADS, 1)
     fw_phase3_ws(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                 const __grid_constant__ CUtensorMap mapC, typename Op::elem *__restrict__ D, Layout L, int64_t n,
-                 int64_t p0, int64_t p1, int tiles_x, int tiles_total, int *err, int sym, int tiles_y) {
+                 const __grid_constant__ CUtensorMap mapBs, const __grid_constant__ CUtensorMap mapC,
+                 typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0, int64_t p1, int *err,
+                 const P3Round<Op> rd) {
   constexpr int BM = 128, BNW = 128, TN = 8;
   using Map = TileMap<BM, BNW, TN>;
   constexpr int NCW = Map::THREADS / 32;  // consumer warps
@@ -584,11 +604,8 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int per = tiles_total / (int)gridDim.x, extra = tiles_total % (int)gridDim.x;
-  const int t_begin = (int)blockIdx.x * per + min((int)blockIdx.x, extra);
-  const int t_end = t_begin + per + ((int)blockIdx.x < extra ? 1 : 0);
+  const int tiles_x = rd.tiles_x, tiles_y = rd.tiles_y;
   pdl_trigger();
-  if (t_begin >= t_end) return;
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&full_ab[i], 1);
@@ -605,6 +622,25 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   }
   __syncthreads();
   pdl_wait();  // the round's panels (previous launches) are complete from here on
+  const int sym = rd.sym_flag ? (__ldcg(rd.sym_flag) == 0 ? 1 : 0) : rd.sym;
+  const CUtensorMap &mapP = sym ? mapBs : mapB;  // the B operand: the symmetric panel, or D's rows
+  const int chain = (BK == 64 && rd.q0 >= 0) ? 1 : 0;
+  const int items = (sym ? rd.tiles_sym : rd.tiles_gen) + chain;
+  const int per = items / (int)gridDim.x, extra = items % (int)gridDim.x;
+  const int i_begin = (int)blockIdx.x * per + min((int)blockIdx.x, extra);
+  const int i_end = i_begin + per + ((int)blockIdx.x < extra ? 1 : 0);
+  const int t_begin = max(i_begin - chain, 0), t_end = i_end - chain;  // item 0 is the next_diag task
+  if constexpr (BK == 64) {
+    if (chain && blockIdx.x == 0) {
+      static_assert(sizeof(NextDiagSmem<Op>) <= P3T_C_BYTES, "next_diag runs in the C buffer");
+      if (warp < NCW)
+        next_diag<Op, Bar256>(D, L, n, p0, rd.q0, rd.colT, rd.ldT, sym ? rd.symB : nullptr, rd.diag,
+                              *reinterpret_cast<NextDiagSmem<Op> *>(Cs), tid);
+      fence_proxy_async_smem();  // the C buffer's next accesses may be TMA's
+      __syncthreads();
+    }
+  }
+  if (t_begin >= t_end) return;
 
   // first tile of this CTA and the row-major step over the (symmetric) tile set
   int ty0, tx0;
@@ -651,7 +687,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
       auto issue_ab = [&](int ty_, int tx_, int h, int s) {
         mbar_arrive_expect_tx(&full_ab[s], STAGE);
         tma_load_2d(stA(s), &mapA, &full_ab[s], ty_ * BM, h * KS);
-        tma_load_2d(stB(s), &mapB, &full_ab[s], tx_ * BNW * Op::EPW, (sym ? 0 : (int)p0) + h * KS);
+        tma_load_2d(stB(s), &mapP, &full_ab[s], tx_ * BNW * Op::EPW, (sym ? 0 : (int)p0) + h * KS);
         if (s == 0) ++n_ab[0];
         else ++n_ab[1];
       };
@@ -2080,6 +2116,9 @@ static void launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
   cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);  // errors surface in cudaGetLastError
 }
 
+// Largest n whose panels are cut into 16-word chunks (otherwise 32 words).
+constexpr int64_t kNarrowPanelN = 6144;
+
 template <class Op, int BK>
 static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64_t ldT, bool vec, int variant,
                                cudaStream_t s, int64_t *launches, PhaseTimer *tm, int *wait_err, bool sym,
@@ -2106,9 +2145,10 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
   // upper-triangular storage: symmetric mode on the warp-specialized Phase 3,
   // one launch per round
   if (tri && (!sym || !vec || variant != 3)) return cudaErrorNotSupported;
-  // the device picks the symmetric mode (single launch only; otherwise the
-  // general path, which is exact for any input)
-  const bool dev_sym = la_on && !sym && sym_flag != nullptr;
+  // the device picks the symmetric mode (the single launch, and the
+  // warp-specialized kernel at width 64; otherwise the general path, which is
+  // exact for any input)
+  bool dev_sym = (la_on || (BK == 64 && use_tma && vec && variant == 3)) && !sym && sym_flag != nullptr;
   const bool any_sym = sym || dev_sym;
   uint32_t *colTb[2], *colT = static_cast<uint32_t *>(colTv);
   colTb[0] = colT;
@@ -2129,8 +2169,11 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
   constexpr int SMEM3 = (BK * C3::BM + BK * C3::BNW) * 4;
   constexpr int KS = P3T<BK>::KS;  // k-steps per stage of the TMA Phase-3 kernels (box height of the A/B maps)
   // the attributes are per device, so they are set on every call (a cheap host call)
-  cudaError_t e = cudaFuncSetAttribute(fw_phase2<Op, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, C2::SMEM);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if constexpr (BK != 64) {
+    e = cudaFuncSetAttribute(fw_phase2<Op, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, C2::SMEM);
+    if (e != cudaSuccess) return e;
+  }
   if constexpr (BK > 64) {
     e = cudaFuncSetAttribute(fw_phase1_w128<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(P1Smem<Op, 128>));
@@ -2183,18 +2226,21 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
     }
   }
   la_on = la_on && tma;
+  dev_sym = dev_sym && tma;
   if (!la_on) {
     colTb[1] = colT;
     rowPb[1] = rowP;
   }
   const int tiles_x = (int)((n + 128 * Op::EPW - 1) / (128 * Op::EPW));
   const int tiles_y = (int)((n + 127) / 128);
-  int tiles_total = tiles_x * tiles_y;
-  if (sym) {  // tiles with tx >= ty / EPW
-    tiles_total = 0;
-    for (int y = 0; y < tiles_y; ++y) tiles_total += tiles_x - std::min(tiles_x, y / Op::EPW);
-  }
+  const int tiles_gen = tiles_x * tiles_y;
+  int tiles_sym = 0;  // tiles with tx >= ty / EPW
+  for (int y = 0; y < tiles_y; ++y) tiles_sym += tiles_x - std::min(tiles_x, y / Op::EPW);
+  const int tiles_total = sym ? tiles_sym : tiles_gen;
   const int grid_tma = std::min(sms, tiles_total);
+  // width 64: the warp-specialized Phase 3 closes the next round's diagonal block
+  const bool chain = BK == 64 && tma && variant == 3 && !la_on;
+  DiagBuf *diag = reinterpret_cast<DiagBuf *>(colT + panel_rows64_words(ldT));
   const int nrow = (int)((n + C2::ROW_BNW * Op::EPW - 1) / (C2::ROW_BNW * Op::EPW));
   const int ncol = (int)((n + C2::COL_BM - 1) / C2::COL_BM);
   const dim3 g3((unsigned)((n + C3::BNW * Op::EPW - 1) / (C3::BNW * Op::EPW)), (unsigned)((n + C3::BM - 1) / C3::BM));
@@ -2202,7 +2248,37 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
     p0 = k * BK;
     p1 = (p0 + BK < n) ? p0 + BK : n;
   };
-  // Phase 1 and Phase 2 of round k as their own launches, into panel cT / rP
+  // Width 64: the panels of round k in one launch, after the closure of its
+  // diagonal block where the previous round's Phase 3 has not done that.
+  auto panels64 = [&](int64_t k) {
+    int64_t p0, p1;
+    span(k, p0, p1);
+    const double w = (double)(p1 - p0), rest = (double)(n - (p1 - p0));
+    if (k == 0 || !chain) {
+      if (tm) tm->before(0, s);
+      launch_pdl(fw_diag<Op>, dim3(1), dim3(256), 0, s, (const Elem *)D, L, n, p0, diag);
+      if (launches) *launches += 1;
+      if (tm) tm->after(0, s, w * w * w);
+    }
+    if (tm) tm->before(1, s);
+    if (q == 1) {
+      launch_pdl(diag_to_matrix<Op>, dim3(1), dim3(1024), 0, s, D, L, n, p0, (const DiagBuf *)diag);
+    } else {
+      const int64_t band = 128 * Op::EPW, b0 = p0 / band * band;
+      auto go = [&](auto xw) {
+        constexpr int XW = decltype(xw)::value;
+        const int64_t nx = (n + XW * Op::EPW - 1) / (XW * Op::EPW);
+        launch_pdl(fw_panels<Op, XW>, dim3((unsigned)(sym ? nx : 2 * nx)), dim3(PANEL_THREADS), 0, s, D, L, n, p0, colT,
+                   ldT, rowP, (const DiagBuf *)diag, vec ? 1 : 0, sym ? 1 : 0, dev_sym ? sym_flag : (const int *)nullptr,
+                   b0, b0 + band);
+      };
+      if (n <= kNarrowPanelN) go(std::integral_constant<int, 16>());
+      else go(std::integral_constant<int, 32>());
+    }
+    if (launches) *launches += 1;
+    if (tm) tm->after(1, s, sym ? rest * w * w : 2.0 * rest * w * w);
+  };
+  // Widths 32 and 128: Phase 1 and Phase 2 of round k as their own launches.
   auto panels = [&](int64_t k, uint32_t *cT, Elem *rP) {
     int64_t p0, p1;
     span(k, p0, p1);
@@ -2248,20 +2324,33 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
     int64_t p0, p1;
     span(k, p0, p1);
     const double w = (double)(p1 - p0), rest = (double)(n - (p1 - p0));
-    const double frac = sym ? (double)tiles_total / ((double)tiles_x * tiles_y) : 1.0;
-    return rest * rest * w * frac;
+    return rest * rest * w * ((double)tiles_total / tiles_gen);
   };
   if (!la_on) {
     for (int64_t k = 0; k < q; ++k) {
       int64_t p0, p1;
       span(k, p0, p1);
-      panels(k, colT, rowP);
+      if constexpr (BK == 64) panels64(k);
+      else panels(k, colT, rowP);
       if (q == 1) break;
       if (tm) tm->before(2, s);
-      if (tma && variant == 3)
-        launch_pdl(fw_phase3_ws<Op, BK, kRedOp<Op>>, dim3(grid_tma), dim3(P3W_THREADS), (size_t)P3T<BK>::SMEM, s,
-                   mA[0], mB[0], mC, D, L, n, p0, p1, tiles_x, tiles_total, err, sym ? 1 : 0, tiles_y);
-      else if constexpr (BK <= 64) {
+      if (tma && variant == 3) {
+        P3Round<Op> rd{};
+        rd.sym = sym ? 1 : 0;
+        rd.sym_flag = dev_sym ? sym_flag : nullptr;
+        rd.tiles_x = tiles_x;
+        rd.tiles_y = tiles_y;
+        rd.tiles_gen = tiles_gen;
+        rd.tiles_sym = tiles_sym;
+        rd.q0 = chain && k + 1 < q ? p0 + BK : -1;
+        rd.colT = colT;
+        rd.ldT = ldT;
+        rd.symB = any_sym ? symB_any(0) : nullptr;
+        rd.diag = diag;
+        const int grid = std::min(sms, tiles_total + (rd.q0 >= 0 ? 1 : 0));
+        launch_pdl(fw_phase3_ws<Op, BK, kRedOp<Op>>, dim3(grid), dim3(P3W_THREADS), (size_t)P3T<BK>::SMEM, s, mA[0],
+                   mB[0], dev_sym ? mBs[0] : mB[0], mC, D, L, n, p0, p1, err, rd);
+      } else if constexpr (BK <= 64) {
         if (tma && variant == 2)
           fw_phase3_tma<Op, BK, 4><<<grid_tma, TileMap<128, 128, 4>::THREADS, P3T<BK>::SMEM, s>>>(
               mA[0], mB[0], mC, D, ld, n, p0, p1, tiles_x, tiles_total, err, sym ? 1 : 0, tiles_y);
@@ -2273,13 +2362,12 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
       } else
         fw_phase3<Op, BK><<<g3, C3::THREADS, SMEM3, s>>>(D, ld, n, p0, p1, colT, ldT, vec ? 1 : 0, symB_of(0));
       if (launches) *launches += 1;
-      if (tm) tm->after(2, s, p3_work(k));
+      if (tm && dev_sym) tm->after_choice(2, s, p3_work(k) * tiles_sym / tiles_gen, p3_work(k), sym_flag);
+      else if (tm) tm->after(2, s, p3_work(k));
     }
   } else if constexpr (kLookaheadWidth<BK>) {
     // every round in one persistent launch (fw_solve_ws)
     constexpr bool RED = kRedOp<Op>;
-    int tiles_sym = 0;  // tiles with tx >= ty / EPW
-    for (int y = 0; y < tiles_y; ++y) tiles_sym += tiles_x - std::min(tiles_x, y / Op::EPW);
     const int grid = std::min(sms, tiles_sym);  // one launch grid for either mode
     char *cbase = reinterpret_cast<char *>(colT) + lookahead_counter_offset(ldT);
     double work[2] = {0.0, 0.0};
@@ -2371,6 +2459,11 @@ static cudaError_t rounds_bk(const RoundConfig &cfg, void *D, Layout L, int64_t 
 bool single_launch(int dtype, const void *D, int64_t ld, int64_t n, const RoundConfig &cfg) {
   const size_t es = dtype == 1 ? 2 : 4;
   return cfg.p3 == 4 && cfg.bk == 64 && n > 64 && aligned16(D, ld, es);
+}
+
+bool device_sym(int dtype, const void *D, int64_t ld, int64_t n, const RoundConfig &cfg) {
+  const size_t es = dtype == 1 ? 2 : 4;
+  return (cfg.p3 == 3 || cfg.p3 == 4) && cfg.bk == 64 && n > 1 && aligned16(D, ld, es);
 }
 
 cudaError_t launch_symmetry_check(int dtype, const void *D, int64_t n, int64_t ld, int *flag, cudaStream_t s) {

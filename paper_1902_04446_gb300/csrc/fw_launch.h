@@ -37,7 +37,7 @@ struct PhaseTimer {
 // one symmetric panel, and a final pass mirrors the upper triangle into the
 // lower; rowP is the BK x ldT element panel that packed 16-bit needs for it
 // (row_panel_bytes(ldT, p3 == 4)).
-// sym_flag (device int, kernel 4 only): the symmetric mode is decided on the
+// sym_flag (device int, where device_sym() holds): the symmetric mode is decided on the
 // device -- symmetric when the int is 0 (as left by launch_symmetry_check) --
 // so the host need not wait for the check; rowP must then be allocated.
 struct RoundConfig {
@@ -54,6 +54,10 @@ struct RoundConfig {
 // Whether launch_rounds would run every round in one launch for this call
 // (kernel 4 with round width 64, a 16-byte addressable D and more than one round).
 bool single_launch(int dtype, const void *D, int64_t ld, int64_t n, const RoundConfig &cfg);
+// Whether launch_rounds can take cfg.sym_flag for this call: the symmetric mode
+// decided on the device, by the single launch or by the warp-specialized kernel
+// at width 64.
+bool device_sym(int dtype, const void *D, int64_t ld, int64_t n, const RoundConfig &cfg);
 // The default Phase-3 kernel for (n, dtype) when nothing was tuned: every round
 // in one launch for mid-size n, one launch per round below and above (timed per
 // n and dtype on GB300, the per-round kernels with programmatic dependent
@@ -90,6 +94,11 @@ constexpr int64_t kMaxRoundWidth = 128;  // panel buffers are sized for this (th
 // Phase-3 kernel 4 (every round in one launch, `all_rounds`) two of them, a
 // 64-bit item counter, 6 counters per round (round width >= 32) and one per
 // Phase-3 tile.
+// Rounds of width up to 64 use 64 rows of the panel; behind them (at
+// panel_rows64_words(ldT)) lies the closed diagonal block of the next round
+// (DiagBuf, fw_panels.cuh).
+constexpr size_t kDiagBufBytes = 2 * 64 * 64 * 4;
+inline size_t panel_rows64_words(int64_t ldT) { return 64 * (size_t)ldT; }
 inline size_t lookahead_counter_offset(int64_t ldT) { return 2 * (size_t)kMaxRoundWidth * (size_t)ldT * 4; }
 inline size_t panel_buffer_bytes(int64_t n, int64_t ldT, bool all_rounds) {
   const size_t one = (size_t)kMaxRoundWidth * (size_t)ldT * 4;

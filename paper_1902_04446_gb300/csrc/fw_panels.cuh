@@ -1,0 +1,305 @@
+// The 64-wide rounds' panels (the paper's Sec. 4.4/4.5, Alg. 3 and 4): Phase 2
+// as one kernel of narrow chunks, and the closure of the next round's diagonal
+// block as a task of this round's Phase 3.
+//
+// With one launch per phase, a round of a small or mid-size matrix was bound
+// by the chain diagonal closure -> panels -> tiles: at n = 2048 38 us, of which
+// the tiles' add-mins need 7.  Here a round is two launches:
+//   fw_panels   relaxes every chunk of the panels with the closed diagonal
+//               block (16 or 32 words wide, so that a small n still fills the
+//               GPU), and publishes them: D, colT, and in symmetric mode the
+//               element panel and the band elements below the diagonal;
+//   Phase 3     whose first CTA, before its tiles, applies this round's update
+//               to the next diagonal block and closes it (next_diag), into a
+//               side buffer that the next fw_panels reads and copies into D.
+// Closing into the side buffer keeps D's block to one writer: the Phase-3 tile
+// that holds it.
+#pragma once
+#include "fw_launch.h"
+#include "fw_tasks.cuh"
+#include "tma.cuh"
+
+namespace apsp {
+
+// A closed 64 x 64 diagonal block as A-operand words, in both orders:
+// t[s][i] = word(D[p0 + i][p0 + s]), n[s][i] = word(D[p0 + s][p0 + i]);
+// entries outside the matrix are INF.
+struct alignas(16) DiagBuf {
+  uint32_t t[64][64];
+  uint32_t n[64][64];
+};
+static_assert(sizeof(DiagBuf) == kDiagBufBytes, "placed after the 64 panel rows of a 64-wide round");
+
+template <class Op>
+__device__ __forceinline__ typename Op::elem word_elem(uint32_t w) {
+  return bits_elem<Op>(Op::EPW == 2 ? (w & 0xFFFFu) : w);
+}
+
+template <class Op, class S>
+__device__ __forceinline__ void store_diag(DiagBuf *out, const S (&s)[64][68], int tid) {
+  for (int idx = tid; idx < 64 * 64; idx += 256) {
+    const int a = idx / 64, b = idx % 64;
+    out->n[a][b] = Op::dup(Op::from_s(s[a][b]));
+    out->t[a][b] = Op::dup(Op::from_s(s[b][a]));
+  }
+}
+
+// Closes D's diagonal block at p0 into `out` (256 threads).
+template <class Op>
+__global__ void __launch_bounds__(256) fw_diag(const typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
+                                               DiagBuf *__restrict__ out) {
+  __shared__ P1Smem<Op, 64> sm;
+  typename Op::scalar v[4][4];
+  const int tid = threadIdx.x;
+  pdl_trigger();
+  pdl_wait();
+  load_block<Op, 64, 256, true, CtaBar>(D, L, n, p0, sm.s, v, tid);
+  close_block<Op, 64, CtaBar>(sm.s, v, tid / 16, tid % 16);
+  store_diag<Op>(out, sm.s, tid);
+}
+
+// Closed D block copied back (a matrix of one round has no fw_panels).
+template <class Op>
+__global__ void diag_to_matrix(typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
+                               const DiagBuf *__restrict__ diag) {
+  pdl_trigger();
+  pdl_wait();
+  for (int idx = threadIdx.x; idx < 64 * 64; idx += blockDim.x) {
+    const int64_t r = p0 + idx / 64, c = p0 + idx % 64;
+    if (r < n && c < n) D[L.off(r, c)] = word_elem<Op>(__ldcg(&diag->n[idx / 64][idx % 64]));
+  }
+}
+
+// Barrier of the 256 threads that run next_diag inside a larger CTA.
+struct Bar256 {
+  __device__ __forceinline__ static void sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+};
+
+template <class Op>
+struct NextDiagSmem {
+  P1Smem<Op, 64> p1;
+  alignas(16) typename Op::scalar a[64][64];  // a[t][i]: this round's column panel at the next block's rows
+  alignas(16) typename Op::scalar b[64][64];  // b[t][j]: its row panel at the next block's columns
+};
+
+// The next round's diagonal block (at q0) after this round's update, closed,
+// into `out`; 256 threads.  D's block may or may not hold this round's update
+// yet (its Phase-3 tile runs meanwhile): the minimum is the same.
+// symB: symmetric mode's panel (64 x ldT elements), else nullptr and the row
+// panel is D's rows p0 ...
+template <class Op, class Bar>
+__device__ __noinline__ void next_diag(const typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
+                                       int64_t q0, const uint32_t *__restrict__ colT, int64_t ldT,
+                                       const typename Op::elem *__restrict__ symB, DiagBuf *__restrict__ out,
+                                       NextDiagSmem<Op> &sm, int tid) {
+  using S = typename Op::scalar;
+  constexpr int IT = 64 * 64 / 256;
+  const S INF = Op::to_s(Op::inf_elem());
+  {
+    S ta[IT], tb[IT];
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int t = (tid + k * 256) / 64, i = tid % 64;
+      ta[k] = Op::to_s(word_elem<Op>(__ldcg(colT + (int64_t)t * ldT + q0 + i)));
+      if (symB) tb[k] = Op::to_s(__ldcg(symB + (int64_t)t * ldT + q0 + i));
+      else tb[k] = (p0 + t < n && q0 + i < n) ? Op::to_s(__ldcg(D + L.off(p0 + t, q0 + i))) : INF;
+    }
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int t = (tid + k * 256) / 64, i = tid % 64;
+      // rows and columns past the matrix: the panel is not defined there
+      sm.a[t][i] = q0 + i < n ? ta[k] : INF;
+      sm.b[t][i] = q0 + i < n ? tb[k] : INF;
+    }
+  }
+  S v[4][4];
+  load_block<Op, 64, 256, true, Bar>(D, L, n, q0, sm.p1.s, v, tid);
+  const int by = tid / 16, bx = tid % 16;
+  const uint32_t one = kOne;
+#pragma unroll 4
+  for (int t = 0; t < 64; t += 2) {
+    S a[2][4], b[2][4];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      lds_vec<4>(a[k], &sm.a[t + k][by * 4]);
+      lds_vec<4>(b[k], &sm.b[t + k][bx * 4]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[r][c] = s_update2<Op>(v[r][c], a[0][r], b[0][c], a[1][r], b[1][c], (r + c) & 1, one);
+  }
+  // every thread has read its part of s (load_block) before this write-back:
+  // the block it writes is its own
+#pragma unroll
+  for (int r = 0; r < 4; ++r) sts_vec<4>(&sm.p1.s[by * 4 + r][bx * 4], v[r]);
+  Bar::sync();
+  close_block<Op, 64, Bar>(sm.p1.s, v, by, bx);
+  store_diag<Op>(out, sm.p1.s, tid);
+}
+
+// ---------------------------------------------------------------- panels
+// One chunk of the panels per CTA: XW words (XE = XW * EPW elements) of
+// columns x0 .. x0 + XE of the row panel, or as many rows of the column panel.
+// Both are out[t][x] = min(S[t][x], min_s A[s][t] + S[s][x]) on the chunk held
+// as S[t][x]: row panel S[t][x] = D[p0 + t][x] and A = diag.t, column panel
+// S[t][x] = D[x][p0 + t] (loaded and stored transposed) and A = diag.n.
+//   symmetric mode: chunk c is a column chunk left of the diagonal block, a row
+//     chunk right of it (only the upper triangle is kept), and its result is
+//     the symmetric panel: colT words, rowP elements (packed 16-bit), and in
+//     the tile band of the diagonal block both D[p0 + t][x] and D[x][p0 + t];
+//   otherwise chunks 0 .. nx-1 are row chunks, nx .. 2 nx - 1 column chunks
+//     (their result also goes to colT).
+// The diagonal block's own chunks copy the closed block.  A chunk never
+// straddles the diagonal block (XE divides 64).
+constexpr int PANEL_THREADS = 128;
+template <class Op, int XW>
+struct PanelSmem {
+  uint32_t a[64][64];
+  // the chunk's words; rows padded so that the transposed accesses (one
+  // element of 8 consecutive t per thread) spread over the banks
+  uint32_t s[64][XW + 4];
+};
+
+template <class Op, int XW>
+__global__ void __launch_bounds__(PANEL_THREADS)
+    fw_panels(typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0, uint32_t *__restrict__ colT,
+              int64_t ldT, typename Op::elem *__restrict__ rowP, const DiagBuf *__restrict__ diag, int vec, int sym,
+              const int *__restrict__ sym_flag, int64_t band_start, int64_t band_end) {
+  using E = typename Op::elem;
+  constexpr int EPW = Op::EPW, XE = XW * EPW, CW = XW / 8;  // words per thread and row
+  constexpr int E4 = 4 * EPW;
+  static_assert(64 % XE == 0 || XE == 64, "a chunk never straddles the diagonal block");
+  __shared__ __align__(16) PanelSmem<Op, XW> sm;
+  const int tid = threadIdx.x;
+  const int nx = (int)((n + XE - 1) / XE);
+  pdl_trigger();
+  pdl_wait();
+  if (sym_flag) sym = __ldcg(sym_flag) == 0;
+  if (sym && (int)blockIdx.x >= nx) return;
+  const bool second = (int)blockIdx.x >= nx;
+  const int64_t x0 = (int64_t)((int)blockIdx.x - (second ? nx : 0)) * XE;
+  const bool on_diag = x0 >= p0 && x0 < p0 + 64;
+  const bool col = sym ? x0 < p0 : second;
+  const bool to_colT = sym || col;
+  const bool wr_row = sym ? x0 >= band_start : !col;
+  const bool wr_col = sym ? x0 < band_end : col;
+  if (on_diag) {
+    const int d0 = (int)(x0 - p0);
+    for (int idx = tid; idx < 64 * XE; idx += PANEL_THREADS) {
+      const int t = idx / XE, x = idx % XE;
+      const uint32_t wn = __ldcg(&diag->n[t][d0 + x]);
+      if (!col && p0 + t < n && x0 + x < n) D[L.off(p0 + t, x0 + x)] = word_elem<Op>(wn);
+      if (to_colT) colT[(int64_t)t * ldT + x0 + x] = __ldcg(&diag->t[t][d0 + x]);
+      if (sym && rowP) rowP[(int64_t)t * ldT + x0 + x] = word_elem<Op>(wn);
+    }
+    return;
+  }
+  // ---- operands: the closed block, and the chunk (all loads first)
+  constexpr int AIT = 64 * 16 / PANEL_THREADS;
+  constexpr int SIT = 64 * (XW / 4) / PANEL_THREADS;  // 16-byte pieces per thread
+  const uint32_t *A = col ? &diag->n[0][0] : &diag->t[0][0];
+  uint4 va[AIT], vs[SIT];
+#pragma unroll
+  for (int k = 0; k < AIT; ++k) va[k] = __ldcg(reinterpret_cast<const uint4 *>(A) + tid + k * PANEL_THREADS);
+#pragma unroll
+  for (int k = 0; k < SIT; ++k) {
+    const int idx = tid + k * PANEL_THREADS;
+    if (!col) vs[k] = load_chunk<Op, true>(D, L, n, n, p0 + idx / (XW / 4), x0 + (idx % (XW / 4)) * E4, vec);
+    else vs[k] = load_chunk<Op, true>(D, L, n, n, x0 + idx / (64 / E4), p0 + (idx % (64 / E4)) * E4, vec);
+  }
+#pragma unroll
+  for (int k = 0; k < AIT; ++k) *(reinterpret_cast<uint4 *>(sm.a) + tid + k * PANEL_THREADS) = va[k];
+  E *se = reinterpret_cast<E *>(sm.s);           // the chunk as elements
+  constexpr int SE = (XW + 4) * EPW;             // elements per row of it
+#pragma unroll
+  for (int k = 0; k < SIT; ++k) {
+    const int idx = tid + k * PANEL_THREADS;
+    if (!col) {
+      *reinterpret_cast<uint4 *>(&sm.s[idx / (XW / 4)][(idx % (XW / 4)) * 4]) = vs[k];
+    } else {
+      const int x = idx / (64 / E4), t = (idx % (64 / E4)) * E4;
+#pragma unroll
+      for (int e = 0; e < E4; ++e) se[(t + e) * SE + x] = bits_elem<Op>(chunk_get<Op>(vs[k], e));
+    }
+  }
+  __syncthreads();
+  // ---- out = min(S, A (x) S): 4 rows x CW words per thread
+  const int ty = tid / 8, tx = tid % 8;
+  uint32_t acc[4][CW];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < CW; ++c) acc[r][c] = sm.s[4 * ty + r][tx * CW + c];
+  const uint32_t one = kOne;
+#pragma unroll 4
+  for (int k = 0; k < 64; k += 2) {
+    uint32_t a[2][4], b[2][CW];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint4 av = *reinterpret_cast<const uint4 *>(&sm.a[k + h][4 * ty]);
+      a[h][0] = av.x; a[h][1] = av.y; a[h][2] = av.z; a[h][3] = av.w;
+#pragma unroll
+      for (int c = 0; c < CW; c += 2) {
+        const uint2 bv = *reinterpret_cast<const uint2 *>(&sm.s[k + h][tx * CW + c]);
+        b[h][c] = bv.x;
+        b[h][c + 1] = bv.y;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < CW; ++c) acc[r][c] = word_update2<Op>(acc[r][c], a[0][r], b[0][c], a[1][r], b[1][c], (r + c) & 1, one);
+  }
+  // ---- results
+  const int64_t xw = x0 + (int64_t)tx * CW * EPW;  // first element of this thread's words
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int t = 4 * ty + r;
+#pragma unroll
+    for (int c = 0; c < CW; c += 2) {
+      const int64_t x = xw + c * EPW;
+      const uint2 w2 = make_uint2(acc[r][c], acc[r][c + 1]);
+      if (to_colT) {
+        uint32_t *cw = colT + (int64_t)t * ldT + x;
+        if constexpr (EPW == 1) *reinterpret_cast<uint2 *>(cw) = w2;
+        else
+          *reinterpret_cast<uint4 *>(cw) = make_uint4(Op::dup(w2.x & 0xFFFFu), Op::dup(w2.x >> 16),
+                                                      Op::dup(w2.y & 0xFFFFu), Op::dup(w2.y >> 16));
+      }
+      if (sym && EPW == 2) *reinterpret_cast<uint2 *>(rowP + (int64_t)t * ldT + x) = w2;
+      if (wr_row && p0 + t < n) {
+        E *dp = D + L.off(p0 + t, x);
+        if (vec && x + 2 * EPW <= n) {
+          *reinterpret_cast<uint2 *>(dp) = w2;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 2 * EPW; ++e) {
+            const uint32_t w = e < EPW ? w2.x : w2.y;
+            if (x + e < n) dp[e] = bits_elem<Op>(EPW == 2 ? ((e & 1) ? (w >> 16) : (w & 0xFFFFu)) : w);
+          }
+        }
+      }
+    }
+  }
+  if (!wr_col) return;
+  // transposed through shared memory: D[x][p0 + t], 16 bytes of one row a store
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < CW; ++c) sm.s[4 * ty + r][tx * CW + c] = acc[r][c];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < SIT; ++k) {
+    const int idx = tid + k * PANEL_THREADS;
+    const int x = idx / (64 / E4), t = (idx % (64 / E4)) * E4;
+    if (x0 + x >= n) continue;
+    uint4 v = make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int e = 0; e < E4; ++e) chunk_set<Op>(v, e, elem_bits<Op>(se[(t + e) * SE + x]));
+    store_chunk<Op>(D, L, x0 + x, p0 + t, v, col_mask<Op>(p0 + t, n, 0, 0), vec);
+  }
+}
+
+}  // namespace apsp

@@ -13,6 +13,8 @@
 // CG = true reads everything through L2 (ld.global.cg), which is required when
 // the producer of the data ran earlier in the same launch.
 #pragma once
+#include <type_traits>
+
 #include "fw_device.cuh"
 
 namespace apsp {
@@ -37,8 +39,148 @@ __device__ __forceinline__ T ld_elem(const T *p) {
 // columns bx*PT + c (PT = BK / 16) in registers.
 template <class Op, int BK>
 struct P1Smem {
-  typename Op::scalar s[BK][BK + 4];
+  alignas(16) typename Op::scalar s[BK][BK + 4];
 };
+
+template <class S>
+__device__ __forceinline__ S bits_scalar(int w) {
+  if constexpr (std::is_same<S, float>::value) return __int_as_float(w);
+  else return w;
+}
+__device__ __forceinline__ int scalar_bits(int x) { return x; }
+__device__ __forceinline__ int scalar_bits(float x) { return __float_as_int(x); }
+
+// N (2 or 4) consecutive scalars by one shared-memory access; p is aligned to N of them.
+template <int N, class S>
+__device__ __forceinline__ void lds_vec(S (&x)[N], const S *p) {
+  static_assert(sizeof(S) == 4 && (N == 2 || N == 4), "8- or 16-byte accesses");
+  if constexpr (N == 4) {
+    const int4 q = *reinterpret_cast<const int4 *>(p);
+    const int w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = bits_scalar<S>(w[i]);
+  } else {
+    const int2 q = *reinterpret_cast<const int2 *>(p);
+    x[0] = bits_scalar<S>(q.x);
+    x[1] = bits_scalar<S>(q.y);
+  }
+}
+template <int N, class S>
+__device__ __forceinline__ void sts_vec(S *p, const S (&x)[N]) {
+  if constexpr (N == 4)
+    *reinterpret_cast<int4 *>(p) = make_int4(scalar_bits(x[0]), scalar_bits(x[1]), scalar_bits(x[2]), scalar_bits(x[3]));
+  else
+    *reinterpret_cast<int2 *>(p) = make_int2(scalar_bits(x[0]), scalar_bits(x[1]));
+}
+
+// v = min(v, a0 + b0, a1 + b1): the add-min twice, or (alt) both sums and one
+// three-input minimum, which takes half the ALU instructions (integer sums on
+// the FMA pipe; see tile_minplus).
+template <class Op>
+__device__ __forceinline__ typename Op::scalar s_update2(typename Op::scalar v, typename Op::scalar a0,
+                                                         typename Op::scalar b0, typename Op::scalar a1,
+                                                         typename Op::scalar b1, bool alt, uint32_t one) {
+  if constexpr (Op::DTYPE == 2) return fmin3(v, a0 + b0, a1 + b1);
+  else if (alt)
+    return __vimin3_s32(v, (int)add_fma_pipe((uint32_t)a0, (uint32_t)b0, one),
+                        (int)add_fma_pipe((uint32_t)a1, (uint32_t)b1, one));
+  else return Op::s_addmin(a1, b1, Op::s_addmin(a0, b0, v));
+}
+
+// Closes the BK x BK block held in s (and, block by block, in v) in place.
+//
+// The pivots are taken two at a time, t0 and t0 + 1: with the corner's
+// off-diagonal entries k01 and k10, the net effect of those two Floyd-Warshall
+// steps on entry (i, j) is min(D_ij, a0' + b0, a1' + b1), where a0' =
+// min(a0, a1 + k10) and a1' = min(a1, a0 + k01) are the row's pivot-column
+// values and b0, b1 the pivot-row values of column j.  (Terms through a
+// diagonal entry are left out: weights are >= 0, so they never improve.)  Every
+// sum has two stored values, so it cannot overflow.  Then the owners of the
+// next two pivots' rows and columns write them back, and one barrier per pivot
+// pair orders the steps.  A write-back that lands while another thread still
+// reads this pair's pivot columns only replaces a0, a1 by a0', a1', from which
+// the same a0', a1' follow.
+// The block is on every round's critical path and bound by latency and by the
+// redundant work that saves barriers.  Add-mins per thread and four pivots:
+// one at a time 64 and four barriers, two at a time 84 and two, four at a time
+// (closing a 4 x 4 corner in every thread) 148 - 192 and one.
+template <class Op, int BK, class Bar = CtaBar>
+__device__ __forceinline__ void close_block(typename Op::scalar (&s)[BK][BK + 4],
+                                            typename Op::scalar (&v)[BK / 16][BK / 16], int by, int bx) {
+  using S = typename Op::scalar;
+  constexpr int PT = BK / 16, PAIRS = PT / 2;
+  static_assert(PT % 2 == 0, "an even number of pivots per thread block");
+  const uint32_t one = kOne;
+#pragma unroll 1
+  for (int p = 0; p < 16; ++p) {
+#pragma unroll
+    for (int h = 0; h < PAIRS; ++h) {
+      const int t0 = p * PT + 2 * h;
+      S a[PT][2], b[2][PT];
+      const S k01 = s[t0][t0 + 1], k10 = s[t0 + 1][t0];
+#pragma unroll
+      for (int r = 0; r < PT; ++r) lds_vec<2>(a[r], &s[by * PT + r][t0]);
+      lds_vec<PT>(b[0], &s[t0][bx * PT]);
+      lds_vec<PT>(b[1], &s[t0 + 1][bx * PT]);
+#pragma unroll
+      for (int r = 0; r < PT; ++r) {
+        const S a0 = Op::s_addmin(a[r][1], k10, a[r][0]), a1 = Op::s_addmin(a[r][0], k01, a[r][1]);
+#pragma unroll
+        for (int c = 0; c < PT; ++c) v[r][c] = s_update2<Op>(v[r][c], a0, b[0][c], a1, b[1][c], (r + c) & 1, one);
+      }
+      // the next pair: rows / columns n0, n0 + 1 of thread block nb
+      const int nb = (h + 1 < PAIRS) ? p : p + 1;
+      constexpr int last = PAIRS - 1;
+      const int n0 = (h == last) ? 0 : 2 * h + 2;
+      if (nb < 16) {
+        if (by == nb) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) sts_vec<PT>(&s[nb * PT + n0 + i][bx * PT], v[n0 + i]);
+        }
+        if (bx == nb) {
+#pragma unroll
+          for (int r = 0; r < PT; ++r) {
+            const S w[2] = {v[r][n0], v[r][n0 + 1]};
+            sts_vec<2>(&s[by * PT + r][nb * PT + n0], w);
+          }
+        }
+      }
+      Bar::sync();
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < PT; ++r) sts_vec<PT>(&s[by * PT + r][bx * PT], v[r]);
+  Bar::sync();
+}
+
+// The block's entries into s and, thread by thread, v.
+template <class Op, int BK, int NT, bool CG, class Bar>
+__device__ __forceinline__ void load_block(const typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
+                                           typename Op::scalar (&s)[BK][BK + 4],
+                                           typename Op::scalar (&v)[BK / 16][BK / 16], int tid) {
+  using S = typename Op::scalar;
+  constexpr int PT = BK / 16;
+  const S INF = Op::to_s(Op::inf_elem());
+  // all of this thread's loads first, then the shared-memory stores
+  constexpr int IT = BK * BK / NT;
+  S tmp[IT];
+#pragma unroll
+  for (int k = 0; k < IT; ++k) {
+    const int idx = tid + k * NT;
+    const int64_t r = p0 + idx / BK, c = p0 + idx % BK;
+    tmp[k] = (r < n && c < n) ? Op::to_s(ld_elem<CG>(D + L.off(r, c))) : INF;
+  }
+#pragma unroll
+  for (int k = 0; k < IT; ++k) {
+    const int idx = tid + k * NT;
+    s[idx / BK][idx % BK] = tmp[k];
+  }
+  Bar::sync();
+#pragma unroll
+  for (int r = 0; r < PT; ++r)
+#pragma unroll
+    for (int c = 0; c < PT; ++c) v[r][c] = s[(tid / 16) * PT + r][(tid % 16) * PT + c];
+}
 
 template <class Op, int BK, int NT, bool CG, class Bar = CtaBar>
 __device__ __forceinline__ void phase1_body(typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
@@ -50,88 +192,9 @@ __device__ __forceinline__ void phase1_body(typename Op::elem *__restrict__ D, L
   static_assert(BK % G == 0 && NT == G * G, "phase 1 layout");
   auto &s = sm.s;
   const int by = tid / G, bx = tid % G;
-  const S INF = Op::to_s(Op::inf_elem());
-  {
-    // all of this thread's loads first, then the shared-memory stores
-    constexpr int IT = BK * BK / NT;
-    S tmp[IT];
-#pragma unroll
-    for (int k = 0; k < IT; ++k) {
-      const int idx = tid + k * NT;
-      const int64_t r = p0 + idx / BK, c = p0 + idx % BK;
-      tmp[k] = (r < n && c < n) ? Op::to_s(ld_elem<CG>(D + L.off(r, c))) : INF;
-    }
-#pragma unroll
-    for (int k = 0; k < IT; ++k) {
-      const int idx = tid + k * NT;
-      s[idx / BK][idx % BK] = tmp[k];
-    }
-  }
-  Bar::sync();
   S v[PT][PT];
-#pragma unroll
-  for (int r = 0; r < PT; ++r)
-#pragma unroll
-    for (int c = 0; c < PT; ++c) v[r][c] = s[by * PT + r][bx * PT + c];
-  // The pivots are taken PT at a time, t0 = p*PT .. t0+PT-1 (the rows and
-  // columns of thread block p): the net effect of those PT Floyd-Warshall steps
-  // on entry (i, j) is min(D_ij, min_{s,s'} D_i,t0+s + K*_ss' + D_t0+s',j), K*
-  // the closure of the PT x PT corner at (t0, t0).  Every thread closes K itself
-  // (PT^3 add-mins), forms a' = a (x) K* for its rows (a = its pivot-column
-  // values, kept with a' >= a, so every sum has two terms and cannot overflow)
-  // and applies a' (x) b (b = the pivot-row values of its columns).  Then the
-  // owners of the next pivot block's rows and columns write their blocks back,
-  // and one barrier per pivot block (not per pivot) orders the steps.  A
-  // write-back that lands while another thread still reads this block's
-  // pivot column only replaces a value by its own update a', which gives the
-  // same a' again (K* is closed).
-#pragma unroll 1
-  for (int p = 0; p < G; ++p) {
-    const int t0 = p * PT;
-    S K[PT][PT], a[PT][PT], b[PT][PT];
-#pragma unroll
-    for (int i = 0; i < PT; ++i)
-#pragma unroll
-      for (int j = 0; j < PT; ++j) {
-        K[i][j] = s[t0 + i][t0 + j];
-        a[i][j] = s[by * PT + i][t0 + j];
-        b[i][j] = s[t0 + i][bx * PT + j];
-      }
-#pragma unroll
-    for (int m = 0; m < PT; ++m)
-#pragma unroll
-      for (int i = 0; i < PT; ++i)
-#pragma unroll
-        for (int j = 0; j < PT; ++j) K[i][j] = Op::s_addmin(K[i][m], K[m][j], K[i][j]);
-    S a2[PT][PT];
-#pragma unroll
-    for (int r = 0; r < PT; ++r)
-#pragma unroll
-      for (int j = 0; j < PT; ++j) {
-        S x = a[r][j];
-#pragma unroll
-        for (int i = 0; i < PT; ++i) x = Op::s_addmin(a[r][i], K[i][j], x);
-        a2[r][j] = x;
-      }
-#pragma unroll
-    for (int r = 0; r < PT; ++r)
-#pragma unroll
-      for (int c = 0; c < PT; ++c)
-#pragma unroll
-        for (int j = 0; j < PT; ++j) v[r][c] = Op::s_addmin(a2[r][j], b[j][c], v[r][c]);
-    if (p + 1 < G && (by == p + 1 || bx == p + 1)) {
-#pragma unroll
-      for (int r = 0; r < PT; ++r)
-#pragma unroll
-        for (int c = 0; c < PT; ++c) s[by * PT + r][bx * PT + c] = v[r][c];
-    }
-    Bar::sync();
-  }
-#pragma unroll
-  for (int r = 0; r < PT; ++r)
-#pragma unroll
-    for (int c = 0; c < PT; ++c) s[by * PT + r][bx * PT + c] = v[r][c];
-  Bar::sync();
+  load_block<Op, BK, NT, CG, Bar>(D, L, n, p0, s, v, tid);
+  close_block<Op, BK, Bar>(s, v, by, bx);
   for (int idx = tid; idx < BK * BK; idx += NT) {
     const int i = idx / BK, j = idx % BK;
     const int64_t r = p0 + i, c = p0 + j;

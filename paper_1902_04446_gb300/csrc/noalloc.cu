@@ -25,9 +25,9 @@
 
 namespace {
 
-// panel buffer: 64 rows (the widest round) x APSP_NOALLOC_MAX_N words, then 64
-// words of which the first is the wait flag
-constexpr int64_t kPanelWords = 64 * (int64_t)APSP_NOALLOC_MAX_N;
+// panel buffer: 64 rows (the widest round) x APSP_NOALLOC_MAX_N words and the
+// next round's diagonal block, then 64 words of which the first is the wait flag
+constexpr int64_t kPanelWords = 64 * (int64_t)APSP_NOALLOC_MAX_N + (int64_t)apsp::kDiagBufBytes / 4;
 static_assert(APSP_NOALLOC_MAX_N % 256 == 0, "panel rows are padded to 256 words");
 
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kPanelWords + 64];
