@@ -53,21 +53,26 @@ __global__ void __launch_bounds__(P1_THREADS) fw_phase1(typename Op::elem *__res
   phase1_body<Op, BK, P1_THREADS, false>(D, L, n, p0, colT, ldT, s, threadIdx.x);
 }
 
-// Phase 1 of a 128-wide round: the pivot-block scheme of phase1_body
-// (fw_tasks.cuh) on a 32 x 32 grid of threads, each owning a 4 x 4 block of
-// D_kk in registers (1024 threads, at most 64 registers each).  Per pivot
+// Phase 1 of a 128-wide round, four pivots a step on a 32 x 32 grid of threads,
+// each owning a 4 x 4 block of D_kk in registers (1024 threads, at most 64
+// registers each; a barrier of 32 warps costs more than the extra work that
+// four pivots a step bring).  Per pivot
 // block p (pivots 4p .. 4p+3) every thread closes the 4 x 4 corner K, then
 // for each of its rows r forms a' = a (x) K* from the row's pivot-column
 // values a (read from shared memory one row at a time, which keeps the
 // registers within the limit) and lowers its row by a' (x) b, b = the
-// pivot-row values of its columns.  Reading a later than phase1_body does is
-// covered by the same argument: a value written back meanwhile is a' itself,
+// pivot-row values of its columns.  A write-back that lands while another
+// thread still reads this block's pivot columns only replaces a by a' itself,
 // and a' (x) K* = a' since K* is closed.  Outputs as phase1_body: D_kk, the
 // transposed panel rows in colT and, with rowP, the element panel.
 constexpr int P1W_THREADS = 1024;
 template <class Op>
+struct P1WSmem {
+  typename Op::scalar s[128][128 + 4];
+};
+template <class Op>
 __device__ __forceinline__ void phase1_body_w128(typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
-                                                 uint32_t *__restrict__ colT, int64_t ldT, P1Smem<Op, 128> &sm,
+                                                 uint32_t *__restrict__ colT, int64_t ldT, P1WSmem<Op> &sm,
                                                  int tid, typename Op::elem *__restrict__ rowP) {
   using S = typename Op::scalar;
   constexpr int BK = 128, G = 32, PT = 4, NT = P1W_THREADS;
@@ -156,7 +161,7 @@ __global__ void __launch_bounds__(P1W_THREADS) fw_phase1_w128(typename Op::elem 
   extern __shared__ __align__(16) uint8_t p1w_raw[];
   pdl_trigger();
   pdl_wait();
-  phase1_body_w128<Op>(D, L, n, p0, colT, ldT, *reinterpret_cast<P1Smem<Op, 128> *>(p1w_raw), threadIdx.x, rowP);
+  phase1_body_w128<Op>(D, L, n, p0, colT, ldT, *reinterpret_cast<P1WSmem<Op> *>(p1w_raw), threadIdx.x, rowP);
 }
 
 // shared-memory loaders: load_As_colT, load_Bs_rows, load_As_transposed (fw_device.cuh)
@@ -634,7 +639,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
     if (chain && blockIdx.x == 0) {
       static_assert(sizeof(NextDiagSmem<Op>) <= P3T_C_BYTES, "next_diag runs in the C buffer");
       if (warp < NCW)
-        next_diag<Op, Bar256>(D, L, n, p0, rd.q0, rd.colT, rd.ldT, sym ? rd.symB : nullptr, rd.diag,
+        next_diag<Op, Bar256>(D, L, n, p0, rd.q0, rd.colT, rd.ldT, sym ? rd.symB : nullptr, 1, rd.diag,
                               *reinterpret_cast<NextDiagSmem<Op> *>(Cs), tid);
       fence_proxy_async_smem();  // the C buffer's next accesses may be TMA's
       __syncthreads();
@@ -2176,7 +2181,7 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
   }
   if constexpr (BK > 64) {
     e = cudaFuncSetAttribute(fw_phase1_w128<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(P1Smem<Op, 128>));
+                             (int)sizeof(P1WSmem<Op>));
     if (e != cudaSuccess) return e;
   }
   e = cudaFuncSetAttribute(fw_phase3<Op, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM3);
@@ -2285,7 +2290,7 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
     const double w = (double)(p1 - p0), rest = (double)(n - (p1 - p0));
     if (tm) tm->before(0, s);
     if constexpr (BK > 64)
-      launch_pdl(fw_phase1_w128<Op>, dim3(1), dim3(P1W_THREADS), sizeof(P1Smem<Op, 128>), s, D, L, n, p0, cT, ldT,
+      launch_pdl(fw_phase1_w128<Op>, dim3(1), dim3(P1W_THREADS), sizeof(P1WSmem<Op>), s, D, L, n, p0, cT, ldT,
                  sym ? rP : nullptr);
     else if (sym && rP)
       launch_pdl(fw_phase1_sym<Op, BK>, dim3(1), dim3(P1_THREADS), 0, s, D, L, n, p0, cT, ldT, rP);

@@ -35,12 +35,15 @@ __device__ __forceinline__ typename Op::elem word_elem(uint32_t w) {
   return bits_elem<Op>(Op::EPW == 2 ? (w & 0xFFFFu) : w);
 }
 
-template <class Op, class S>
-__device__ __forceinline__ void store_diag(DiagBuf *out, const S (&s)[64][68], int tid) {
-  for (int idx = tid; idx < 64 * 64; idx += 256) {
-    const int a = idx / 64, b = idx % 64;
-    out->n[a][b] = Op::dup(Op::from_s(s[a][b]));
-    out->t[a][b] = Op::dup(Op::from_s(s[b][a]));
+template <class Op>
+__device__ __forceinline__ void store_diag(DiagBuf *out, const typename Op::scalar (&v)[4][4], int tid) {
+  const int i0 = (tid / 16) * 4, j0 = (tid % 16) * 4;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) store_words<Op>(&out->n[i0 + r][j0], v[r]);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const typename Op::scalar x[4] = {v[0][c], v[1][c], v[2][c], v[3][c]};
+    store_words<Op>(&out->t[j0 + c][i0], x);
   }
 }
 
@@ -53,9 +56,9 @@ __global__ void __launch_bounds__(256) fw_diag(const typename Op::elem *__restri
   const int tid = threadIdx.x;
   pdl_trigger();
   pdl_wait();
-  load_block<Op, 64, 256, true, CtaBar>(D, L, n, p0, sm.s, v, tid);
-  close_block<Op, 64, CtaBar>(sm.s, v, tid / 16, tid % 16);
-  store_diag<Op>(out, sm.s, tid);
+  load_block<Op, 64, true>(D, L, n, p0, v, tid);
+  close_block<Op, 64, CtaBar>(sm, v, tid);
+  store_diag<Op>(out, v, tid);
 }
 
 // Closed D block copied back (a matrix of one round has no fw_panels).
@@ -90,30 +93,49 @@ struct NextDiagSmem {
 template <class Op, class Bar>
 __device__ __noinline__ void next_diag(const typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
                                        int64_t q0, const uint32_t *__restrict__ colT, int64_t ldT,
-                                       const typename Op::elem *__restrict__ symB, DiagBuf *__restrict__ out,
-                                       NextDiagSmem<Op> &sm, int tid) {
+                                       const typename Op::elem *__restrict__ symB, int vec,
+                                       DiagBuf *__restrict__ out, NextDiagSmem<Op> &sm, int tid) {
   using S = typename Op::scalar;
-  constexpr int IT = 64 * 64 / 256;
-  const S INF = Op::to_s(Op::inf_elem());
+  constexpr int E4 = 4 * Op::EPW, BIT = 64 * 64 / E4 / 256;
+  S v[4][4];
   {
-    S ta[IT], tb[IT];
+    // all loads first: the panels' 64 x 64 parts and this thread's part of the
+    // block.  Rows and columns past the matrix read as INF.
+    uint4 ta[4], tb[BIT];
 #pragma unroll
-    for (int k = 0; k < IT; ++k) {
-      const int t = (tid + k * 256) / 64, i = tid % 64;
-      ta[k] = Op::to_s(word_elem<Op>(__ldcg(colT + (int64_t)t * ldT + q0 + i)));
-      if (symB) tb[k] = Op::to_s(__ldcg(symB + (int64_t)t * ldT + q0 + i));
-      else tb[k] = (p0 + t < n && q0 + i < n) ? Op::to_s(__ldcg(D + L.off(p0 + t, q0 + i))) : INF;
+    for (int k = 0; k < 4; ++k)
+      ta[k] = load_chunk<OpI32, true>(reinterpret_cast<const int32_t *>(colT), ldT, 64, ldT, (tid + k * 256) / 16,
+                                      q0 + (tid % 16) * 4, true);
+#pragma unroll
+    for (int k = 0; k < BIT; ++k) {
+      const int t = (tid + k * 256) / (64 / E4);
+      const int64_t x = q0 + (tid % (64 / E4)) * E4;
+      tb[k] = symB ? load_chunk<Op, true>(symB, ldT, 64, n, t, x, true)
+                   : load_chunk<Op, true>(D, L, n, n, p0 + t, x, vec != 0);
+    }
+    load_block<Op, 64, true>(D, L, n, q0, v, tid);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int t = (tid + k * 256) / 16, i = (tid % 16) * 4;
+      const uint32_t w[4] = {ta[k].x, ta[k].y, ta[k].z, ta[k].w};
+      S x[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] = Op::to_s(q0 + i + e < n ? word_elem<Op>(w[e]) : Op::inf_elem());
+      sts_vec<4>(&sm.a[t][i], x);
     }
 #pragma unroll
-    for (int k = 0; k < IT; ++k) {
-      const int t = (tid + k * 256) / 64, i = tid % 64;
-      // rows and columns past the matrix: the panel is not defined there
-      sm.a[t][i] = q0 + i < n ? ta[k] : INF;
-      sm.b[t][i] = q0 + i < n ? tb[k] : INF;
+    for (int k = 0; k < BIT; ++k) {
+      const int t = (tid + k * 256) / (64 / E4), i = (tid % (64 / E4)) * E4;
+#pragma unroll
+      for (int g = 0; g < E4; g += 4) {
+        S x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = Op::to_s(bits_elem<Op>(chunk_get<Op>(tb[k], g + e)));
+        sts_vec<4>(&sm.b[t][i + g], x);
+      }
     }
   }
-  S v[4][4];
-  load_block<Op, 64, 256, true, Bar>(D, L, n, q0, sm.p1.s, v, tid);
+  Bar::sync();
   const int by = tid / 16, bx = tid % 16;
   const uint32_t one = kOne;
 #pragma unroll 4
@@ -129,13 +151,8 @@ __device__ __noinline__ void next_diag(const typename Op::elem *__restrict__ D, 
 #pragma unroll
       for (int c = 0; c < 4; ++c) v[r][c] = s_update2<Op>(v[r][c], a[0][r], b[0][c], a[1][r], b[1][c], (r + c) & 1, one);
   }
-  // every thread has read its part of s (load_block) before this write-back:
-  // the block it writes is its own
-#pragma unroll
-  for (int r = 0; r < 4; ++r) sts_vec<4>(&sm.p1.s[by * 4 + r][bx * 4], v[r]);
-  Bar::sync();
-  close_block<Op, 64, Bar>(sm.p1.s, v, by, bx);
-  store_diag<Op>(out, sm.p1.s, tid);
+  close_block<Op, 64, Bar>(sm.p1, v, tid);
+  store_diag<Op>(out, v, tid);
 }
 
 // ---------------------------------------------------------------- panels

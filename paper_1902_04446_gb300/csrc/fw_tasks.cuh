@@ -34,12 +34,13 @@ __device__ __forceinline__ T ld_elem(const T *p) {
 }
 
 // ---------------------------------------------------------------- Phase 1
-// Needs blockDim.x == NT (NT = 256) and BK * (BK + 4) scalars of shared memory.
-// Thread (by, bx) of a 16 x 16 grid owns the PT x PT block of rows by*PT + r,
-// columns bx*PT + c (PT = BK / 16) in registers.
+// 256 threads: thread (by, bx) of a 16 x 16 grid owns the PT x PT block of rows
+// by*PT + r, columns bx*PT + c (PT = BK / 16) in registers; the pivot's row and
+// column pass through shared memory, double buffered.
 template <class Op, int BK>
 struct P1Smem {
-  alignas(16) typename Op::scalar s[BK][BK + 4];
+  alignas(16) typename Op::scalar row[2][BK];
+  alignas(16) typename Op::scalar col[2][BK];
 };
 
 template <class S>
@@ -87,99 +88,83 @@ __device__ __forceinline__ typename Op::scalar s_update2(typename Op::scalar v, 
   else return Op::s_addmin(a1, b1, Op::s_addmin(a0, b0, v));
 }
 
-// Closes the BK x BK block held in s (and, block by block, in v) in place.
-//
-// The pivots are taken two at a time, t0 and t0 + 1: with the corner's
-// off-diagonal entries k01 and k10, the net effect of those two Floyd-Warshall
-// steps on entry (i, j) is min(D_ij, a0' + b0, a1' + b1), where a0' =
-// min(a0, a1 + k10) and a1' = min(a1, a0 + k01) are the row's pivot-column
-// values and b0, b1 the pivot-row values of column j.  (Terms through a
-// diagonal entry are left out: weights are >= 0, so they never improve.)  Every
-// sum has two stored values, so it cannot overflow.  Then the owners of the
-// next two pivots' rows and columns write them back, and one barrier per pivot
-// pair orders the steps.  A write-back that lands while another thread still
-// reads this pair's pivot columns only replaces a0, a1 by a0', a1', from which
-// the same a0', a1' follow.
-// The block is on every round's critical path and bound by latency and by the
-// redundant work that saves barriers.  Add-mins per thread and four pivots:
-// one at a time 64 and four barriers, two at a time 84 and two, four at a time
-// (closing a 4 x 4 corner in every thread) 148 - 192 and one.
-template <class Op, int BK, class Bar = CtaBar>
-__device__ __forceinline__ void close_block(typename Op::scalar (&s)[BK][BK + 4],
-                                            typename Op::scalar (&v)[BK / 16][BK / 16], int by, int bx) {
+// Closes the BK x BK block held block by block in v, in place: Floyd-Warshall,
+// one pivot and one barrier a step.  A step reads the pivot's row and column
+// (one 16-byte access each), updates the thread's block, and its owners write
+// the next pivot's row and column into the other buffer.
+// The closure is on every round's critical path and runs on one SM, bound by
+// the ALU (PT^2 add-mins a thread, 64 cycles a pivot at width 64) and the
+// latency of one shared-memory read and one barrier.  Taking several pivots a
+// step saves barriers but adds work to every thread, and each was measured
+// slower: cycles for 64 x 64, int32 -- one pivot 8.5 thousand, two 9.0
+// (redundant pivot-column updates), four 11.7 - 12.1 (closing the corner in
+// every thread), pivot rows handed from warp to warp instead of barriers 13.6.
+template <class Op, int BK, class Bar>
+__device__ __forceinline__ void close_block(P1Smem<Op, BK> &sm, typename Op::scalar (&v)[BK / 16][BK / 16], int tid) {
   using S = typename Op::scalar;
-  constexpr int PT = BK / 16, PAIRS = PT / 2;
-  static_assert(PT % 2 == 0, "an even number of pivots per thread block");
-  const uint32_t one = kOne;
+  constexpr int PT = BK / 16;
+  static_assert(PT % 2 == 0, "the buffers alternate within a thread block");
+  const int by = tid / 16, bx = tid % 16;
+  auto publish = [&](int nb, int t, int buf) {  // row and column t of thread block nb
+    if (by == nb) sts_vec<PT>(&sm.row[buf][bx * PT], v[t]);
+    if (bx == nb) {
+      S w[PT];
+#pragma unroll
+      for (int r = 0; r < PT; ++r) w[r] = v[r][t];
+      sts_vec<PT>(&sm.col[buf][by * PT], w);
+    }
+  };
+  publish(0, 0, 0);
+  Bar::sync();
 #pragma unroll 1
   for (int p = 0; p < 16; ++p) {
 #pragma unroll
-    for (int h = 0; h < PAIRS; ++h) {
-      const int t0 = p * PT + 2 * h;
-      S a[PT][2], b[2][PT];
-      const S k01 = s[t0][t0 + 1], k10 = s[t0 + 1][t0];
+    for (int h = 0; h < PT; ++h) {
+      S a[PT], b[PT];
+      lds_vec<PT>(a, &sm.col[h & 1][by * PT]);
+      lds_vec<PT>(b, &sm.row[h & 1][bx * PT]);
 #pragma unroll
-      for (int r = 0; r < PT; ++r) lds_vec<2>(a[r], &s[by * PT + r][t0]);
-      lds_vec<PT>(b[0], &s[t0][bx * PT]);
-      lds_vec<PT>(b[1], &s[t0 + 1][bx * PT]);
+      for (int r = 0; r < PT; ++r)
 #pragma unroll
-      for (int r = 0; r < PT; ++r) {
-        const S a0 = Op::s_addmin(a[r][1], k10, a[r][0]), a1 = Op::s_addmin(a[r][0], k01, a[r][1]);
-#pragma unroll
-        for (int c = 0; c < PT; ++c) v[r][c] = s_update2<Op>(v[r][c], a0, b[0][c], a1, b[1][c], (r + c) & 1, one);
-      }
-      // the next pair: rows / columns n0, n0 + 1 of thread block nb
-      const int nb = (h + 1 < PAIRS) ? p : p + 1;
-      constexpr int last = PAIRS - 1;
-      const int n0 = (h == last) ? 0 : 2 * h + 2;
-      if (nb < 16) {
-        if (by == nb) {
-#pragma unroll
-          for (int i = 0; i < 2; ++i) sts_vec<PT>(&s[nb * PT + n0 + i][bx * PT], v[n0 + i]);
-        }
-        if (bx == nb) {
-#pragma unroll
-          for (int r = 0; r < PT; ++r) {
-            const S w[2] = {v[r][n0], v[r][n0 + 1]};
-            sts_vec<2>(&s[by * PT + r][nb * PT + n0], w);
-          }
-        }
-      }
+        for (int c = 0; c < PT; ++c) v[r][c] = Op::s_addmin(a[r], b[c], v[r][c]);
+      publish(h + 1 < PT ? p : p + 1, (h + 1) % PT, (h + 1) & 1);  // block 16: nobody's
       Bar::sync();
     }
   }
-#pragma unroll
-  for (int r = 0; r < PT; ++r) sts_vec<PT>(&s[by * PT + r][bx * PT], v[r]);
-  Bar::sync();
 }
 
-// The block's entries into s and, thread by thread, v.
-template <class Op, int BK, int NT, bool CG, class Bar>
+// Thread (by, bx)'s part of the BK x BK diagonal block at p0 (INF outside the
+// matrix): one 16-byte load per row where the addresses allow it.
+template <class Op, int BK, bool CG>
 __device__ __forceinline__ void load_block(const typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
-                                           typename Op::scalar (&s)[BK][BK + 4],
                                            typename Op::scalar (&v)[BK / 16][BK / 16], int tid) {
-  using S = typename Op::scalar;
   constexpr int PT = BK / 16;
-  const S INF = Op::to_s(Op::inf_elem());
-  // all of this thread's loads first, then the shared-memory stores
-  constexpr int IT = BK * BK / NT;
-  S tmp[IT];
+  const int64_t r0 = p0 + (tid / 16) * PT, c0 = p0 + (tid % 16) * PT;
 #pragma unroll
-  for (int k = 0; k < IT; ++k) {
-    const int idx = tid + k * NT;
-    const int64_t r = p0 + idx / BK, c = p0 + idx % BK;
-    tmp[k] = (r < n && c < n) ? Op::to_s(ld_elem<CG>(D + L.off(r, c))) : INF;
+  for (int r = 0; r < PT; ++r) {
+    const typename Op::elem *q = D + L.off(r0 + r, c0);
+    if (Op::EPW == 1 && PT == 4 && r0 + r < n && c0 + 4 <= n && (reinterpret_cast<uintptr_t>(q) & 15) == 0) {
+      const uint4 w = ld16<CG>(q);
+      v[r][0] = Op::to_s(bits_elem<Op>(w.x));
+      v[r][1] = Op::to_s(bits_elem<Op>(w.y));
+      v[r][PT - 2] = Op::to_s(bits_elem<Op>(w.z));
+      v[r][PT - 1] = Op::to_s(bits_elem<Op>(w.w));
+    } else {
+#pragma unroll
+      for (int c = 0; c < PT; ++c)
+        v[r][c] = Op::to_s((r0 + r < n && c0 + c < n) ? ld_elem<CG>(q + c) : Op::inf_elem());
+    }
   }
+}
+
+// PT consecutive words from PT scalars (an aligned 8- or 16-byte store).
+template <class Op, int PT>
+__device__ __forceinline__ void store_words(uint32_t *p, const typename Op::scalar (&x)[PT]) {
+  uint32_t w[PT];
 #pragma unroll
-  for (int k = 0; k < IT; ++k) {
-    const int idx = tid + k * NT;
-    s[idx / BK][idx % BK] = tmp[k];
-  }
-  Bar::sync();
-#pragma unroll
-  for (int r = 0; r < PT; ++r)
-#pragma unroll
-    for (int c = 0; c < PT; ++c) v[r][c] = s[(tid / 16) * PT + r][(tid % 16) * PT + c];
+  for (int i = 0; i < PT; ++i) w[i] = Op::dup(Op::from_s(x[i]));
+  if constexpr (PT == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+  else *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
 }
 
 template <class Op, int BK, int NT, bool CG, class Bar = CtaBar>
@@ -187,28 +172,27 @@ __device__ __forceinline__ void phase1_body(typename Op::elem *__restrict__ D, L
                                             uint32_t *__restrict__ colT, int64_t ldT, P1Smem<Op, BK> &sm, int tid,
                                             typename Op::elem *__restrict__ rowP = nullptr) {
   using S = typename Op::scalar;
-  constexpr int G = 16;
-  constexpr int PT = BK / G;
-  static_assert(BK % G == 0 && NT == G * G, "phase 1 layout");
-  auto &s = sm.s;
-  const int by = tid / G, bx = tid % G;
+  constexpr int PT = BK / 16;
+  static_assert(BK % 16 == 0 && NT == 256, "phase 1 layout");
   S v[PT][PT];
-  load_block<Op, BK, NT, CG, Bar>(D, L, n, p0, s, v, tid);
-  close_block<Op, BK, Bar>(s, v, by, bx);
-  for (int idx = tid; idx < BK * BK; idx += NT) {
-    const int i = idx / BK, j = idx % BK;
-    const int64_t r = p0 + i, c = p0 + j;
-    if (r < n && c < n) D[L.off(r, c)] = Op::from_s(s[i][j]);
-  }
-  for (int idx = tid; idx < BK * BK; idx += NT) {
-    const int t = idx / BK, i = idx % BK;
-    colT[t * ldT + p0 + i] = Op::dup(Op::from_s(s[i][t]));
-  }
-  if (rowP) {  // symmetric mode: the panel as elements (row t = D[p0 + t][.])
-    for (int idx = tid; idx < BK * BK; idx += NT) {
-      const int t = idx / BK, j = idx % BK;
-      rowP[t * ldT + p0 + j] = Op::from_s(s[t][j]);
+  load_block<Op, BK, CG>(D, L, n, p0, v, tid);
+  close_block<Op, BK, Bar>(sm, v, tid);
+  const int i0 = (tid / 16) * PT, j0 = (tid % 16) * PT;
+#pragma unroll
+  for (int r = 0; r < PT; ++r)
+#pragma unroll
+    for (int c = 0; c < PT; ++c) {
+      const int64_t row = p0 + i0 + r, col = p0 + j0 + c;
+      if (row < n && col < n) D[L.off(row, col)] = Op::from_s(v[r][c]);
+      // symmetric mode: the panel as elements (row t = D[p0 + t][.])
+      if (rowP) rowP[(i0 + r) * ldT + col] = Op::from_s(v[r][c]);
     }
+#pragma unroll
+  for (int c = 0; c < PT; ++c) {
+    S x[PT];
+#pragma unroll
+    for (int r = 0; r < PT; ++r) x[r] = v[r][c];
+    store_words<Op>(colT + (j0 + c) * ldT + p0 + i0, x);
   }
 }
 
