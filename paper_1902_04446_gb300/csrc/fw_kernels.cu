@@ -610,7 +610,6 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tiles_x = rd.tiles_x, tiles_y = rd.tiles_y;
-  pdl_trigger();
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&full_ab[i], 1);
