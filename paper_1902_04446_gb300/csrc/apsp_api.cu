@@ -159,6 +159,8 @@ struct apsp_handle {
   size_t ws16_bytes = 0;
   void *wsb = nullptr;  // batched solve: plan + panel buffers
   size_t wsb_bytes = 0;
+  void *wsD = nullptr;  // a matrix without 16-byte rows is solved in this copy
+  size_t wsD_bytes = 0;
   void *rowP = nullptr;  // symmetric mode, packed 16-bit: element panel
   size_t rowP_bytes = 0;
   void *mpT = nullptr;  // min-plus product: A^T (32-bit words)
@@ -259,12 +261,66 @@ apsp::RoundConfig config_for(apsp_handle *h, int dtype, int64_t n) {
   return c;
 }
 
+// Whether the rounds of an n x n matrix at D run on a copy with 16-byte rows:
+// the TMA kernels need them, and the kernel without (plain loads, one CTA per
+// tile, 0.56 of the add-min peak) costs far more than two passes over the
+// matrix (directed int32 n = 3001 in rows of 3001: 3.68 ms on that kernel,
+// 2.09 on a copy).  `copy_ld` is the copy's leading dimension.
+bool needs_aligned_copy(const void *D, int64_t ld, int64_t n, int dtype, const apsp::RoundConfig &rc,
+                        int64_t *copy_ld) {
+  const int64_t es = dtype == APSP_U16 ? 2 : 4;
+  *copy_ld = round_up(n, 16 / es);
+  return n > 64 && rc.p3 != 0 && (reinterpret_cast<uintptr_t>(D) % 16 != 0 || ld * es % 16 != 0);
+}
+
+// The copy stays with the handle, so it is kept to an eighth of the device's memory.
+bool aligned_copy_fits(apsp_handle *h, size_t bytes) {
+  if (h->wsD && h->wsD_bytes >= bytes) return true;
+  size_t fr = 0, tot = 0;
+  if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return bytes <= tot / 8 && bytes <= fr / 2;
+}
+
+apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
+                               bool known_sym, apsp::RoundConfig rc);
+
 // Enqueues the q rounds on D (already holding W) using the handle's panel buffer.
 // known_sym: D is symmetric by construction (edge-list input).
 apsp_status run_rounds_locked(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
                               bool known_sym = false) {
+  const apsp::RoundConfig rc = config_for(h, dtype, n);
+  int64_t ldc = 0;
+  if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc)) {
+    const size_t bytes = (size_t)n * ldc * (dtype == APSP_U16 ? 2 : 4);
+    if (aligned_copy_fits(h, bytes)) {
+      if (ensure(&h->wsD, &h->wsD_bytes, bytes) == cudaSuccess) {
+        int64_t l = 0;
+        cudaError_t e = apsp::launch_copy(dtype, D, ld, h->wsD, ldc, n, s, &l);
+        if (e == cudaSuccess) {
+          const apsp_status st = run_rounds_aligned(h, dtype, h->wsD, n, ldc, s, known_sym, rc);
+          if (st != APSP_OK) return st;
+          e = apsp::launch_copy(dtype, h->wsD, ldc, D, ld, n, s, &l);
+        }
+        h->launches += l;
+        if (e != cudaSuccess) {
+          h->last_error = std::string("aligned copy: ") + cudaGetErrorString(e);
+          return APSP_E_CUDA;
+        }
+        return APSP_OK;
+      }
+      cudaGetLastError();  // out of memory: the kernel for any alignment
+    }
+  }
+  return run_rounds_aligned(h, dtype, D, n, ld, s, known_sym, rc);
+}
+
+// The rounds on D itself.
+apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
+                               bool known_sym, apsp::RoundConfig rc) {
   const int64_t ldT = panel_ld(n);
-  apsp::RoundConfig rc = config_for(h, dtype, n);
   cudaError_t e = ensure(&h->colT, &h->colT_bytes, apsp::panel_buffer_bytes(n, ldT, rc.p3 == 4));
   if (e != cudaSuccess) {
     h->last_error = std::string("panel workspace: ") + cudaGetErrorString(e);
@@ -472,6 +528,7 @@ apsp_status apsp_destroy(apsp_handle *h) {
   if (h->colT) cudaFree(h->colT);
   if (h->ws16) cudaFree(h->ws16);
   if (h->wsb) cudaFree(h->wsb);
+  if (h->wsD) cudaFree(h->wsD);
   if (h->rowP) cudaFree(h->rowP);
   if (h->mpT) cudaFree(h->mpT);
   if (h->d_status) cudaFree(h->d_status);
@@ -1192,6 +1249,7 @@ int64_t large_extra_bytes(apsp_handle *h, const apsp_request &q) {
   int64_t b = (int64_t)apsp::panel_buffer_bytes(q.n, ldT, all);
   if (q.dtype == APSP_AUTO)
     b += 512 + (int64_t)apsp::row_panel_bytes(ldT, all) + q.n * round_up(q.n, 8) * 2;
+  if (q.n % 4 != 0) b += 256 + q.n * round_up(q.n, 4) * 4;  // the copy with 16-byte rows
   return b;
 }
 
@@ -1344,16 +1402,25 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
       }
     }
     apsp::RoundConfig rc = large_round_config(h, APSP_I32, rn);
-    if (cudaMallocAsync(&g->ws, apsp::panel_buffer_bytes(rn, ldT, rc.p3 == 4), s) != cudaSuccess) {
+    void *M = rs[0]->D;  // the matrix the rounds run on: the request's, or a copy with 16-byte rows
+    int64_t ldm = rn;
+    const bool copy = needs_aligned_copy(rs[0]->D, rn, rn, APSP_I32, rc, &ldm);
+    if (!copy) ldm = rn;
+    const size_t pb = (apsp::panel_buffer_bytes(rn, ldT, rc.p3 == 4) + 255) & ~size_t(255);
+    if (cudaMallocAsync(&g->ws, pb + (copy ? (size_t)rn * ldm * 4 : 0), s) != cudaSuccess) {
       g->ws = nullptr;
       return APSP_E_CUDA;
+    }
+    if (copy) {
+      M = static_cast<char *>(g->ws) + pb;
+      if (apsp::launch_copy(APSP_I32, rs[0]->D, rn, M, ldm, rn, s, &l) != cudaSuccess) return APSP_E_CUDA;
     }
     if (h->cfg.symmetric == 1) {
       rc.sym = true;
     } else if (h->cfg.symmetric == 0) {
       int *dflag = g->status + 2;  // zeroed with the status words
-      if (apsp::launch_symmetry_check(APSP_I32, rs[0]->D, rn, rn, dflag, s) != cudaSuccess) return APSP_E_CUDA;
-      if (apsp::device_sym(APSP_I32, rs[0]->D, rn, rn, rc)) {
+      if (apsp::launch_symmetry_check(APSP_I32, M, rn, ldm, dflag, s) != cudaSuccess) return APSP_E_CUDA;
+      if (apsp::device_sym(APSP_I32, M, ldm, rn, rc)) {
         rc.sym_flag = dflag;  // the kernels read the answer themselves
       } else {
         // one launch per round: the answer is read back before the rounds are enqueued
@@ -1364,9 +1431,9 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
         rc.sym = flag == 0;
       }
     }
-    if (apsp::launch_rounds(APSP_I32, rs[0]->D, rn, rn, g->ws, ldT, s, &l, nullptr, rc, g->status + 1) !=
-        cudaSuccess)
+    if (apsp::launch_rounds(APSP_I32, M, ldm, rn, g->ws, ldT, s, &l, nullptr, rc, g->status + 1) != cudaSuccess)
       return APSP_E_CUDA;
+    if (copy && apsp::launch_copy(APSP_I32, M, ldm, rs[0]->D, rn, rn, s, &l) != cudaSuccess) return APSP_E_CUDA;
     h->launches += l;
     if (cudaEventRecord(g->done_ev, s) != cudaSuccess) return APSP_E_CUDA;
     g->graphs_dev = nullptr;

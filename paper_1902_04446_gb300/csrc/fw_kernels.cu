@@ -1842,6 +1842,13 @@ __global__ void ingest_kernel(const typename Op::elem *__restrict__ W, typename 
   if (bad) atomicOr(status, bad);
 }
 
+template <class T>
+__global__ void copy_kernel(const T *__restrict__ s, int64_t lds, T *__restrict__ d, int64_t ldd, int64_t n) {
+  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
+      d[i * ldd + j] = s[i * lds + j];
+}
+
 __global__ void pack_kernel(const int32_t *__restrict__ s, int64_t lds, uint16_t *__restrict__ d, int64_t ldd,
                             int64_t n) {
   for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
@@ -2628,6 +2635,18 @@ cudaError_t launch_ingest(int dtype, const void *W, void *D, int64_t n, int64_t 
     case 2: return ingest_impl<OpF32>(W, D, n, ld, status, s, launches);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_copy(int dtype, const void *src, int64_t lds, void *dst, int64_t ldd, int64_t n, cudaStream_t s,
+                        int64_t *launches) {
+  if (n <= 0) return cudaSuccess;
+  const dim3 g(grid_cols(n, 256), grid_rows(n));
+  if (dtype == 1)
+    copy_kernel<<<g, 256, 0, s>>>(static_cast<const uint16_t *>(src), lds, static_cast<uint16_t *>(dst), ldd, n);
+  else
+    copy_kernel<<<g, 256, 0, s>>>(static_cast<const uint32_t *>(src), lds, static_cast<uint32_t *>(dst), ldd, n);
+  if (launches) *launches += 1;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_synth(int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s) {

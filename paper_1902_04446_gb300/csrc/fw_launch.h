@@ -149,6 +149,9 @@ cudaError_t launch_tri_rows(int dtype, const void *T, int64_t n, const int64_t *
 // Copies W to D when they differ and checks the input (status |= 1 invalid, 2 range).
 cudaError_t launch_ingest(int dtype, const void *W, void *D, int64_t n, int64_t ld, int *status, cudaStream_t s,
                           int64_t *launches);
+// dst <- src, n x n of the given element type, separate leading dimensions.
+cudaError_t launch_copy(int dtype, const void *src, int64_t lds, void *dst, int64_t ldd, int64_t n, cudaStream_t s,
+                        int64_t *launches);
 // Fills D with a synthetic symmetric graph (autotuner input).
 cudaError_t launch_synth(int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s);
 cudaError_t launch_pack(const int32_t *src, int64_t lds, uint16_t *dst, int64_t ldd, int64_t n, cudaStream_t s,
