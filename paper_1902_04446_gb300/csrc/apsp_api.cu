@@ -840,53 +840,44 @@ apsp_status apsp_unpack_u16(const uint16_t *src, int64_t lds, int32_t *dst, int6
 
 namespace {
 
-// Lays out the batched-solve workspace: plan tables, then one panel buffer
-// per graph.  Returns the total bytes; fills colT pointers relative to base.
-size_t batch_layout(const std::vector<int64_t> &n, char *base, std::vector<uint32_t *> &colT, size_t plan_bytes) {
-  size_t off = (plan_bytes + 255) / 256 * 256;
-  colT.resize(n.size());
-  for (size_t i = 0; i < n.size(); ++i) {
-    colT[i] = reinterpret_cast<uint32_t *>(base + off);
-    off += ((size_t)64 * apsp::batch_panel_ld(n[i]) * 4 + 255) / 256 * 256;
-  }
-  return off;
-}
-
 // Enqueues ingest checks and one batched launch (the handle lock is held).
 apsp_status batch_locked(apsp_handle *h, const std::vector<const int32_t *> &W, const std::vector<int64_t> &n,
                          const std::vector<int64_t> &ld, const std::vector<int32_t *> &D, cudaStream_t s,
                          int64_t spin_limit, const int *gate) {
   cudaError_t e = cudaMemsetAsync(h->d_status, 0, sizeof(int), s);
   if (e != cudaSuccess) return APSP_E_CUDA;
-  std::vector<int32_t *> Dl;
-  std::vector<int64_t> nl, ldl;
+  // copies with 16-byte rows for the matrices that have none, unless they would
+  // take more than an eighth of the device's memory or cannot be had
+  std::vector<apsp::BatchInput> in;
+  int64_t copies = 0;
   for (size_t i = 0; i < n.size(); ++i) {
     if (n[i] == 0) continue;
-    int64_t l = 0;
-    e = apsp::launch_ingest(APSP_I32, W[i], D[i], n[i], ld[i], h->d_status, s, &l);
-    h->launches += l;
-    if (e != cudaSuccess) {
-      h->last_error = std::string("ingest: ") + cudaGetErrorString(e);
-      return APSP_E_CUDA;
-    }
-    Dl.push_back(D[i]);
-    nl.push_back(n[i]);
-    ldl.push_back(ld[i]);
+    const bool unaligned = reinterpret_cast<uintptr_t>(D[i]) % 16 != 0 || ld[i] % 4 != 0;
+    if (unaligned) copies += apsp::batch_copy_bytes(n[i]);
+    in.push_back(apsp::BatchInput{W[i], D[i], n[i], ld[i], ld[i], h->d_status, unaligned});
   }
-  if (Dl.empty()) return APSP_OK;
-  // plan sizes do not depend on the panel pointers: build once to size, once for real
+  if (in.empty()) return APSP_OK;
   apsp::BatchPlan plan;
-  std::vector<uint32_t *> colT(Dl.size(), nullptr);
-  plan.build(Dl, nl, ldl, colT);
-  const size_t plan_bytes = plan.workspace_bytes();
-  const size_t need = batch_layout(nl, nullptr, colT, plan_bytes);
+  size_t need = plan.build(in, nullptr);
+  if (need > h->wsb_bytes && copies > 0) {
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) cudaGetLastError();
+    if ((size_t)copies > tot / 8 || (size_t)copies > fr / 2) {
+      for (apsp::BatchInput &x : in) x.copy = false;
+      need = plan.build(in, nullptr);
+    }
+  }
   e = ensure(&h->wsb, &h->wsb_bytes, need);
+  if (e == cudaErrorMemoryAllocation && copies > 0) {
+    cudaGetLastError();
+    for (apsp::BatchInput &x : in) x.copy = false;
+    e = ensure(&h->wsb, &h->wsb_bytes, plan.build(in, nullptr));
+  }
   if (e != cudaSuccess) {
     h->last_error = std::string("batch workspace: ") + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? APSP_E_NOMEM : APSP_E_CUDA;
   }
-  batch_layout(nl, static_cast<char *>(h->wsb), colT, plan_bytes);
-  plan.build(Dl, nl, ldl, colT);
+  plan.build(in, static_cast<char *>(h->wsb));
   int64_t l = 0;
   e = apsp::launch_batch(plan, h->wsb, s, spin_limit, gate, h->d_status, nullptr, &l);
   h->launches += l;
@@ -1229,6 +1220,16 @@ int64_t large_n(const apsp_handle *h) { return h->cfg.serving_large_n > 0 ? h->c
 
 int64_t panel_bytes(int64_t n) { return 64 * apsp::batch_panel_ld(n) * 4 + 256; }
 
+// Bytes of the copy with 16-byte rows that a request is solved in: a result has
+// rows of n elements, so n % 4 != 0 needs one.  0 where the rows are aligned, or
+// where the copy would take more than an eighth of the budget (such a request
+// runs on the kernels for any alignment).
+int64_t request_copy_bytes(const apsp_handle *h, int64_t n) {
+  if (n <= 64 || n % 4 == 0) return 0;
+  const int64_t b = apsp::batch_copy_bytes(n);
+  return b <= h->budget / 8 ? b : 0;
+}
+
 // Round shape of a large request: the size's own shape, but with the whole GPU
 // (serving_large_grid 0) one launch per round, so that the batched groups on
 // other streams keep running between its rounds; with a capped grid (the cap
@@ -1249,7 +1250,6 @@ int64_t large_extra_bytes(apsp_handle *h, const apsp_request &q) {
   int64_t b = (int64_t)apsp::panel_buffer_bytes(q.n, ldT, all);
   if (q.dtype == APSP_AUTO)
     b += 512 + (int64_t)apsp::row_panel_bytes(ldT, all) + q.n * round_up(q.n, 8) * 2;
-  if (q.n % 4 != 0) b += 256 + q.n * round_up(q.n, 4) * 4;  // the copy with 16-byte rows
   return b;
 }
 
@@ -1324,8 +1324,6 @@ void undo_admission(apsp_handle *h, const std::vector<Request *> &rs, const std:
 apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, Group *g) {
   if (!g->stream) return APSP_E_CUDA;
   cudaStream_t s = g->stream;
-  std::vector<int32_t *> D;
-  std::vector<int64_t> n, ld;
   for (Request *r : rs) {
     const int64_t rn = r->req.n;
     if (cudaMallocAsync(&r->D, (size_t)std::max<int64_t>(1, rn * rn) * 4, s) != cudaSuccess) {
@@ -1336,11 +1334,6 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
                                     (size_t)rn, r->req.is_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
                                     s) != cudaSuccess)
       return APSP_E_CUDA;
-    if (rn > 0) {
-      D.push_back(static_cast<int32_t *>(r->D));
-      n.push_back(rn);
-      ld.push_back(rn);
-    }
   }
   if (cudaEventCreateWithFlags(&g->copy_ev, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&g->done_ev, cudaEventDisableTiming) != cudaSuccess ||
@@ -1356,16 +1349,13 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
   }
   if (cudaMemsetAsync(g->status, 0, sbytes, s) != cudaSuccess) return APSP_E_CUDA;
   int64_t l = 0;
-  for (size_t i = 0; i < rs.size(); ++i) {
-    const int64_t rn = rs[i]->req.n;
-    if (rn > 0 && apsp::launch_ingest(APSP_I32, rs[i]->D, rs[i]->D, rn, rn, g->status + i, s, &l) != cudaSuccess)
-      return APSP_E_CUDA;
-  }
   if (rs.size() == 1 && (rs[0]->req.n >= large_n(h) || rs[0]->alone)) {
     // one large graph: per-round kernels on the group's stream; an undirected
     // (symmetric) matrix takes the symmetric mode, decided by a device check
     const int64_t rn = rs[0]->req.n;
     const int64_t ldT = panel_ld(rn);
+    if (rn > 0 && apsp::launch_ingest(APSP_I32, rs[0]->D, rs[0]->D, rn, rn, g->status, s, &l) != cudaSuccess)
+      return APSP_E_CUDA;
     if (rs[0]->req.dtype == APSP_AUTO) {
       // precision selection: the 16-bit bound (synchronizes the group's
       // stream), then the rounds in packed 16-bit when it holds
@@ -1404,7 +1394,7 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
     apsp::RoundConfig rc = large_round_config(h, APSP_I32, rn);
     void *M = rs[0]->D;  // the matrix the rounds run on: the request's, or a copy with 16-byte rows
     int64_t ldm = rn;
-    const bool copy = needs_aligned_copy(rs[0]->D, rn, rn, APSP_I32, rc, &ldm);
+    const bool copy = needs_aligned_copy(rs[0]->D, rn, rn, APSP_I32, rc, &ldm) && request_copy_bytes(h, rn) > 0;
     if (!copy) ldm = rn;
     const size_t pb = (apsp::panel_buffer_bytes(rn, ldT, rc.p3 == 4) + 255) & ~size_t(255);
     if (cudaMallocAsync(&g->ws, pb + (copy ? (size_t)rn * ldm * 4 : 0), s) != cudaSuccess) {
@@ -1440,25 +1430,26 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
     return APSP_OK;
   }
   // only graphs with n > 0 take part; group indices follow the tickets
+  std::vector<apsp::BatchInput> in;
+  for (size_t i = 0; i < rs.size(); ++i) {
+    const int64_t rn = rs[i]->req.n;
+    int32_t *Di = static_cast<int32_t *>(rs[i]->D);
+    if (rn > 0) in.push_back(apsp::BatchInput{Di, Di, rn, rn, rn, g->status + i, request_copy_bytes(h, rn) > 0});
+  }
   apsp::BatchPlan plan;
-  std::vector<uint32_t *> colT(D.size(), nullptr);
-  plan.build(D, n, ld, colT);
-  const size_t plan_bytes = plan.workspace_bytes();
-  const size_t need = batch_layout(n, nullptr, colT, plan_bytes);
-  if (cudaMallocAsync(&g->ws, need, s) != cudaSuccess) {
+  if (cudaMallocAsync(&g->ws, std::max<size_t>(plan.build(in, nullptr), 256), s) != cudaSuccess) {
     g->ws = nullptr;
     return APSP_E_CUDA;
   }
-  batch_layout(n, static_cast<char *>(g->ws), colT, plan_bytes);
-  plan.build(D, n, ld, colT);
-  if (!D.empty() &&
+  plan.build(in, static_cast<char *>(g->ws));
+  if (!in.empty() &&
       apsp::launch_batch(plan, g->ws, s, h->cfg.spin_limit, nullptr, g->status + rs.size(), &g->graphs_dev, &l) !=
           cudaSuccess)
     return APSP_E_CUDA;
   h->launches += l;
   if (cudaEventRecord(g->done_ev, s) != cudaSuccess) return APSP_E_CUDA;
   // graphs_dev indexes only n > 0 graphs; map statuses back by skipping n == 0
-  if (D.size() != rs.size()) g->graphs_dev = nullptr;
+  if (in.size() != rs.size()) g->graphs_dev = nullptr;
   return APSP_OK;
 }
 
@@ -1481,10 +1472,11 @@ void worker_loop(apsp_handle *h) {
         const bool big = r->req.n >= large_n(h);
         bool large = lone || big;
         if (large && !rs.empty()) break;  // a large request starts its own group
-        int64_t b = r->bytes + panel_bytes(r->req.n) + (large ? large_extra_bytes(h, r->req) : 0);
+        const int64_t base = r->bytes + panel_bytes(r->req.n) + request_copy_bytes(h, r->req.n);
+        int64_t b = base + (large ? large_extra_bytes(h, r->req) : 0);
         if (large && !big && h->used + add + b > h->budget) {
           large = false;  // no room for the per-round workspace: the batched kernel after all
-          b = r->bytes + panel_bytes(r->req.n);
+          b = base;
         }
         if (h->used + add + b > h->budget) break;  // wait for memory to free up
         h->queue.pop_front();

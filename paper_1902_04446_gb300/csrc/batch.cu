@@ -1,25 +1,35 @@
-// Batched persistent blocked Floyd-Warshall: many graphs of uneven n solved in
-// one launch.
+// Batched persistent blocked Floyd-Warshall: many graphs of uneven n in one
+// launch (the rounds are Alg. 3/4's; the paper solves one graph at a time).
 //
-// The rounds of every graph (Phase 1 -> Phase 2 -> Phase 3 per round, the
-// paper's Alg. 3/4) are cut into tasks: one Phase-1 task, one task per
-// row-panel and column-panel chunk, one task per Phase-3 output tile.  The
-// host lists them as segments in the order
-//     for round r: for phase p: for every graph with more than r rounds,
-// which is a topological order of the dependencies below.  Resident CTAs take
-// task ids from a device counter in that order, wait for the task's
-// dependency, run it, and count it done:
-//     Phase 1 of round r   waits for all Phase-3 tasks of round r-1,
-//     Phase 2 of round r   waits for Phase 1 of round r,
-//     Phase 3 of round r   waits for all Phase-2 tasks of round r.
-// A task only ever waits for tasks with smaller ids, which running CTAs have
-// already taken, so the launch always makes progress; rounds of different
-// graphs interleave and fill the GPU.  Every wait is bounded: past the spin
-// limit the task marks its graph timed out, and the graph's remaining tasks
-// are skipped (still counted done) so that nothing waits forever.
-//
+// Every graph's rounds are cut into tasks:
+//   phase 0  P1  closes the round's diagonal block into the graph's DiagBuf
+//                (round 0 from the matrix, later rounds by next_diag);
+//   phase 1  P2  one chunk of the panels (panel_chunk);
+//   phase 2  P3  one 128 x 128 tile.
+// The task list is in dependency order, round by round: every graph's P2(r),
+// every graph's P1(r + 1), every graph's P3(r), with P1(0) first.  Resident CTAs
+// take task ids from a device counter and wait for the task's dependencies on
+// per-(graph, round, phase) counters:
+//   P2(r)      <- P1(r), and P3(r - 1): the tiles hold the panels' values and
+//                 read the panel buffer that P2(r) rewrites;
+//   P1(r + 1)  <- P2(r): it applies round r's update to its block itself, so
+//                 the closure runs beside the round's tiles;
+//   P3(r)      <- P2(r).
+// A task waits only on tasks with smaller ids, which running CTAs already hold,
+// so the launch always progresses.  Every wait is bounded: past the limit the
+// graph is marked timed out, its remaining tasks are skipped but still counted.
 // Data written earlier in the same launch is read through L2 only
 // (ld.global.cg); producers publish with __threadfence + atomicAdd.
+//
+// Before the rounds one pass over pairs of mirrored 64 x 64 blocks checks every
+// input, copies it where it has to be copied, and notes whether it is
+// symmetric; a symmetric graph then computes only the tiles that touch the
+// upper triangle.  A graph whose D has no 16-byte rows is solved in a copy that
+// has: 4-byte accesses at every tile edge and row cost more than the copy.  The
+// last pass writes the lower triangles and the copies' results.
+// Measured (64 undirected graphs, n log-uniform in 128 .. 1024): 2.64 ms with
+// every round's closure after its tiles, 256-word panel chunks, general mode
+// and element-wise access to unaligned rows; 1.43 ms in this form.
 #include <algorithm>
 #include <cstdint>
 #include <vector>
@@ -27,6 +37,7 @@
 #include <cuda_runtime.h>
 
 #include "batch.h"
+#include "fw_panels.cuh"
 #include "fw_tasks.cuh"
 
 namespace apsp {
@@ -35,41 +46,65 @@ namespace {
 
 constexpr int BK = 64;
 constexpr int NT = 256;
-constexpr int P2_ROW_BNW = 256;  // row-panel chunk: 64 x 256 words
-constexpr int P2_COL_BM = 256;   // column-panel chunk: 256 x 64 words
-constexpr int SMEM_WORDS = BK * BK + BK * P2_ROW_BNW;  // 80 KB: the largest task (Phase 2)
-static_assert(SMEM_WORDS >= BK * P2_COL_BM + BK * BK && SMEM_WORDS >= 2 * BK * 128 &&
-                  SMEM_WORDS * 4 >= (int)sizeof(P1Smem<OpI32, BK>),
+constexpr int P2_XW = 32;  // panel chunk: 64 x 32 words
+constexpr int SMEM_BYTES = 2 * BK * 128 * 4;  // the largest task (P3)
+static_assert(SMEM_BYTES >= (int)sizeof(PanelSmem<OpI32, P2_XW>) && SMEM_BYTES >= (int)sizeof(NextDiagSmem<OpI32>),
               "shared memory");
 
 __device__ __forceinline__ int ld_volatile(const int *p) { return *reinterpret_cast<const volatile int *>(p); }
 
+__device__ __forceinline__ DiagBuf *diag_of(const BatchGraph &g) {
+  return reinterpret_cast<DiagBuf *>(g.colT + 64 * g.ldT);
+}
+
 // Each task kind is compiled as its own function so that its register
 // allocation does not add to the others' under the kernel's 128-register cap.
-__device__ __noinline__ void task_p1(const BatchGraph &g, int64_t p0, uint32_t *smem, int tid) {
-  auto &s = *reinterpret_cast<P1Smem<OpI32, BK> *>(smem);
-  phase1_body<OpI32, BK, NT, true>(g.D, g.ld, g.n, p0, g.colT, g.ldT, s, tid);
+__device__ __noinline__ void task_p1(const BatchGraph &g, int round, uint8_t *smem, int tid) {
+  auto &sm = *reinterpret_cast<NextDiagSmem<OpI32> *>(smem);
+  const int64_t q0 = (int64_t)round * BK;
+  if (round > 0) {
+    next_diag<OpI32, CtaBar>(g.M, g.ld, g.n, q0 - BK, q0, g.colT, g.ldT,
+                             g.asym ? nullptr : reinterpret_cast<const int32_t *>(g.colT), g.vec, diag_of(g), sm, tid);
+    return;
+  }
+  int v[4][4];
+  load_block<OpI32, 64, true>(g.M, g.ld, g.n, 0, v, tid);
+  close_block<OpI32, 64, CtaBar>(sm.p1, v, tid);
+  store_diag<OpI32>(diag_of(g), v, tid);
 }
-__device__ __noinline__ void task_p2_row(const BatchGraph &g, int64_t p0, int64_t p1, int idx, uint32_t *smem,
-                                         int tid) {
-  p2_row_task<OpI32, BK, P2_ROW_BNW, NT, true>(g.D, g.ld, g.n, p0, p1, g.colT, g.ldT, (int64_t)idx * P2_ROW_BNW,
-                                              g.vec != 0, smem, tid);
+__device__ __noinline__ void task_p2(const BatchGraph &g, int64_t p0, int idx, uint8_t *smem, int tid) {
+  panel_chunk<OpI32, P2_XW, NT>(g.M, g.ld, g.n, p0, g.colT, g.ldT, nullptr, diag_of(g), g.vec, !g.asym, idx,
+                                *reinterpret_cast<PanelSmem<OpI32, P2_XW> *>(smem), tid);
 }
-__device__ __noinline__ void task_p2_col(const BatchGraph &g, int64_t p0, int64_t p1, int idx, uint32_t *smem,
-                                         int tid) {
-  p2_col_task<OpI32, BK, P2_COL_BM, NT, true>(g.D, g.ld, g.n, p0, p1, g.colT, g.ldT, (int64_t)idx * P2_COL_BM,
-                                             g.vec != 0, smem, tid);
+__device__ __noinline__ void task_p3(const BatchGraph &g, int64_t p0, int64_t p1, int idx, uint8_t *smem, int tid) {
+  int ty, tx;
+  if (g.asym) {
+    ty = idx / g.tiles_x;
+    tx = idx % g.tiles_x;
+  } else {  // the tiles (ty, tx) with tx >= ty, row by row; later indices have none
+    ty = 0;
+    for (; ty < g.tiles_x && idx >= g.tiles_x - ty; ++ty) idx -= g.tiles_x - ty;
+    if (ty == g.tiles_x) return;
+    tx = ty + idx;
+  }
+  p3_task<OpI32, BK, true>(g.M, g.ld, g.n, p0, p1, g.colT, g.ldT, (int64_t)ty * 128, (int64_t)tx * 128, g.vec != 0,
+                           reinterpret_cast<uint32_t *>(smem), tid,
+                           g.asym ? nullptr : reinterpret_cast<const int32_t *>(g.colT));
 }
-__device__ __noinline__ void task_p3(const BatchGraph &g, int64_t p0, int64_t p1, int idx, uint32_t *smem, int tid) {
-  const int64_t row0 = (int64_t)(idx / g.tiles_x) * 128;
-  const int64_t col0 = (int64_t)(idx % g.tiles_x) * 128;
-  p3_task<OpI32, BK, true>(g.D, g.ld, g.n, p0, p1, g.colT, g.ldT, row0, col0, g.vec != 0, smem, tid);
+
+// Waits (thread 0) until *dep reaches target; false when the limit ran out.
+__device__ __forceinline__ bool wait_count(const int *dep, int target, long long spin_limit) {
+  for (long long spins = 0; ld_volatile(dep) < target; ++spins) {
+    if (spins > spin_limit) return false;
+    __nanosleep(64);
+  }
+  return true;
 }
 
 __global__ void __launch_bounds__(NT, 2)
     fw_batch_kernel(BatchGraph *G, const BatchSeg *__restrict__ segs, int nsegs, long long total,
                     unsigned long long *head, int *cnt, long long spin_limit, const int *gate, int *err) {
-  extern __shared__ __align__(16) uint32_t smem[];
+  extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ long long s_task;
   __shared__ int s_seg, s_ok;
   const int tid = threadIdx.x;
@@ -88,33 +123,20 @@ __global__ void __launch_bounds__(NT, 2)
         const BatchSeg sg = segs[lo];
         const BatchGraph &g = G[sg.graph];
         int ok = ld_volatile(&G[sg.graph].status) == 0;
-        const int *dep = nullptr;
-        int target = 0;
-        if (sg.phase == 0) {
-          if (sg.round > 0) {
-            dep = cnt + g.cnt_base + (sg.round - 1) * 3 + 2;
-            target = g.tiles;
-          } else if (gate) {
-            dep = gate;
-            target = 1;
+        if (ok) {
+          const int *c = cnt + g.cnt_base + sg.round * 3;  // this round's counters; the previous round's lie before
+          if (sg.phase == 0) {
+            if (sg.round > 0) ok = wait_count(c - 3 + 1, g.chunks, spin_limit);
+            else if (gate) ok = wait_count(gate, 1, spin_limit);
+          } else if (sg.phase == 1) {
+            ok = wait_count(c, 1, spin_limit);
+            if (ok && sg.round > 0) ok = wait_count(c - 3 + 2, g.tiles, spin_limit);
+          } else {
+            ok = wait_count(c + 1, g.chunks, spin_limit);
           }
-        } else if (sg.phase == 1) {
-          dep = cnt + g.cnt_base + sg.round * 3 + 0;
-          target = 1;
-        } else {
-          dep = cnt + g.cnt_base + sg.round * 3 + 1;
-          target = g.nrow + g.ncol;
-        }
-        if (ok && dep) {
-          long long spins = 0;
-          while (ld_volatile(dep) < target) {
-            if (++spins > spin_limit) {
-              atomicOr(&G[sg.graph].status, 4);
-              atomicOr(err, 4);
-              ok = 0;
-              break;
-            }
-            __nanosleep(64);
+          if (!ok) {
+            atomicOr(&G[sg.graph].status, 4);
+            atomicOr(err, 4);
           }
           __threadfence();
         }
@@ -126,19 +148,99 @@ __global__ void __launch_bounds__(NT, 2)
     if (task >= total) break;
     const BatchSeg sg = segs[s_seg];
     if (s_ok) {
-      const BatchGraph g = G[sg.graph];
+      const BatchGraph &g = G[sg.graph];
       const int idx = (int)(task - sg.first);
       const int64_t p0 = (int64_t)sg.round * BK;
       const int64_t p1 = (p0 + BK < g.n) ? p0 + BK : g.n;
-      if (sg.phase == 0) task_p1(g, p0, smem, tid);
-      else if (sg.phase == 1 && idx < g.nrow) task_p2_row(g, p0, p1, idx, smem, tid);
-      else if (sg.phase == 1) task_p2_col(g, p0, p1, idx - g.nrow, smem, tid);
+      if (sg.phase == 0) task_p1(g, sg.round, smem, tid);
+      else if (sg.phase == 1) task_p2(g, p0, idx, smem, tid);
       else task_p3(g, p0, p1, idx, smem, tid);
     }
     __syncthreads();  // every thread's writes of this task are done
     if (tid == 0) {
       __threadfence();
       atomicAdd(cnt + G[sg.graph].cnt_base + sg.round * 3 + sg.phase, 1);
+    }
+  }
+}
+
+// Pair p of mirrored blocks (R, C), R >= C, counted row by row.
+__device__ __forceinline__ void pair_of(int p, int &R, int &C) {
+  R = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
+  while ((long long)R * (R + 1) / 2 > p) --R;
+  while ((long long)(R + 1) * (R + 2) / 2 <= p) ++R;
+  C = p - (int)((long long)R * (R + 1) / 2);
+}
+__device__ __forceinline__ int graph_of_pair(const BatchGraph *G, int count, int p) {
+  int lo = 0, hi = count - 1;  // last graph with pair_base <= p
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (G[mid].pair_base <= p) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Checks, copies (W != M) and compares the mirrored blocks of one pair: the
+// conventions of ingest_kernel (status |= 1 invalid, 2 range).
+__global__ void __launch_bounds__(256) batch_input_kernel(BatchGraph *G, int count) {
+  __shared__ int32_t tile[64][65];
+  const int gi = graph_of_pair(G, count, blockIdx.x);
+  const BatchGraph &g = G[gi];
+  int R, C;
+  pair_of((int)blockIdx.x - g.pair_base, R, C);
+  const int tx = threadIdx.x % 64, ty = threadIdx.x / 64;
+  int bad = 0, asym = 0;
+  auto take = [&](int64_t r, int64_t c) {
+    const int32_t e = g.W[r * g.ldw + c];
+    if (e < 0 || (r == c && e != 0)) bad |= 1;
+    if (e > OpI32::inf_elem()) bad |= 2;
+    if (g.W != g.M) g.M[r * g.ld + c] = e;
+    return e;
+  };
+#pragma unroll 4
+  for (int k = ty; k < 64; k += 4) {  // block (C, R), on or above the diagonal
+    const int64_t r = C * 64 + k, c = R * 64 + tx;
+    if (r < g.n && c < g.n) tile[k][tx] = take(r, c);
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int k = ty; k < 64; k += 4) {  // block (R, C)
+    const int64_t r = R * 64 + k, c = C * 64 + tx;
+    if (r < g.n && c < g.n) asym |= (R == C ? tile[k][tx] : take(r, c)) != tile[tx][k];
+  }
+  if (bad) atomicOr(g.in_status, bad);
+  if (__syncthreads_or(asym) && threadIdx.x == 0) atomicOr(&G[gi].asym, 1);
+}
+
+// The result from M: D's lower blocks from the upper ones of a symmetric
+// graph, and all of D when the graph was solved in a copy.
+__global__ void __launch_bounds__(256) batch_output_kernel(const BatchGraph *G, int count) {
+  __shared__ int32_t tile[64][65];
+  const BatchGraph &g = G[graph_of_pair(G, count, blockIdx.x)];
+  const bool copy = g.M != g.D, sym = g.asym == 0;
+  if (!copy && !sym) return;
+  int R, C;
+  pair_of((int)blockIdx.x - g.pair_base, R, C);
+  const int tx = threadIdx.x % 64, ty = threadIdx.x / 64;
+#pragma unroll 4
+  for (int k = ty; k < 64; k += 4) {
+    const int64_t r = C * 64 + k, c = R * 64 + tx;
+    if (r < g.n && c < g.n) {
+      const int32_t e = g.M[r * g.ld + c];
+      tile[k][tx] = e;
+      if (copy && (R != C || !sym || c >= r)) g.D[r * g.ldd + c] = e;
+    }
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int k = ty; k < 64; k += 4) {
+    const int64_t r = R * 64 + k, c = C * 64 + tx;
+    if (r >= g.n || c >= g.n) continue;
+    if (sym) {
+      if (c < r) g.D[r * g.ldd + c] = tile[tx][k];
+    } else if (R != C) {
+      g.D[r * g.ldd + c] = g.M[r * g.ld + c];
     }
   }
 }
@@ -150,84 +252,101 @@ int sm_count_now() {
   return c > 0 ? c : 1;
 }
 
+size_t pad256(size_t b) { return (b + 255) / 256 * 256; }
+
 }  // namespace
 
 int64_t batch_panel_ld(int64_t n) { return ((n > 0 ? n : 1) + 255) / 256 * 256; }
 
-size_t BatchPlan::workspace_bytes() const {
-  const size_t a = graphs.size() * sizeof(BatchGraph);
-  const size_t b = segs.size() * sizeof(BatchSeg);
-  const size_t c = (size_t)ncounters * sizeof(int);
-  return ((a + 255) / 256 + (b + 255) / 256 + (c + 255) / 256 + 1) * 256;
-}
-
-void BatchPlan::build(const std::vector<int32_t *> &D, const std::vector<int64_t> &n, const std::vector<int64_t> &ld,
-                      const std::vector<uint32_t *> &colT) {
+size_t BatchPlan::build(const std::vector<BatchInput> &in, char *base) {
   graphs.clear();
   segs.clear();
   ncounters = 0;
+  pairs = 0;
   int maxq = 0;
-  for (size_t i = 0; i < D.size(); ++i) {
+  for (const BatchInput &x : in) {
     BatchGraph g{};
-    g.D = D[i];
-    g.colT = colT[i];
-    g.n = n[i];
-    g.ld = ld[i];
-    g.vec = (reinterpret_cast<uintptr_t>(D[i]) % 16 == 0 && (ld[i] * 4) % 16 == 0) ? 1 : 0;
-    g.ldT = batch_panel_ld(n[i]);
-    g.q = (int)((n[i] + BK - 1) / BK);
-    g.nrow = (int)((n[i] + P2_ROW_BNW - 1) / P2_ROW_BNW);
-    g.ncol = (int)((n[i] + P2_COL_BM - 1) / P2_COL_BM);
-    g.tiles_x = (int)((n[i] + 127) / 128);
-    g.tiles = g.tiles_x * g.tiles_x;
+    g.W = x.W;
+    g.D = x.D;
+    g.in_status = x.in_status;
+    g.n = x.n;
+    g.ldw = x.ldw;
+    g.ldd = x.ldd;
+    const bool aligned = reinterpret_cast<uintptr_t>(x.D) % 16 == 0 && x.ldd % 4 == 0;
+    g.vec = aligned || x.copy ? 1 : 0;
+    g.ld = aligned || !x.copy ? x.ldd : (x.n + 3) / 4 * 4;
+    g.ldT = batch_panel_ld(x.n);
+    g.q = (int)((x.n + BK - 1) / BK);
+    g.chunks = (int)(2 * panel_chunks<OpI32, P2_XW>(x.n));
+    g.tiles_x = (int)((x.n + 127) / 128);
+    g.tiles = g.q == 1 ? 0 : g.tiles_x * g.tiles_x;
     g.cnt_base = ncounters;
-    g.status = 0;
-    ncounters += 3 * std::max(1, g.q);
+    g.pair_base = pairs;
+    ncounters += 3 * g.q;
+    pairs += g.q * (g.q + 1) / 2;
     maxq = std::max(maxq, g.q);
     graphs.push_back(g);
   }
   long long first = 0;
-  for (int r = 0; r < maxq; ++r)
-    for (int p = 0; p < 3; ++p)
-      for (size_t i = 0; i < graphs.size(); ++i) {
-        const BatchGraph &g = graphs[i];
-        if (g.q <= r) continue;
-        // a single round closes the whole matrix in Phase 1
-        const int count = p == 0 ? 1 : (g.q == 1 ? 0 : (p == 1 ? g.nrow + g.ncol : g.tiles));
-        if (count == 0) continue;
-        segs.push_back(BatchSeg{first, (int)i, r, p, count});
-        first += count;
-      }
+  auto add = [&](int r, int phase) {
+    for (size_t i = 0; i < graphs.size(); ++i) {
+      const BatchGraph &g = graphs[i];
+      const int count = r >= g.q ? 0 : phase == 0 ? 1 : phase == 1 ? g.chunks : g.tiles;
+      if (count == 0) continue;
+      segs.push_back(BatchSeg{first, (int)i, r, phase, count});
+      first += count;
+    }
+  };
+  add(0, 0);
+  for (int r = 0; r < maxq; ++r) {
+    add(r, 1);
+    add(r + 1, 0);
+    add(r, 2);
+  }
   total = first;
+  // workspace: graphs, segments, counters and the task counter, then per graph
+  // the panel buffer with its DiagBuf and the copy
+  size_t off = pad256(graphs.size() * sizeof(BatchGraph)) + pad256(segs.size() * sizeof(BatchSeg)) +
+               pad256(ncounters * sizeof(int) + sizeof(unsigned long long));
+  for (size_t i = 0; i < graphs.size(); ++i) {
+    BatchGraph &g = graphs[i];
+    g.colT = reinterpret_cast<uint32_t *>(base + off);
+    off += pad256((size_t)64 * g.ldT * 4 + sizeof(DiagBuf));
+    g.M = g.D;
+    if (g.ld != g.ldd || (in[i].copy && reinterpret_cast<uintptr_t>(g.D) % 16 != 0)) {
+      g.M = reinterpret_cast<int32_t *>(base + off);
+      off += pad256((size_t)g.n * g.ld * 4);
+    }
+  }
+  return off;
 }
 
-cudaError_t launch_batch(const BatchPlan &plan, void *workspace, cudaStream_t s, int64_t spin_limit,
-                         const int *gate, int *err, BatchGraph **graphs_dev, int64_t *launches) {
+cudaError_t launch_batch(BatchPlan &plan, void *workspace, cudaStream_t s, int64_t spin_limit, const int *gate,
+                         int *err, BatchGraph **graphs_dev, int64_t *launches) {
   if (plan.total == 0) return cudaSuccess;
   char *w = static_cast<char *>(workspace);
   BatchGraph *G = reinterpret_cast<BatchGraph *>(w);
-  w += (plan.graphs.size() * sizeof(BatchGraph) + 255) / 256 * 256;
+  w += pad256(plan.graphs.size() * sizeof(BatchGraph));
   BatchSeg *S = reinterpret_cast<BatchSeg *>(w);
-  w += (plan.segs.size() * sizeof(BatchSeg) + 255) / 256 * 256;
-  int *cnt = reinterpret_cast<int *>(w);
-  w += ((size_t)plan.ncounters * sizeof(int) + 255) / 256 * 256;
+  w += pad256(plan.segs.size() * sizeof(BatchSeg));
   unsigned long long *head = reinterpret_cast<unsigned long long *>(w);
+  int *cnt = reinterpret_cast<int *>(head + 1);
   cudaError_t e;
   e = cudaMemcpyAsync(G, plan.graphs.data(), plan.graphs.size() * sizeof(BatchGraph), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(S, plan.segs.data(), plan.segs.size() * sizeof(BatchSeg), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(cnt, 0, (size_t)plan.ncounters * sizeof(int), s);
+  e = cudaMemsetAsync(head, 0, sizeof(unsigned long long) + (size_t)plan.ncounters * sizeof(int), s);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(head, 0, sizeof(unsigned long long), s);
+  e = cudaFuncSetAttribute(fw_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  const int smem = SMEM_WORDS * 4;
-  e = cudaFuncSetAttribute(fw_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
+  const int count = (int)plan.graphs.size();
+  batch_input_kernel<<<(unsigned)plan.pairs, 256, 0, s>>>(G, count);
   const long long grid = std::min<long long>(2LL * sm_count_now(), plan.total);
-  fw_batch_kernel<<<(unsigned)grid, NT, smem, s>>>(G, S, (int)plan.segs.size(), plan.total, head, cnt,
-                                                   spin_limit > 0 ? spin_limit : kDefaultSpinLimit, gate, err);
-  if (launches) *launches += 1;
+  fw_batch_kernel<<<(unsigned)grid, NT, SMEM_BYTES, s>>>(G, S, (int)plan.segs.size(), plan.total, head, cnt,
+                                                         spin_limit > 0 ? spin_limit : kDefaultSpinLimit, gate, err);
+  batch_output_kernel<<<(unsigned)plan.pairs, 256, 0, s>>>(G, count);
+  if (launches) *launches += 3;
   if (graphs_dev) *graphs_dev = G;
   return cudaGetLastError();
 }

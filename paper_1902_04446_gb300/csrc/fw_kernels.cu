@@ -2275,13 +2275,12 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
     if (q == 1) {
       launch_pdl(diag_to_matrix<Op>, dim3(1), dim3(1024), 0, s, D, L, n, p0, (const DiagBuf *)diag);
     } else {
-      const int64_t band = 128 * Op::EPW, b0 = p0 / band * band;
       auto go = [&](auto xw) {
         constexpr int XW = decltype(xw)::value;
-        const int64_t nx = (n + XW * Op::EPW - 1) / (XW * Op::EPW);
+        const int64_t nx = panel_chunks<Op, XW>(n);
         launch_pdl(fw_panels<Op, XW>, dim3((unsigned)(sym ? nx : 2 * nx)), dim3(PANEL_THREADS), 0, s, D, L, n, p0, colT,
-                   ldT, rowP, (const DiagBuf *)diag, vec ? 1 : 0, sym ? 1 : 0, dev_sym ? sym_flag : (const int *)nullptr,
-                   b0, b0 + band);
+                   ldT, rowP, (const DiagBuf *)diag, vec ? 1 : 0, sym ? 1 : 0,
+                   dev_sym ? sym_flag : (const int *)nullptr);
       };
       if (n <= kNarrowPanelN) go(std::integral_constant<int, 16>());
       else go(std::integral_constant<int, 32>());

@@ -161,7 +161,7 @@ __device__ __noinline__ void next_diag(const typename Op::elem *__restrict__ D, 
 // Both are out[t][x] = min(S[t][x], min_s A[s][t] + S[s][x]) on the chunk held
 // as S[t][x]: row panel S[t][x] = D[p0 + t][x] and A = diag.t, column panel
 // S[t][x] = D[x][p0 + t] (loaded and stored transposed) and A = diag.n.
-//   symmetric mode: chunk c is a column chunk left of the diagonal block, a row
+//   symmetric mode (chunks 0 .. nx-1): a chunk is a column chunk left of the diagonal block, a row
 //     chunk right of it (only the upper triangle is kept), and its result is
 //     the symmetric panel: colT words, rowP elements (packed 16-bit), and in
 //     the tile band of the diagonal block both D[p0 + t][x] and D[x][p0 + t];
@@ -171,6 +171,10 @@ __device__ __noinline__ void next_diag(const typename Op::elem *__restrict__ D, 
 // straddles the diagonal block (XE divides 64).
 constexpr int PANEL_THREADS = 128;
 template <class Op, int XW>
+__host__ __device__ constexpr int64_t panel_chunks(int64_t n) {  // of one panel
+  return (n + XW * Op::EPW - 1) / (XW * Op::EPW);
+}
+template <class Op, int XW>
 struct PanelSmem {
   uint32_t a[64][64];
   // the chunk's words; rows padded so that the transposed accesses (one
@@ -178,24 +182,22 @@ struct PanelSmem {
   uint32_t s[64][XW + 4];
 };
 
-template <class Op, int XW>
-__global__ void __launch_bounds__(PANEL_THREADS)
-    fw_panels(typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0, uint32_t *__restrict__ colT,
-              int64_t ldT, typename Op::elem *__restrict__ rowP, const DiagBuf *__restrict__ diag, int vec, int sym,
-              const int *__restrict__ sym_flag, int64_t band_start, int64_t band_end) {
+// NT threads (128 or 256), whole-CTA barriers.
+template <class Op, int XW, int NT>
+__device__ __forceinline__ void panel_chunk(typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
+                                            uint32_t *__restrict__ colT, int64_t ldT,
+                                            typename Op::elem *__restrict__ rowP, const DiagBuf *__restrict__ diag,
+                                            int vec, int sym, int chunk, PanelSmem<Op, XW> &sm, int tid) {
   using E = typename Op::elem;
-  constexpr int EPW = Op::EPW, XE = XW * EPW, CW = XW / 8;  // words per thread and row
+  constexpr int EPW = Op::EPW, XE = XW * EPW, TXN = NT / 16, CW = XW / TXN;  // CW words per thread and row
   constexpr int E4 = 4 * EPW;
-  static_assert(64 % XE == 0 || XE == 64, "a chunk never straddles the diagonal block");
-  __shared__ __align__(16) PanelSmem<Op, XW> sm;
-  const int tid = threadIdx.x;
+  static_assert(64 % XE == 0, "a chunk never straddles the diagonal block");
+  static_assert(CW % 2 == 0, "words in pairs");
+  const int64_t band_start = p0 / (128 * EPW) * (128 * EPW), band_end = band_start + 128 * EPW;
   const int nx = (int)((n + XE - 1) / XE);
-  pdl_trigger();
-  pdl_wait();
-  if (sym_flag) sym = __ldcg(sym_flag) == 0;
-  if (sym && (int)blockIdx.x >= nx) return;
-  const bool second = (int)blockIdx.x >= nx;
-  const int64_t x0 = (int64_t)((int)blockIdx.x - (second ? nx : 0)) * XE;
+  if (sym && chunk >= nx) return;
+  const bool second = chunk >= nx;
+  const int64_t x0 = (int64_t)(chunk - (second ? nx : 0)) * XE;
   const bool on_diag = x0 >= p0 && x0 < p0 + 64;
   const bool col = sym ? x0 < p0 : second;
   const bool to_colT = sym || col;
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(PANEL_THREADS)
   const bool wr_col = sym ? x0 < band_end : col;
   if (on_diag) {
     const int d0 = (int)(x0 - p0);
-    for (int idx = tid; idx < 64 * XE; idx += PANEL_THREADS) {
+    for (int idx = tid; idx < 64 * XE; idx += NT) {
       const int t = idx / XE, x = idx % XE;
       const uint32_t wn = __ldcg(&diag->n[t][d0 + x]);
       if (!col && p0 + t < n && x0 + x < n) D[L.off(p0 + t, x0 + x)] = word_elem<Op>(wn);
@@ -213,25 +215,25 @@ __global__ void __launch_bounds__(PANEL_THREADS)
     return;
   }
   // ---- operands: the closed block, and the chunk (all loads first)
-  constexpr int AIT = 64 * 16 / PANEL_THREADS;
-  constexpr int SIT = 64 * (XW / 4) / PANEL_THREADS;  // 16-byte pieces per thread
+  constexpr int AIT = 64 * 16 / NT;
+  constexpr int SIT = 64 * (XW / 4) / NT;  // 16-byte pieces per thread
   const uint32_t *A = col ? &diag->n[0][0] : &diag->t[0][0];
   uint4 va[AIT], vs[SIT];
 #pragma unroll
-  for (int k = 0; k < AIT; ++k) va[k] = __ldcg(reinterpret_cast<const uint4 *>(A) + tid + k * PANEL_THREADS);
+  for (int k = 0; k < AIT; ++k) va[k] = __ldcg(reinterpret_cast<const uint4 *>(A) + tid + k * NT);
 #pragma unroll
   for (int k = 0; k < SIT; ++k) {
-    const int idx = tid + k * PANEL_THREADS;
+    const int idx = tid + k * NT;
     if (!col) vs[k] = load_chunk<Op, true>(D, L, n, n, p0 + idx / (XW / 4), x0 + (idx % (XW / 4)) * E4, vec);
     else vs[k] = load_chunk<Op, true>(D, L, n, n, x0 + idx / (64 / E4), p0 + (idx % (64 / E4)) * E4, vec);
   }
 #pragma unroll
-  for (int k = 0; k < AIT; ++k) *(reinterpret_cast<uint4 *>(sm.a) + tid + k * PANEL_THREADS) = va[k];
+  for (int k = 0; k < AIT; ++k) *(reinterpret_cast<uint4 *>(sm.a) + tid + k * NT) = va[k];
   E *se = reinterpret_cast<E *>(sm.s);           // the chunk as elements
   constexpr int SE = (XW + 4) * EPW;             // elements per row of it
 #pragma unroll
   for (int k = 0; k < SIT; ++k) {
-    const int idx = tid + k * PANEL_THREADS;
+    const int idx = tid + k * NT;
     if (!col) {
       *reinterpret_cast<uint4 *>(&sm.s[idx / (XW / 4)][(idx % (XW / 4)) * 4]) = vs[k];
     } else {
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(PANEL_THREADS)
   }
   __syncthreads();
   // ---- out = min(S, A (x) S): 4 rows x CW words per thread
-  const int ty = tid / 8, tx = tid % 8;
+  const int ty = tid / TXN, tx = tid % TXN;
   uint32_t acc[4][CW];
 #pragma unroll
   for (int r = 0; r < 4; ++r)
@@ -309,7 +311,7 @@ __global__ void __launch_bounds__(PANEL_THREADS)
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < SIT; ++k) {
-    const int idx = tid + k * PANEL_THREADS;
+    const int idx = tid + k * NT;
     const int x = idx / (64 / E4), t = (idx % (64 / E4)) * E4;
     if (x0 + x >= n) continue;
     uint4 v = make_uint4(0, 0, 0, 0);
@@ -317,6 +319,18 @@ __global__ void __launch_bounds__(PANEL_THREADS)
     for (int e = 0; e < E4; ++e) chunk_set<Op>(v, e, elem_bits<Op>(se[(t + e) * SE + x]));
     store_chunk<Op>(D, L, x0 + x, p0 + t, v, col_mask<Op>(p0 + t, n, 0, 0), vec);
   }
+}
+
+template <class Op, int XW>
+__global__ void __launch_bounds__(PANEL_THREADS)
+    fw_panels(typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0, uint32_t *__restrict__ colT,
+              int64_t ldT, typename Op::elem *__restrict__ rowP, const DiagBuf *__restrict__ diag, int vec, int sym,
+              const int *__restrict__ sym_flag) {
+  __shared__ __align__(16) PanelSmem<Op, XW> sm;
+  pdl_trigger();
+  pdl_wait();
+  if (sym_flag) sym = __ldcg(sym_flag) == 0;
+  panel_chunk<Op, XW, PANEL_THREADS>(D, L, n, p0, colT, ldT, rowP, diag, vec, sym, blockIdx.x, sm, threadIdx.x);
 }
 
 }  // namespace apsp
