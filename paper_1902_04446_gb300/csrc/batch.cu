@@ -6,8 +6,8 @@
 //                (round 0 from the matrix, later rounds by next_diag);
 //   phase 1  P2  one chunk of the panels (panel_chunk);
 //   phase 2  P3  one 128 x 128 tile.
-// The task list is in dependency order, round by round: every graph's P2(r),
-// every graph's P1(r + 1), every graph's P3(r), with P1(0) first.  Resident CTAs
+// The task list is in dependency order, step by step: every active graph's
+// P2(r), then every P1(r + 1), then every P3(r), with P1(0) in the step before.  Resident CTAs
 // take task ids from a device counter and wait for the task's dependencies on
 // per-(graph, round, phase) counters:
 //   P2(r)      <- P1(r), and P3(r - 1): the tiles hold the panels' values and
@@ -29,7 +29,7 @@
 // last pass writes the lower triangles and the copies' results.
 // Measured (64 undirected graphs, n log-uniform in 128 .. 1024): 2.64 ms with
 // every round's closure after its tiles, 256-word panel chunks, general mode
-// and element-wise access to unaligned rows; 1.43 ms in this form.
+// and element-wise access to unaligned rows; 1.19 ms in this form.
 #include <algorithm>
 #include <cstdint>
 #include <vector>
@@ -46,7 +46,7 @@ namespace {
 
 constexpr int BK = 64;
 constexpr int NT = 256;
-constexpr int P2_XW = 32;  // panel chunk: 64 x 32 words
+constexpr int P2_XW = 32;  // panel chunk: 64 x 32 words (64: 64 graphs of 128 - 1024 4 % faster, small batches 5 % slower)
 constexpr int SMEM_BYTES = 2 * BK * 128 * 4;  // the largest task (P3)
 static_assert(SMEM_BYTES >= (int)sizeof(PanelSmem<OpI32, P2_XW>) && SMEM_BYTES >= (int)sizeof(NextDiagSmem<OpI32>),
               "shared memory");
@@ -81,10 +81,9 @@ __device__ __noinline__ void task_p3(const BatchGraph &g, int64_t p0, int64_t p1
   if (g.asym) {
     ty = idx / g.tiles_x;
     tx = idx % g.tiles_x;
-  } else {  // the tiles (ty, tx) with tx >= ty, row by row; later indices have none
+  } else {  // the tiles (ty, tx) with tx >= ty, row by row
     ty = 0;
-    for (; ty < g.tiles_x && idx >= g.tiles_x - ty; ++ty) idx -= g.tiles_x - ty;
-    if (ty == g.tiles_x) return;
+    for (; idx >= g.tiles_x - ty; ++ty) idx -= g.tiles_x - ty;
     tx = ty + idx;
   }
   p3_task<OpI32, BK, true>(g.M, g.ld, g.n, p0, p1, g.colT, g.ldT, (int64_t)ty * 128, (int64_t)tx * 128, g.vec != 0,
@@ -102,12 +101,13 @@ __device__ __forceinline__ bool wait_count(const int *dep, int target, long long
 }
 
 __global__ void __launch_bounds__(NT, 2)
-    fw_batch_kernel(BatchGraph *G, const BatchSeg *__restrict__ segs, int nsegs, long long total,
-                    unsigned long long *head, int *cnt, long long spin_limit, const int *gate, int *err) {
+    fw_batch_kernel(BatchGraph *G, const BatchSeg *__restrict__ segs, int nsegs, unsigned long long *head, int *cnt,
+                    long long spin_limit, const int *gate, int *err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ long long s_task;
   __shared__ int s_seg, s_ok;
   const int tid = threadIdx.x;
+  const long long total = segs[nsegs - 1].first + segs[nsegs - 1].count;
   for (;;) {
     if (tid == 0) {
       const long long task = (long long)atomicAdd(head, 1ull);
@@ -213,6 +213,55 @@ __global__ void __launch_bounds__(256) batch_input_kernel(BatchGraph *G, int cou
   if (__syncthreads_or(asym) && threadIdx.x == 0) atomicOr(&G[gi].asym, 1);
 }
 
+// After the input pass: the tasks that a symmetric graph has (one panel of
+// chunks, the upper tiles), and every segment's first task.  One CTA.
+__global__ void __launch_bounds__(1024) batch_plan_kernel(BatchGraph *G, int count, BatchSeg *segs, int nsegs) {
+  __shared__ long long warp_sum[32];
+  __shared__ long long carry;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < count; i += blockDim.x)
+    if (!G[i].asym) {
+      G[i].chunks /= 2;
+      if (G[i].q > 1) G[i].tiles = G[i].tiles_x * (G[i].tiles_x + 1) / 2;
+    }
+  if (tid == 0) carry = 0;
+  __syncthreads();
+  for (int b = 0; b < nsegs; b += (int)blockDim.x) {
+    const int i = b + tid;
+    long long c = 0;
+    if (i < nsegs) {
+      const BatchGraph &g = G[segs[i].graph];
+      c = segs[i].phase == 0 ? 1 : segs[i].phase == 1 ? g.chunks : g.tiles;
+    }
+    long long x = c;  // inclusive scan
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
+    }
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      long long y = warp_sum[lane];
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const long long z = __shfl_up_sync(0xffffffffu, y, d);
+        if (lane >= d) y += z;
+      }
+      warp_sum[lane] = y;
+    }
+    __syncthreads();
+    const long long base = carry + (warp > 0 ? warp_sum[warp - 1] : 0);
+    if (i < nsegs) {
+      segs[i].first = base + x - c;
+      segs[i].count = (int)c;
+    }
+    __syncthreads();
+    if (tid == 0) carry += warp_sum[31];
+    __syncthreads();
+  }
+}
+
 // The result from M: D's lower blocks from the upper ones of a symmetric
 // graph, and all of D when the graph was solved in a copy.
 __global__ void __launch_bounds__(256) batch_output_kernel(const BatchGraph *G, int count) {
@@ -287,21 +336,44 @@ size_t BatchPlan::build(const std::vector<BatchInput> &in, char *base) {
     maxq = std::max(maxq, g.q);
     graphs.push_back(g);
   }
+  // Where each graph's rounds lie among the maxq steps of the list: the graph
+  // with the most rounds takes all of them, the others (most rounds first) the
+  // window that holds the least work so far, so that every step has tiles enough
+  // to hide the largest graphs' chains of dependent tasks.
+  std::vector<int> order(graphs.size()), start(graphs.size(), 0);
+  for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return graphs[a].q > graphs[b].q; });
+  std::vector<double> load(maxq, 0.0);
+  for (int i : order) {
+    const BatchGraph &g = graphs[i];
+    double sum = 0.0, best = 0.0;
+    for (int t = 0; t < maxq; ++t) {
+      sum += load[t];
+      if (t >= g.q) sum -= load[t - g.q];
+      if (t + 1 == g.q || (t + 1 > g.q && sum < best)) {
+        best = sum;
+        start[i] = t + 1 - g.q;
+      }
+    }
+    const double work = g.tiles + 0.25 * g.chunks;  // a chunk costs about a quarter of a tile
+    for (int r = 0; r < g.q; ++r) load[start[i] + r] += work;
+  }
   long long first = 0;
-  auto add = [&](int r, int phase) {
-    for (size_t i = 0; i < graphs.size(); ++i) {
+  auto add = [&](int t, int phase) {  // step t: round t - start (phase 0: the closure for the next round)
+    for (int i : order) {
       const BatchGraph &g = graphs[i];
-      const int count = r >= g.q ? 0 : phase == 0 ? 1 : phase == 1 ? g.chunks : g.tiles;
+      const int r = t - start[i] + (phase == 0 ? 1 : 0);
+      const int count = r < 0 || r >= g.q ? 0 : phase == 0 ? 1 : phase == 1 ? g.chunks : g.tiles;
       if (count == 0) continue;
-      segs.push_back(BatchSeg{first, (int)i, r, phase, count});
+      segs.push_back(BatchSeg{first, i, r, phase, count});
       first += count;
     }
   };
-  add(0, 0);
-  for (int r = 0; r < maxq; ++r) {
-    add(r, 1);
-    add(r + 1, 0);
-    add(r, 2);
+  add(-1, 0);
+  for (int t = 0; t < maxq; ++t) {
+    add(t, 1);
+    add(t, 0);
+    add(t, 2);
   }
   total = first;
   // workspace: graphs, segments, counters and the task counter, then per graph
@@ -342,11 +414,12 @@ cudaError_t launch_batch(BatchPlan &plan, void *workspace, cudaStream_t s, int64
   if (e != cudaSuccess) return e;
   const int count = (int)plan.graphs.size();
   batch_input_kernel<<<(unsigned)plan.pairs, 256, 0, s>>>(G, count);
+  batch_plan_kernel<<<1, 1024, 0, s>>>(G, count, S, (int)plan.segs.size());
   const long long grid = std::min<long long>(2LL * sm_count_now(), plan.total);
-  fw_batch_kernel<<<(unsigned)grid, NT, SMEM_BYTES, s>>>(G, S, (int)plan.segs.size(), plan.total, head, cnt,
+  fw_batch_kernel<<<(unsigned)grid, NT, SMEM_BYTES, s>>>(G, S, (int)plan.segs.size(), head, cnt,
                                                          spin_limit > 0 ? spin_limit : kDefaultSpinLimit, gate, err);
   batch_output_kernel<<<(unsigned)plan.pairs, 256, 0, s>>>(G, count);
-  if (launches) *launches += 3;
+  if (launches) *launches += 4;
   if (graphs_dev) *graphs_dev = G;
   return cudaGetLastError();
 }
