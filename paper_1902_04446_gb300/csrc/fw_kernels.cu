@@ -28,7 +28,6 @@
 
 #include <algorithm>
 #include <mutex>
-#include <type_traits>
 #include <utility>
 
 #include <cudaTypedefs.h>
@@ -2127,8 +2126,10 @@ static void launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
   cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);  // errors surface in cudaGetLastError
 }
 
-// Largest n whose panels are cut into 16-word chunks (otherwise 32 words).
-constexpr int64_t kNarrowPanelN = 6144;
+// Words per panel chunk of the per-round path.  Measured with 16 / 32 words (ms
+// per solve): int32 n = 2048 0.532 / 0.577, n = 25000 377.0 / 377.2, packed
+// 16-bit n = 4096 1.695 / 1.813, n = 16384 63.7 / 64.0.
+constexpr int kPanelWords = 16;
 
 template <class Op, int BK>
 static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64_t ldT, bool vec, int variant,
@@ -2275,15 +2276,10 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
     if (q == 1) {
       launch_pdl(diag_to_matrix<Op>, dim3(1), dim3(1024), 0, s, D, L, n, p0, (const DiagBuf *)diag);
     } else {
-      auto go = [&](auto xw) {
-        constexpr int XW = decltype(xw)::value;
-        const int64_t nx = panel_chunks<Op, XW>(n);
-        launch_pdl(fw_panels<Op, XW>, dim3((unsigned)(sym ? nx : 2 * nx)), dim3(PANEL_THREADS), 0, s, D, L, n, p0, colT,
-                   ldT, rowP, (const DiagBuf *)diag, vec ? 1 : 0, sym ? 1 : 0,
-                   dev_sym ? sym_flag : (const int *)nullptr);
-      };
-      if (n <= kNarrowPanelN) go(std::integral_constant<int, 16>());
-      else go(std::integral_constant<int, 32>());
+      const int64_t nx = panel_chunks<Op, kPanelWords>(n);
+      launch_pdl(fw_panels<Op, kPanelWords>, dim3((unsigned)(sym ? nx : 2 * nx)), dim3(PANEL_THREADS), 0, s, D, L, n,
+                 p0, colT, ldT, rowP, (const DiagBuf *)diag, vec ? 1 : 0, sym ? 1 : 0,
+                 dev_sym ? sym_flag : (const int *)nullptr);
     }
     if (launches) *launches += 1;
     if (tm) tm->after(1, s, sym ? rest * w * w : 2.0 * rest * w * w);

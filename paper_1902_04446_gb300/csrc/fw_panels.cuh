@@ -6,8 +6,7 @@
 // by the chain diagonal closure -> panels -> tiles: at n = 2048 38 us, of which
 // the tiles' add-mins need 7.  Here a round is two launches:
 //   fw_panels   relaxes every chunk of the panels with the closed diagonal
-//               block (16 or 32 words wide, so that a small n still fills the
-//               GPU), and publishes them: D, colT, and in symmetric mode the
+//               block (16 words wide, so that a small n still fills the GPU), and publishes them: D, colT, and in symmetric mode the
 //               element panel and the band elements below the diagonal;
 //   Phase 3     whose first CTA, before its tiles, applies this round's update
 //               to the next diagonal block and closes it (next_diag), into a
@@ -177,9 +176,7 @@ __host__ __device__ constexpr int64_t panel_chunks(int64_t n) {  // of one panel
 template <class Op, int XW>
 struct PanelSmem {
   uint32_t a[64][64];
-  // the chunk's words; rows padded so that the transposed accesses (one
-  // element of 8 consecutive t per thread) spread over the banks
-  uint32_t s[64][XW + 4];
+  uint32_t s[64][XW + 4];  // the chunk's words
 };
 
 // NT threads (128 or 256), whole-CTA barriers.
@@ -204,28 +201,60 @@ __device__ __forceinline__ void panel_chunk(typename Op::elem *__restrict__ D, L
   const bool wr_row = sym ? x0 >= band_start : !col;
   const bool wr_col = sym ? x0 < band_end : col;
   if (on_diag) {
+    // all loads first: taken one at a time they made this the round's slowest
+    // CTA (packed 16-bit n = 4096: 1847 us per solve, 1699 in this form)
+    constexpr int IT = 64 * (XE / 4) / NT;
     const int d0 = (int)(x0 - p0);
-    for (int idx = tid; idx < 64 * XE; idx += NT) {
-      const int t = idx / XE, x = idx % XE;
-      const uint32_t wn = __ldcg(&diag->n[t][d0 + x]);
-      if (!col && p0 + t < n && x0 + x < n) D[L.off(p0 + t, x0 + x)] = word_elem<Op>(wn);
-      if (to_colT) colT[(int64_t)t * ldT + x0 + x] = __ldcg(&diag->t[t][d0 + x]);
-      if (sym && rowP) rowP[(int64_t)t * ldT + x0 + x] = word_elem<Op>(wn);
+    uint4 wn[IT], wt[IT];
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int idx = tid + k * NT, t = idx / (XE / 4), x = idx % (XE / 4) * 4;
+      wn[k] = __ldcg(reinterpret_cast<const uint4 *>(&diag->n[t][d0 + x]));
+      wt[k] = __ldcg(reinterpret_cast<const uint4 *>(&diag->t[t][d0 + x]));
+    }
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int idx = tid + k * NT, t = idx / (XE / 4), x = idx % (XE / 4) * 4;
+      if (to_colT) *reinterpret_cast<uint4 *>(colT + (int64_t)t * ldT + x0 + x) = wt[k];
+      const uint32_t w[4] = {wn[k].x, wn[k].y, wn[k].z, wn[k].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const E v = word_elem<Op>(w[e]);
+        if (!col && p0 + t < n && x0 + x + e < n) D[L.off(p0 + t, x0 + x + e)] = v;
+        if (sym && EPW == 2) rowP[(int64_t)t * ldT + x0 + x + e] = v;
+      }
     }
     return;
   }
-  // ---- operands: the closed block, and the chunk (all loads first)
+  // ---- operands: the closed block, and the chunk (all loads first).  A column
+  // chunk is loaded 32 bytes of one row per thread, consecutive threads in
+  // consecutive rows: full sectors from memory, and the transposed element
+  // stores of a warp fall into consecutive words (16 bytes a thread along the
+  // rows made them conflict 8-fold).
   constexpr int AIT = 64 * 16 / NT;
   constexpr int SIT = 64 * (XW / 4) / NT;  // 16-byte pieces per thread
+  constexpr int PB = SIT < 2 ? SIT : 2;    // pieces of one row that a thread takes in a row
+  static_assert(SIT % PB == 0, "pieces");
   const uint32_t *A = col ? &diag->n[0][0] : &diag->t[0][0];
+  // column chunk: row and first column of this thread's piece k
+  auto col_piece = [&](int k, int &x, int &t) {
+    const int u = tid + (k / PB) * NT;
+    x = u % XE;
+    t = (u / XE * PB + k % PB) * E4;
+  };
   uint4 va[AIT], vs[SIT];
 #pragma unroll
   for (int k = 0; k < AIT; ++k) va[k] = __ldcg(reinterpret_cast<const uint4 *>(A) + tid + k * NT);
 #pragma unroll
   for (int k = 0; k < SIT; ++k) {
-    const int idx = tid + k * NT;
-    if (!col) vs[k] = load_chunk<Op, true>(D, L, n, n, p0 + idx / (XW / 4), x0 + (idx % (XW / 4)) * E4, vec);
-    else vs[k] = load_chunk<Op, true>(D, L, n, n, x0 + idx / (64 / E4), p0 + (idx % (64 / E4)) * E4, vec);
+    if (!col) {
+      const int idx = tid + k * NT;
+      vs[k] = load_chunk<Op, true>(D, L, n, n, p0 + idx / (XW / 4), x0 + (idx % (XW / 4)) * E4, vec);
+    } else {
+      int x, t;
+      col_piece(k, x, t);
+      vs[k] = load_chunk<Op, true>(D, L, n, n, x0 + x, p0 + t, vec);
+    }
   }
 #pragma unroll
   for (int k = 0; k < AIT; ++k) *(reinterpret_cast<uint4 *>(sm.a) + tid + k * NT) = va[k];
@@ -233,11 +262,12 @@ __device__ __forceinline__ void panel_chunk(typename Op::elem *__restrict__ D, L
   constexpr int SE = (XW + 4) * EPW;             // elements per row of it
 #pragma unroll
   for (int k = 0; k < SIT; ++k) {
-    const int idx = tid + k * NT;
     if (!col) {
+      const int idx = tid + k * NT;
       *reinterpret_cast<uint4 *>(&sm.s[idx / (XW / 4)][(idx % (XW / 4)) * 4]) = vs[k];
     } else {
-      const int x = idx / (64 / E4), t = (idx % (64 / E4)) * E4;
+      int x, t;
+      col_piece(k, x, t);
 #pragma unroll
       for (int e = 0; e < E4; ++e) se[(t + e) * SE + x] = bits_elem<Op>(chunk_get<Op>(vs[k], e));
     }
@@ -302,7 +332,7 @@ __device__ __forceinline__ void panel_chunk(typename Op::elem *__restrict__ D, L
     }
   }
   if (!wr_col) return;
-  // transposed through shared memory: D[x][p0 + t], 16 bytes of one row a store
+  // transposed through shared memory: D[x][p0 + t], as the column chunk was loaded
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < 4; ++r)
@@ -311,13 +341,14 @@ __device__ __forceinline__ void panel_chunk(typename Op::elem *__restrict__ D, L
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < SIT; ++k) {
-    const int idx = tid + k * NT;
-    const int x = idx / (64 / E4), t = (idx % (64 / E4)) * E4;
+    int x, t;
+    col_piece(k, x, t);
     if (x0 + x >= n) continue;
     uint4 v = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int e = 0; e < E4; ++e) chunk_set<Op>(v, e, elem_bits<Op>(se[(t + e) * SE + x]));
-    store_chunk<Op>(D, L, x0 + x, p0 + t, v, col_mask<Op>(p0 + t, n, 0, 0), vec);
+    if (vec && p0 + t + E4 <= n) *reinterpret_cast<uint4 *>(D + L.off(x0 + x, p0 + t)) = v;
+    else store_chunk<Op>(D, L, x0 + x, p0 + t, v, col_mask<Op>(p0 + t, n, 0, 0), vec);
   }
 }
 
