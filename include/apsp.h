@@ -82,7 +82,8 @@ typedef struct {
   int64_t memory_budget; /* serving: bytes of device memory for admitted requests (0 = free HBM - reserve) */
   int64_t spin_limit;    /* bounded device waits: iterations before APSP_E_TIMEOUT (0 = default) */
   int phase3_variant;    /* Phase-3 kernel: 0 = tuned, else by n and dtype (5 for 6144 <= n < 24576,
-                            6144 <= n < 49152 for packed 16-bit; 4 otherwise), 1 = one
+                            6144 <= n < 49152 for packed 16-bit; 4 otherwise -- and 5 so chosen runs as 4
+                            where one launch per round is faster, see apsp_tuned_config), 1 = one
                             CTA per tile, 2 = persistent TMA kernel with 256 threads, 3 = persistent TMA
                             kernel with 512 threads, 4 = warp-specialized persistent kernel (TMA producer
                             warp; int32 results leave by a TMA min-reduction), one launch per round,
@@ -347,7 +348,9 @@ apsp_status apsp_autotune(apsp_handle *h, int dtype, int64_t n_max, const char *
 /* The round shape the handle uses for (dtype, n): *block_k and *tma, the
  * Phase-3 kernel numbered as apsp_config.phase3_variant minus one (0 = one
  * CTA per tile, 1-3 = the persistent TMA kernels launched per round, 4 = every
- * round in one launch). */
+ * round in one launch).  A 4 that neither apsp_config nor apsp_autotune chose
+ * runs as 3 where that was measured faster: int32 below n = 7680 and from 14336,
+ * packed 16-bit below 9216 and from 32768, fp32 at every n. */
 apsp_status apsp_tuned_config(apsp_handle *h, int dtype, int64_t n, int *block_k, int *tma);
 
 /* ---- solve without allocation -------------------------------------------- */

@@ -287,11 +287,21 @@ bool aligned_copy_fits(apsp_handle *h, size_t bytes) {
 apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
                                bool known_sym, apsp::RoundConfig rc);
 
+// The shape a solve runs with: config_for, except that kernel 4 as a default
+// (neither forced nor tuned) runs as kernel 3 where that is faster.
+apsp::RoundConfig run_config(apsp_handle *h, int dtype, int64_t n) {
+  apsp::RoundConfig c = config_for(h, dtype, n);
+  bool tuned = h->cfg.phase3_variant >= 1;
+  for (const auto &kv : h->tuned) tuned = tuned || kv.first.first == dtype;
+  if (c.p3 == 4 && !tuned) c.p3 = apsp::solve_phase3(n, dtype);
+  return c;
+}
+
 // Enqueues the q rounds on D (already holding W) using the handle's panel buffer.
 // known_sym: D is symmetric by construction (edge-list input).
 apsp_status run_rounds_locked(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
                               bool known_sym = false) {
-  const apsp::RoundConfig rc = config_for(h, dtype, n);
+  const apsp::RoundConfig rc = run_config(h, dtype, n);
   int64_t ldc = 0;
   if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc)) {
     const size_t bytes = (size_t)n * ldc * (dtype == APSP_U16 ? 2 : 4);
@@ -1235,7 +1245,7 @@ int64_t request_copy_bytes(const apsp_handle *h, int64_t n) {
 // other streams keep running between its rounds; with a capped grid (the cap
 // leaves SMs to the other groups) the size's default.
 apsp::RoundConfig large_round_config(apsp_handle *h, int dtype, int64_t n) {
-  apsp::RoundConfig rc = config_for(h, dtype, n);
+  apsp::RoundConfig rc = run_config(h, dtype, n);
   rc.grid_cap = h->cfg.serving_large_grid;
   if (rc.p3 == 4 && rc.grid_cap == 0) rc.p3 = 3;
   return rc;

@@ -320,10 +320,11 @@ struct KLoop {
 // Kernels with at most 128 registers a thread (Phase 2, one CTA per tile, batched).
 using KLoopSmall = KLoop<false, 1, false, 1>;
 
-// Runs compute(a, b) on every pair of k-steps: load(t, a, b) fetches the
-// operands of k-steps t and t + 1.
+// Runs compute(a, b) on every pair of the first `ksteps` k-steps (BK, or a
+// smaller multiple of 4): load(t, a, b) fetches the operands of k-steps t and
+// t + 1 of a buffer of BK.
 template <class KL, int BK, class RegA, class RegB, class Load, class Compute>
-__device__ __forceinline__ void k_pairs(const Load &load, const Compute &compute) {
+__device__ __forceinline__ void k_pairs(const Load &load, const Compute &compute, int ksteps) {
   if constexpr (KL::PREFETCH) {
     static_assert(BK % 4 == 0 && (BK & (BK - 1)) == 0, "k-steps in pairs of pairs");
     RegA a0, a1;
@@ -331,17 +332,17 @@ __device__ __forceinline__ void k_pairs(const Load &load, const Compute &compute
     load(0, a0, b0);
     constexpr int U = KL::UNROLL;
 #pragma unroll U
-    for (int t = 0; t < BK; t += 4) {
+    for (int t = 0; t < ksteps; t += 4) {
       load(t + 2, a1, b1);
       compute(a0, b0);
-      load((t + 4) & (BK - 1), a0, b0);  // the last trip re-reads k-step 0: in bounds, unused
+      load((t + 4) & (BK - 1), a0, b0);  // the last trip's load is in bounds and unused
       compute(a1, b1);
     }
   } else {
     static_assert(BK % 2 == 0, "k-steps in pairs");
     constexpr int U = KL::UNROLL;
 #pragma unroll U
-    for (int t = 0; t < BK; t += 2) {
+    for (int t = 0; t < ksteps; t += 2) {
       RegA a;
       RegB b;
       load(t, a, b);
@@ -386,7 +387,7 @@ struct RegsF32B {
 };
 template <class KL, int BM, int BNW, int BK, int TN>
 __device__ __forceinline__ void tile_minplus_f32(const uint32_t *__restrict__ As, const uint32_t *__restrict__ Bs,
-                                                 uint32_t (&acc)[8][TN], int ty, int tx) {
+                                                 uint32_t (&acc)[8][TN], int ty, int tx, int ksteps) {
   float f[8][TN];
 #pragma unroll
   for (int r = 0; r < 8; ++r)
@@ -429,7 +430,7 @@ __device__ __forceinline__ void tile_minplus_f32(const uint32_t *__restrict__ As
         f[r][2 * p + 1] = fmin3(f[r][2 * p + 1], y0, y1);
       }
   };
-  k_pairs<KL, BK, RA, RegsF32B<TN>>(load, compute);
+  k_pairs<KL, BK, RA, RegsF32B<TN>>(load, compute, ksteps);
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -478,9 +479,9 @@ struct RegsU32 {
 // <= 0x7FFF, so the low lane's sum never carries into the high lane.
 template <class Op, int BM, int BNW, int BK, int TN = 8, class KL = KLoopSmall>
 __device__ __forceinline__ void tile_minplus(const uint32_t *__restrict__ As, const uint32_t *__restrict__ Bs,
-                                             uint32_t (&acc)[8][TN], int ty, int tx) {
+                                             uint32_t (&acc)[8][TN], int ty, int tx, int ksteps = BK) {
   if constexpr (Op::DTYPE == 2) {
-    tile_minplus_f32<KL, BM, BNW, BK, TN>(As, Bs, acc, ty, tx);
+    tile_minplus_f32<KL, BM, BNW, BK, TN>(As, Bs, acc, ty, tx, ksteps);
   } else {
     const uint32_t one = kOne;
     auto load = [&](int t, RegsU32<8> &ra, RegsU32<TN> &rb) {
@@ -511,7 +512,7 @@ __device__ __forceinline__ void tile_minplus(const uint32_t *__restrict__ As, co
                                        one);
         }
     };
-    k_pairs<KL, BK, RegsU32<8>, RegsU32<TN>>(load, compute);
+    k_pairs<KL, BK, RegsU32<8>, RegsU32<TN>>(load, compute, ksteps);
   }
 }
 

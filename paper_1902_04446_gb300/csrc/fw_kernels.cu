@@ -28,6 +28,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include <cudaTypedefs.h>
@@ -539,8 +540,7 @@ __device__ __forceinline__ void red_tail_store(int32_t *D, int64_t ld, int64_t n
       for (int e = 0; e < 4; ++e) {
         const int64_t c = cw + e;
         if (c >= n4 && c < ncols) {
-          int32_t *p = D + row * ld + c;
-          *p = (int32_t)OpI32::addmin(acc[r][4 * h + e], 0u, (uint32_t)*p);
+          atomicMin(D + row * ld + c, (int32_t)acc[r][4 * h + e]);  // another CTA may hold a part of this tile
         }
       }
     }
@@ -550,10 +550,13 @@ __device__ __forceinline__ void red_tail_store(int32_t *D, int64_t ld, int64_t n
 // Schedules of the warp-specialized kernels' k-loops (KLoop, fw_device.cuh).
 // Per element type the fastest measured of prefetch x unroll x walk x mix on
 // n = 16384 solves (one launch per round at widths 64 and 128, every round in
-// one launch) and on a 4096-cubed product; fp32 has no mix.
+// one launch) and on a 4096-cubed product; fp32 has no mix.  The compiled loop
+// depends on its surroundings as much as on these, so a change to a kernel's
+// tile loop calls for timing them again (int32 per round, n = 16384, ms: the
+// fastest 108.7, the others 110.9 - 119.9).
 template <class Op, int BK>
 struct P3Loop {
-  using Round = KLoop<true, 1, true, 1>;
+  using Round = typename std::conditional<BK == 128, KLoop<true, 1, true, 1>, KLoop<false, 1, false, 1>>::type;
   using Solve = KLoop<true, 2, true, 0>;
   using Product = KLoop<true, 2, true, 0>;
 };
@@ -584,10 +587,133 @@ struct P3Round {
   DiagBuf *diag;                       // next_diag: where the closed block goes
 };
 
-// With a next_diag task (round width 64), block 0 runs it before its tiles: the
-// task costs about as much as one tile, so it counts as one in the split of the
-// tiles over the CTAs.
-template <class Op, int BK, bool RED>
+// The tiles that touch the upper triangle (symmetric mode) or all of them, in
+// row-major order.
+template <class Op>
+struct TileGrid {
+  int tiles_x, tiles_y, sym;
+  int ty, tx;
+  __device__ __forceinline__ void locate(int tile) {
+    if (!sym) {
+      ty = tile / tiles_x;
+      tx = tile % tiles_x;
+      return;
+    }
+    int lo = 0, hi = tiles_y - 1;  // last tile row whose prefix <= tile
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (sym_prefix(mid, tiles_x, Op::EPW) <= tile) lo = mid;
+      else hi = mid - 1;
+    }
+    ty = lo;
+    tx = lo / Op::EPW + (int)(tile - sym_prefix(lo, tiles_x, Op::EPW));
+  }
+  __device__ __forceinline__ void step() {
+    if (++tx == tiles_x) {
+      ++ty;
+      tx = sym ? ty / Op::EPW : 0;
+    }
+  }
+};
+
+// How a launch's tiles are split over its CTAs (every thread of a CTA computes
+// the same split).  With a next_diag task (round width 64) block 0 runs it
+// before its tiles; it costs about as much as one tile and counts as one.
+// TileRun: contiguous runs of whole tiles.
+template <class Op>
+struct TileRun : TileGrid<Op> {
+  int first, nu;  // this CTA's first tile, number of tiles
+  static constexpr int part = 0;
+  __device__ __forceinline__ void plan(int tiles, int chain) {
+    const int items = tiles + chain, per = items / (int)gridDim.x, extra = items % (int)gridDim.x;
+    const int b = (int)blockIdx.x * per + min((int)blockIdx.x, extra);
+    first = max(b - chain, 0);
+    nu = b + per + ((int)blockIdx.x < extra ? 1 : 0) - chain - first;
+  }
+  __device__ __forceinline__ void begin() { this->locate(first); }
+  __device__ __forceinline__ void next() { this->step(); }
+  __device__ __forceinline__ int ksteps(int ks) const { return ks; }
+};
+// TileWalk: `a` whole tiles each, and the tiles left over (fewer than CTAs),
+// which would fill part of one more wave, cut into 2 or 4 parts of the k-steps
+// where that ends the wave earlier; the CTAs reduce their parts into the same
+// tile (a minimum, so the order does not matter).  A part costs kPartCost
+// k-steps besides its own (epilogue, stage hand-over).  The extra bookkeeping
+// makes the kernel 2 - 4 % slower, so the host takes it only where the cut
+// gains more (split_gain).  Measured, ms per solve, whole tiles / cut: int32
+// n = 2304 0.922 / 0.747, n = 2560 1.041 / 0.925, n = 4096 2.69 / 2.55.
+constexpr int kPartCost = 6;
+constexpr int kPartBox = 16;  // k-steps per TMA box of the cut stages: the smallest part
+// Parts (as a power of two) for `rem` left-over tiles on nb CTAs, and the cost
+// of their wave in k-steps.
+__host__ __device__ inline int wave_parts(int rem, int nb, int &cost) {
+  int lp = 0;
+  cost = rem > 0 ? (rem + nb - 1) / nb * (64 + kPartCost) : 0;
+  for (int l = 1; l <= 2; ++l) {
+    const int c = ((rem << l) + nb - 1) / nb * ((64 >> l) + kPartCost);
+    if (c < cost) {
+      cost = c;
+      lp = l;
+    }
+  }
+  return lp;
+}
+template <class Op>
+struct TileWalk : TileGrid<Op> {
+  static constexpr int first = 0;
+  int nf, nu;      // whole tiles, and tiles and parts together, of this CTA
+  int lp;          // log2 of the parts per left-over tile
+  int f0, r0, u0;  // first whole tile, first left-over tile, first part (counted from r0's)
+  int i, part;
+  __device__ __forceinline__ void plan(int tiles, int chain) {
+    const int g = (int)gridDim.x, b = (int)blockIdx.x;
+    const int a = (tiles + chain) / g;
+    f0 = max(b * a - chain, 0);
+    nf = a == 0 ? 0 : (b + 1) * a - chain - f0;
+    r0 = max(a * g - chain, 0);
+    const int rem = tiles - r0;
+    const int skip = a == 0 ? chain : 0;  // block 0 then has the next_diag task only
+    const int nb = g - skip, bb = b - skip;
+    int cost;
+    lp = wave_parts(rem, nb, cost);
+    const int units = rem << lp, per = units / nb, extra = units % nb;
+    u0 = bb < 0 ? 0 : bb * per + min(bb, extra);
+    nu = nf + (bb < 0 ? 0 : per + (bb < extra ? 1 : 0));
+  }
+  __device__ __forceinline__ void begin() {
+    i = 0;
+    part = nf > 0 ? 0 : u0 & ((1 << lp) - 1);
+    this->locate(nf > 0 ? f0 : r0 + (u0 >> lp));
+  }
+  __device__ __forceinline__ void next() {
+    ++i;
+    if (i == nf) {
+      part = u0 & ((1 << lp) - 1);
+      if (i < nu) this->locate(r0 + (u0 >> lp));
+      return;
+    }
+    if (i > nf && ++part < (1 << lp)) return;
+    part = 0;
+    this->step();
+  }
+  __device__ __forceinline__ int ksteps(int ks) const { return i < nf ? ks : ks >> lp; }
+};
+// The estimated share of a launch's time that cutting its left-over tiles must
+// save for the kernel with cut tiles to be taken (it is 2 - 4 % slower by itself).
+constexpr double kSplitGain = 0.05;
+// Share of a launch's time that cutting its left-over tiles saves on `sms` CTAs.
+static double split_gain(int tiles, int chain, int sms) {
+  const int g = (int)std::min<int64_t>(sms, 4 * (int64_t)tiles + chain), a = (tiles + chain) / g;
+  const int nb = a == 0 ? g - chain : g, rem = tiles - std::max(a * g - chain, 0);
+  if (nb <= 0) return 0.0;
+  int cut = 0;
+  const int whole = rem > 0 ? (rem + nb - 1) / nb * (64 + kPartCost) : 0;
+  wave_parts(rem, nb, cut);
+  const double total = (double)a * (64 + kPartCost) + whole;
+  return total > 0 ? (whole - cut) / total : 0.0;
+}
+
+template <class Op, int BK, bool RED, bool SPLIT>
 __global__ void __launch_bounds__(P3W_THREADS, 1)
     fw_phase3_ws(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                  const __grid_constant__ CUtensorMap mapBs, const __grid_constant__ CUtensorMap mapC,
@@ -599,6 +725,8 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   static_assert(Map::THREADS + 32 == P3W_THREADS, "one producer warp after the consumers");
   constexpr int STAGE = P3T<BK>::STAGE_BYTES;
   constexpr int KS = P3T<BK>::KS, NSPLIT = P3T<BK>::NSPLIT;  // k-steps per stage, stages per tile
+  using Walk = typename std::conditional<SPLIT, TileWalk<Op>, TileRun<Op>>::type;
+  constexpr int KBOX = SPLIT ? kPartBox : KS;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_ab[2], empty_ab[2], full_c, cdone, cfree;
   __shared__ int abort_flag;
@@ -608,7 +736,6 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tiles_x = rd.tiles_x, tiles_y = rd.tiles_y;
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&full_ab[i], 1);
@@ -628,11 +755,12 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   const int sym = rd.sym_flag ? (__ldcg(rd.sym_flag) == 0 ? 1 : 0) : rd.sym;
   const CUtensorMap &mapP = sym ? mapBs : mapB;  // the B operand: the symmetric panel, or D's rows
   const int chain = (BK == 64 && rd.q0 >= 0) ? 1 : 0;
-  const int items = (sym ? rd.tiles_sym : rd.tiles_gen) + chain;
-  const int per = items / (int)gridDim.x, extra = items % (int)gridDim.x;
-  const int i_begin = (int)blockIdx.x * per + min((int)blockIdx.x, extra);
-  const int i_end = i_begin + per + ((int)blockIdx.x < extra ? 1 : 0);
-  const int t_begin = max(i_begin - chain, 0), t_end = i_end - chain;  // item 0 is the next_diag task
+  Walk walk;
+  walk.tiles_x = rd.tiles_x;
+  walk.tiles_y = rd.tiles_y;
+  walk.sym = sym;
+  walk.plan(sym ? rd.tiles_sym : rd.tiles_gen, chain);
+  const int t_begin = SPLIT ? 0 : walk.first, t_end = t_begin + walk.nu;
   if constexpr (BK == 64) {
     if (chain && blockIdx.x == 0) {
       static_assert(sizeof(NextDiagSmem<Op>) <= P3T_C_BYTES, "next_diag runs in the C buffer");
@@ -644,23 +772,9 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
     }
   }
   if (t_begin >= t_end) return;
-
-  // first tile of this CTA and the row-major step over the (symmetric) tile set
-  int ty0, tx0;
-  if (!sym) {
-    ty0 = t_begin / tiles_x;
-    tx0 = t_begin % tiles_x;
-  } else {
-    int lo = 0, hi = tiles_y - 1;  // last tile row whose prefix <= t_begin
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (sym_prefix(mid, tiles_x, Op::EPW) <= t_begin) lo = mid;
-      else hi = mid - 1;
-    }
-    ty0 = lo;
-    tx0 = lo / Op::EPW + (int)(t_begin - sym_prefix(lo, tiles_x, Op::EPW));
-  }
-  auto step = [&](int &ty_, int &tx_) {
+  walk.begin();
+  const int tiles_x = rd.tiles_x;
+  auto step = [&](int &ty_, int &tx_) {  // row-major over the (symmetric) tile set
     if (++tx_ == tiles_x) {
       ++ty_;
       tx_ = sym ? ty_ / Op::EPW : 0;
@@ -686,11 +800,14 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
     if (lane == 0) {
       int n_ab[2] = {0, 0}, n_c = 0;
       bool ok = true;
-      // k-steps [h * KS, (h + 1) * KS) of tile (ty_, tx_) into stage s
-      auto issue_ab = [&](int ty_, int tx_, int h, int s) {
-        mbar_arrive_expect_tx(&full_ab[s], STAGE);
-        tma_load_2d(stA(s), &mapA, &full_ab[s], ty_ * BM, h * KS);
-        tma_load_2d(stB(s), &mapP, &full_ab[s], tx_ * BNW * Op::EPW, (sym ? 0 : (int)p0) + h * KS);
+      // the k-steps from k0 that the stage takes, of tile (ty, tx), into stage s
+      auto issue_ab = [&](const Walk &w, int h, int s) {
+        const int kn = w.ksteps(KS), k0 = h * KS + w.part * kn;
+        mbar_arrive_expect_tx(&full_ab[s], kn * 128 * 4 * 2);
+        for (int r = 0; r < kn; r += KBOX) {
+          tma_load_2d(stA(s) + r * BM, &mapA, &full_ab[s], w.ty * BM, k0 + r);
+          tma_load_2d(stB(s) + r * BNW, &mapP, &full_ab[s], w.tx * BNW * Op::EPW, (sym ? 0 : (int)p0) + k0 + r);
+        }
         if (s == 0) ++n_ab[0];
         else ++n_ab[1];
       };
@@ -701,25 +818,24 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
         tma_load_2d(Cs, &mapC, &full_c, x, y);
         ++n_c;
       };
-      // the item stream: (tile, k-part h) in tile order, item j in stage j & 1
-      const int n_items = (t_end - t_begin) * NSPLIT;
-      int aty = ty0, atx = tx0, ah = 0;  // next item to load
+      // the item stream: (tile or part, stage h of it) in order, item j in stage j & 1
+      const int nu = t_end - t_begin, n_items = nu * NSPLIT;
+      Walk ld = walk, out = walk;  // next item to load, next result to write
+      int ah = 0;
       auto next_item = [&]() {
         if (++ah == NSPLIT) {
           ah = 0;
-          step(aty, atx);
+          ld.next();
         }
       };
-      int cty = ty0, ctx = tx0;  // tile whose result is written next
-      issue_ab(aty, atx, ah, 0);
+      issue_ab(ld, ah, 0);
       next_item();
       if (n_items > 1) {
-        issue_ab(aty, atx, ah, 1);
+        issue_ab(ld, ah, 1);
         next_item();
       }
-      if (!RED) issue_c(cty, ctx);
-      for (int t = t_begin; t < t_end; ++t) {
-        const int i = t - t_begin;
+      if (!RED) issue_c(out.ty, out.tx);
+      for (int i = 0; i < nu; ++i) {
         for (int h = 0; h < NSPLIT; ++h) {
           const int j = i * NSPLIT + h, s = j & 1;
           if (!mbar_wait_sleep_bounded(&empty_ab[s], (uint32_t)(j >> 1) & 1u, P3T_WAIT_LIMIT, P3T_SLEEP_NS)) {
@@ -727,7 +843,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
             break;
           }
           if (j + 2 < n_items) {
-            issue_ab(aty, atx, ah, s);
+            issue_ab(ld, ah, s);
             next_item();
           }
         }
@@ -736,9 +852,9 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
           ok = false;
           break;
         }
-        const int r0 = cty * BM, c0 = ctx * BNW * Op::EPW;
+        const int r0 = out.ty * BM, c0 = out.tx * BNW * Op::EPW;
         int cx, cy;
-        cxy(cty, ctx, cx, cy);
+        cxy(out.ty, out.tx, cx, cy);
         if (RED) {
           if (c0 < ncr) {  // a dense D's mapC ends at red_cols(n) in this mode
             tma_reduce_min_2d(&mapC, Cs, cx, cy);
@@ -751,8 +867,8 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
           bulk_commit();
           bulk_wait_read_all();
         }
-        step(cty, ctx);
-        if (!RED && t + 1 < t_end) issue_c(cty, ctx);
+        out.next();
+        if (!RED && i + 1 < nu) issue_c(out.ty, out.tx);
       }
       bulk_wait_all();
       if (!ok) {
@@ -765,7 +881,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   } else {
     // ------------------------------------------------------------ consumers
     const int tx = tid % Map::TX, ty = tid / Map::TX;
-    int cty = ty0, ctx = tx0;
+    int cty = walk.ty, ctx = walk.tx;
     uint32_t acc[8][TN];
     for (int t = t_begin; t < t_end; ++t) {
       const int i = t - t_begin;
@@ -775,11 +891,12 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
         for (int c = 0; c < TN; ++c) acc[r][c] = Op::INF_WORD;
       bool bad = false;
 #pragma unroll 1
-      for (int h = 0; h < NSPLIT; ++h) {  // the tile's k-parts, one stage each (one copy of the k-loop)
+      for (int h = 0; h < NSPLIT; ++h) {  // the tile's stages (one copy of the k-loop)
         const int j = i * NSPLIT + h, s = j & 1;
         bad = !mbar_wait_bounded(&full_ab[s], (uint32_t)(j >> 1) & 1u, P3T_WAIT_LIMIT);
         if (__any_sync(0xffffffffu, bad)) break;
-        tile_minplus<Op, BM, BNW, KS, TN, typename P3Loop<Op, BK>::Round>(stA(s), stB(s), acc, ty, tx);
+        tile_minplus<Op, BM, BNW, KS, TN, typename P3Loop<Op, BK>::Round>(stA(s), stB(s), acc, ty, tx,
+                                                                                   walk.ksteps(KS));
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty_ab[s]);
       }
@@ -830,7 +947,13 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&cdone);
-      step(cty, ctx);
+      if constexpr (SPLIT) {
+        walk.next();
+        cty = walk.ty;
+        ctx = walk.tx;
+      } else {
+        step(cty, ctx);
+      }
     }
   }
   __syncthreads();
@@ -2193,6 +2316,16 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
   }
   e = cudaFuncSetAttribute(fw_phase3<Op, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM3);
   if (e != cudaSuccess) return e;
+  const int tiles_x = (int)((n + 128 * Op::EPW - 1) / (128 * Op::EPW));
+  const int tiles_y = (int)((n + 127) / 128);
+  const int tiles_gen = tiles_x * tiles_y;
+  int tiles_sym = 0;  // tiles with tx >= ty / EPW
+  for (int y = 0; y < tiles_y; ++y) tiles_sym += tiles_x - std::min(tiles_x, y / Op::EPW);
+  // cut left-over tiles where that gains in the mode the solve is expected to run in
+  constexpr bool CAN_SPLIT = kRedOp<Op> && BK == 64;
+  const bool split = CAN_SPLIT && variant == 3 && !la_on && q > 1 &&
+                     split_gain(any_sym ? tiles_sym : tiles_gen, 1, sms) > kSplitGain;
+  const uint32_t kbox = split ? kPartBox : KS;
   // persistent TMA Phase 3 when D is 16-byte addressable (otherwise the
   // per-tile kernel with scalar edge handling); A (and B in symmetric mode)
   // maps for each panel buffer
@@ -2205,13 +2338,13 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
                                                         : CU_TENSOR_MAP_DATA_TYPE_INT32;
     for (int b = 0; b < (la_on ? 2 : 1) && tma; ++b)
       tma = make_map(&mA[b], CU_TENSOR_MAP_DATA_TYPE_UINT32, colTb[b], (uint64_t)ldT, (uint64_t)BK,
-                     (uint64_t)ldT * 4, 128, KS) &&
+                     (uint64_t)ldT * 4, 128, kbox) &&
             (sym ? make_map(&mB[b], dt, symB_of(b), (uint64_t)ldT, (uint64_t)BK, (uint64_t)ldT * sizeof(E),
-                            128 * Op::EPW, KS)
-                 : make_map(&mB[b], dt, D, (uint64_t)n, (uint64_t)n, (uint64_t)ld * sizeof(E), 128 * Op::EPW, KS));
+                            128 * Op::EPW, kbox)
+                 : make_map(&mB[b], dt, D, (uint64_t)n, (uint64_t)n, (uint64_t)ld * sizeof(E), 128 * Op::EPW, kbox));
     for (int b = 0; b < 2 && dev_sym && tma; ++b)
       tma = make_map(&mBs[b], dt, symB_any(b), (uint64_t)ldT, (uint64_t)BK, (uint64_t)ldT * sizeof(E), 128 * Op::EPW,
-                     KS);
+                     kbox);
     // int32 and fp32 (TMA min-reduction epilogue of variant 3): x extent
     // red_cols(n), and an int32 map (fp32 bits of non-negative values order
     // like int32); upper-triangular storage: the whole rectangle
@@ -2232,8 +2365,12 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
                                    P3T<BK>::SMEM);
       }
       if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fw_phase3_ws<Op, BK, kRedOp<Op>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(fw_phase3_ws<Op, BK, kRedOp<Op>, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  P3T<BK>::SMEM);
+      if constexpr (CAN_SPLIT)
+        if (e == cudaSuccess)
+          e = cudaFuncSetAttribute(fw_phase3_ws<Op, BK, kRedOp<Op>, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   P3T<BK>::SMEM);
       if (e != cudaSuccess) return e;
     }
   }
@@ -2243,11 +2380,6 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
     colTb[1] = colT;
     rowPb[1] = rowP;
   }
-  const int tiles_x = (int)((n + 128 * Op::EPW - 1) / (128 * Op::EPW));
-  const int tiles_y = (int)((n + 127) / 128);
-  const int tiles_gen = tiles_x * tiles_y;
-  int tiles_sym = 0;  // tiles with tx >= ty / EPW
-  for (int y = 0; y < tiles_y; ++y) tiles_sym += tiles_x - std::min(tiles_x, y / Op::EPW);
   const int tiles_total = sym ? tiles_sym : tiles_gen;
   const int grid_tma = std::min(sms, tiles_total);
   // width 64: the warp-specialized Phase 3 closes the next round's diagonal block
@@ -2353,9 +2485,17 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
         rd.ldT = ldT;
         rd.symB = any_sym ? symB_any(0) : nullptr;
         rd.diag = diag;
-        const int grid = std::min(sms, tiles_total + (rd.q0 >= 0 ? 1 : 0));
-        launch_pdl(fw_phase3_ws<Op, BK, kRedOp<Op>>, dim3(grid), dim3(P3W_THREADS), (size_t)P3T<BK>::SMEM, s, mA[0],
-                   mB[0], dev_sym ? mBs[0] : mB[0], mC, D, L, n, p0, p1, err, rd);
+        const int grid = (int)std::min<int64_t>(sms, (split ? 4 : 1) * (int64_t)tiles_total + (rd.q0 >= 0 ? 1 : 0));
+        auto go = [&](auto k3) {
+          launch_pdl(k3, dim3(grid), dim3(P3W_THREADS), (size_t)P3T<BK>::SMEM, s, mA[0], mB[0],
+                     dev_sym ? mBs[0] : mB[0], mC, D, L, n, p0, p1, err, rd);
+        };
+        if constexpr (CAN_SPLIT) {
+          if (split) go(fw_phase3_ws<Op, BK, kRedOp<Op>, true>);
+          else go(fw_phase3_ws<Op, BK, kRedOp<Op>, false>);
+        } else {
+          go(fw_phase3_ws<Op, BK, kRedOp<Op>, false>);
+        }
       } else if constexpr (BK <= 64) {
         if (tma && variant == 2)
           fw_phase3_tma<Op, BK, 4><<<grid_tma, TileMap<128, 128, 4>::THREADS, P3T<BK>::SMEM, s>>>(

@@ -85,6 +85,26 @@ inline int default_round_width(int64_t n, int dtype) {
   return dtype != 0 && default_phase3(n, dtype) == 3 && n >= 6144 ? 128 : 64;
 }
 
+// The Phase-3 kernel a solve runs with when neither the caller nor the autotuner
+// chose one: default_phase3, except that the single launch is kept only where it
+// is still the faster one.
+// With two launches a round (fw_panels and a Phase 3 that closes the next
+// diagonal block) the per-round path no longer pays for the chain of small
+// launches that the single launch was made to hide; the single launch still
+// gains, for the integer types, where a round is a few dozen waves of tiles, by
+// starting a round's tiles before the previous round's last wave has ended.
+// Measured (symmetric mode, ms per solve, per round / single launch): int32
+// n = 6144 7.07 / 7.98, 7168 10.9 / 10.9, 8192 15.4 / 14.7, 12288 47.8 / 47.4,
+// 16384 108.7 / 109.5; packed 16-bit n = 6144 4.52 / 7.03, 8192 10.1 / 11.6,
+// 10240 18.1 / 17.1, 24576 205.0 / 201.1, 49152 1498 / 1534; fp32 n = 6144
+// 6.92 / 8.06, 8192 15.1 / 15.5, 16384 105.7 / 113.9.
+inline int solve_phase3(int64_t n, int dtype) {
+  if (default_phase3(n, dtype) != 4) return 3;
+  if (dtype == 0) return n >= 7680 && n < 14336 ? 4 : 3;
+  if (dtype == 1) return n >= 9216 && n < 32768 ? 4 : 3;
+  return 3;
+}
+
 // flag |= 1 when D (n x n, leading dimension ld) is not symmetric.
 cudaError_t launch_symmetry_check(int dtype, const void *D, int64_t n, int64_t ld, int *flag, cudaStream_t s);
 constexpr int64_t kMaxRoundWidth = 128;  // panel buffers are sized for this (the widest round)
