@@ -284,9 +284,6 @@ bool aligned_copy_fits(apsp_handle *h, size_t bytes) {
   return bytes <= tot / 8 && bytes <= fr / 2;
 }
 
-apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
-                               bool known_sym, apsp::RoundConfig rc);
-
 // The shape a solve runs with: config_for, except that kernel 4 as a default
 // (neither forced nor tuned) runs as kernel 3 where that is faster.
 apsp::RoundConfig run_config(apsp_handle *h, int dtype, int64_t n) {
@@ -297,39 +294,81 @@ apsp::RoundConfig run_config(apsp_handle *h, int dtype, int64_t n) {
   return c;
 }
 
-// Enqueues the q rounds on D (already holding W) using the handle's panel buffer.
-// known_sym: D is symmetric by construction (edge-list input).
-apsp_status run_rounds_locked(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
-                              bool known_sym = false) {
-  const apsp::RoundConfig rc = run_config(h, dtype, n);
+apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
+                               bool known_sym, apsp::RoundConfig rc, bool flag_ready);
+
+// The matrix the rounds of D run on: D, or the handle's copy with 16-byte rows;
+// *ldm its leading dimension.
+void *round_matrix(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, const apsp::RoundConfig &rc,
+                   int64_t *ldm) {
   int64_t ldc = 0;
   if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc)) {
     const size_t bytes = (size_t)n * ldc * (dtype == APSP_U16 ? 2 : 4);
     if (aligned_copy_fits(h, bytes)) {
       if (ensure(&h->wsD, &h->wsD_bytes, bytes) == cudaSuccess) {
-        int64_t l = 0;
-        cudaError_t e = apsp::launch_copy(dtype, D, ld, h->wsD, ldc, n, s, &l);
-        if (e == cudaSuccess) {
-          const apsp_status st = run_rounds_aligned(h, dtype, h->wsD, n, ldc, s, known_sym, rc);
-          if (st != APSP_OK) return st;
-          e = apsp::launch_copy(dtype, h->wsD, ldc, D, ld, n, s, &l);
-        }
-        h->launches += l;
-        if (e != cudaSuccess) {
-          h->last_error = std::string("aligned copy: ") + cudaGetErrorString(e);
-          return APSP_E_CUDA;
-        }
-        return APSP_OK;
+        *ldm = ldc;
+        return h->wsD;
       }
       cudaGetLastError();  // out of memory: the kernel for any alignment
     }
   }
-  return run_rounds_aligned(h, dtype, D, n, ld, s, known_sym, rc);
+  *ldm = ld;
+  return D;
 }
 
-// The rounds on D itself.
+// Enqueues the q rounds on D (already holding W) using the handle's panel buffer.
+// known_sym: D is symmetric by construction (edge-list input).
+apsp_status run_rounds_locked(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
+                              bool known_sym = false) {
+  apsp::RoundConfig rc = run_config(h, dtype, n);
+  int64_t ldm = ld, l = 0;
+  void *M = round_matrix(h, dtype, D, n, ld, rc, &ldm);
+  if (M != D) {
+    const cudaError_t e = apsp::launch_input(dtype, D, ld, M, ldm, n, nullptr, nullptr, s, &l);
+    h->launches += l;
+    if (e != cudaSuccess) {
+      h->last_error = std::string("aligned copy: ") + cudaGetErrorString(e);
+      return APSP_E_CUDA;
+    }
+    rc.out = D;
+    rc.out_ld = ld;
+  }
+  return run_rounds_aligned(h, dtype, M, n, ldm, s, known_sym, rc, false);
+}
+
+// The input pass from W and the q rounds into D (status word and symmetry flag zeroed).
+apsp_status solve_dense_locked(apsp_handle *h, int dtype, const void *W, int64_t n, int64_t ld, void *D,
+                               cudaStream_t s) {
+  apsp::RoundConfig rc = run_config(h, dtype, n);
+  int64_t ldm = ld, l = 0;
+  void *M = round_matrix(h, dtype, D, n, ld, rc, &ldm);
+  if (M != D) {
+    rc.out = D;
+    rc.out_ld = ld;
+  }
+  const bool flag = h->cfg.symmetric == 0 && n > 1;  // the symmetry flag lies behind the status word
+  const cudaError_t e =
+      apsp::launch_input(dtype, W, ld, M, ldm, n, h->d_status, flag ? h->d_status + 1 : nullptr, s, &l);
+  h->launches += l;
+  if (e != cudaSuccess) {
+    h->last_error = std::string("ingest: ") + cudaGetErrorString(e);
+    return APSP_E_CUDA;
+  }
+  return run_rounds_aligned(h, dtype, M, n, ldm, s, false, rc, flag);
+}
+
+// D's symmetry flag into d_status[1], unless the input pass has put it there.
+cudaError_t check_symmetry(apsp_handle *h, int dtype, const void *D, int64_t n, int64_t ld, bool ready,
+                           cudaStream_t s) {
+  if (ready) return cudaSuccess;
+  h->launches += 1;
+  const cudaError_t e = cudaMemsetAsync(h->d_status + 1, 0, sizeof(int), s);
+  return e != cudaSuccess ? e : apsp::launch_symmetry_check(dtype, D, n, ld, h->d_status + 1, s);
+}
+
+// The rounds on D itself.  flag_ready: the symmetry flag of D is in place.
 apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s,
-                               bool known_sym, apsp::RoundConfig rc) {
+                               bool known_sym, apsp::RoundConfig rc, bool flag_ready) {
   const int64_t ldT = panel_ld(n);
   cudaError_t e = ensure(&h->colT, &h->colT_bytes, apsp::panel_buffer_bytes(n, ldT, rc.p3 == 4));
   if (e != cudaSuccess) {
@@ -342,26 +381,22 @@ apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, in
     // device check of W == W^T whose answer the kernels read themselves:
     // no host round trip before the rounds are enqueued
     int *flag = h->d_status + 1;
-    e = cudaMemsetAsync(flag, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = apsp::launch_symmetry_check(dtype, D, n, ld, flag, s);
+    e = check_symmetry(h, dtype, D, n, ld, flag_ready, s);
     if (e != cudaSuccess) {
       h->last_error = std::string("symmetry check: ") + cudaGetErrorString(e);
       return APSP_E_CUDA;
     }
-    h->launches += 1;
     rc.sym_flag = flag;
   } else if (h->cfg.symmetric == 0 && n > 1) {
     // device check of W == W^T; the answer is read back before the rounds are enqueued
     int *flag = h->d_status + 1;
-    e = cudaMemsetAsync(flag, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = apsp::launch_symmetry_check(dtype, D, n, ld, flag, s);
+    e = check_symmetry(h, dtype, D, n, ld, flag_ready, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_status + 1, flag, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
       h->last_error = std::string("symmetry check: ") + cudaGetErrorString(e);
       return APSP_E_CUDA;
     }
-    h->launches += 1;
     rc.sym = h->h_status[1] == 0;
   }
   if ((rc.sym || rc.sym_flag) && dtype == APSP_U16) {
@@ -383,22 +418,14 @@ apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, in
 }
 
 apsp_status solve_locked(apsp_handle *h, int dtype, const void *W, int64_t n, int64_t ld, void *D, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(h->d_status, 0, sizeof(int), s);
+  cudaError_t e = cudaMemsetAsync(h->d_status, 0, 2 * sizeof(int), s);  // status and symmetry flag
   if (e != cudaSuccess) {
     h->last_error = std::string("status reset: ") + cudaGetErrorString(e);
     return APSP_E_CUDA;
   }
   if (n == 0) return APSP_OK;
   int64_t l = 0;
-  if (dtype != APSP_AUTO) {
-    e = apsp::launch_ingest(dtype, W, D, n, ld, h->d_status, s, &l);
-    h->launches += l;
-    if (e != cudaSuccess) {
-      h->last_error = std::string("ingest: ") + cudaGetErrorString(e);
-      return APSP_E_CUDA;
-    }
-    return run_rounds_locked(h, dtype, D, n, ld, s);
-  }
+  if (dtype != APSP_AUTO) return solve_dense_locked(h, dtype, W, n, ld, D, s);
   // AUTO: int32 in and out; packed 16-bit when the bound allows (precision
   // selection).  The bound synchronizes the stream.
   e = apsp::launch_ingest(APSP_I32, W, const_cast<void *>(W), n, ld, h->d_status, s, &l);  // checks only (W == D: no copy)
@@ -1364,7 +1391,9 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
     // (symmetric) matrix takes the symmetric mode, decided by a device check
     const int64_t rn = rs[0]->req.n;
     const int64_t ldT = panel_ld(rn);
-    if (rn > 0 && apsp::launch_ingest(APSP_I32, rs[0]->D, rs[0]->D, rn, rn, g->status, s, &l) != cudaSuccess)
+    const bool checked = rs[0]->req.dtype == APSP_AUTO;  // otherwise with the symmetry check, below
+    if (rn > 0 && checked &&
+        apsp::launch_ingest(APSP_I32, rs[0]->D, rs[0]->D, rn, rn, g->status, s, &l) != cudaSuccess)
       return APSP_E_CUDA;
     if (rs[0]->req.dtype == APSP_AUTO) {
       // precision selection: the 16-bit bound (synchronizes the group's
@@ -1413,17 +1442,20 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
     }
     if (copy) {
       M = static_cast<char *>(g->ws) + pb;
-      if (apsp::launch_copy(APSP_I32, rs[0]->D, rn, M, ldm, rn, s, &l) != cudaSuccess) return APSP_E_CUDA;
+      rc.out = rs[0]->D;
+      rc.out_ld = rn;
     }
+    int *dflag = g->status + 2;  // zeroed with the status words
+    if (rn > 0 && apsp::launch_input(APSP_I32, rs[0]->D, rn, M, ldm, rn, checked ? nullptr : g->status,
+                                     h->cfg.symmetric == 0 ? dflag : nullptr, s, &l) != cudaSuccess)
+      return APSP_E_CUDA;
     if (h->cfg.symmetric == 1) {
       rc.sym = true;
     } else if (h->cfg.symmetric == 0) {
-      int *dflag = g->status + 2;  // zeroed with the status words
-      if (apsp::launch_symmetry_check(APSP_I32, M, rn, ldm, dflag, s) != cudaSuccess) return APSP_E_CUDA;
       if (apsp::device_sym(APSP_I32, M, ldm, rn, rc)) {
         rc.sym_flag = dflag;  // the kernels read the answer themselves
       } else {
-        // one launch per round: the answer is read back before the rounds are enqueued
+        // otherwise it is read back before the rounds are enqueued
         int flag = 0;
         if (cudaMemcpyAsync(&flag, dflag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
@@ -1433,7 +1465,6 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
     }
     if (apsp::launch_rounds(APSP_I32, M, ldm, rn, g->ws, ldT, s, &l, nullptr, rc, g->status + 1) != cudaSuccess)
       return APSP_E_CUDA;
-    if (copy && apsp::launch_copy(APSP_I32, M, ldm, rs[0]->D, rn, rn, s, &l) != cudaSuccess) return APSP_E_CUDA;
     h->launches += l;
     if (cudaEventRecord(g->done_ev, s) != cudaSuccess) return APSP_E_CUDA;
     g->graphs_dev = nullptr;

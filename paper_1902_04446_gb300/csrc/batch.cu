@@ -38,6 +38,7 @@
 
 #include "batch.h"
 #include "fw_panels.cuh"
+#include "fw_passes.cuh"
 #include "fw_tasks.cuh"
 
 namespace apsp {
@@ -164,13 +165,6 @@ __global__ void __launch_bounds__(NT, 2)
   }
 }
 
-// Pair p of mirrored blocks (R, C), R >= C, counted row by row.
-__device__ __forceinline__ void pair_of(int p, int &R, int &C) {
-  R = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
-  while ((long long)R * (R + 1) / 2 > p) --R;
-  while ((long long)(R + 1) * (R + 2) / 2 <= p) ++R;
-  C = p - (int)((long long)R * (R + 1) / 2);
-}
 __device__ __forceinline__ int graph_of_pair(const BatchGraph *G, int count, int p) {
   int lo = 0, hi = count - 1;  // last graph with pair_base <= p
   while (lo < hi) {
@@ -182,7 +176,7 @@ __device__ __forceinline__ int graph_of_pair(const BatchGraph *G, int count, int
 }
 
 // Checks, copies (W != M) and compares the mirrored blocks of one pair: the
-// conventions of ingest_kernel (status |= 1 invalid, 2 range).
+// conventions of input_pairs_kernel (status |= 1 invalid, 2 range).
 __global__ void __launch_bounds__(256) batch_input_kernel(BatchGraph *G, int count) {
   __shared__ int32_t tile[64][65];
   const int gi = graph_of_pair(G, count, blockIdx.x);

@@ -31,10 +31,16 @@ __global__ void init_keys(unsigned long long *key, int64_t n) {
     key[v] = (unsigned long long)v << 32;
 }
 
+// `inner` sweeps over the edges, each thread over its own without waiting for
+// the others: keys only fall, and a launch in which no thread lowered any key
+// has checked every edge against the final keys, so any order gives the same
+// result.  A sweep of its own launch costs 5 us at 120 thousand edges, most of
+// it launch latency; inside a launch it is one round trip to L2.
 template <typename WT>
 __global__ void bf_sweep(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, const WT *__restrict__ w,
-                         int64_t m, int64_t n, uint64_t inf, unsigned long long *key, int *changed) {
+                         int64_t m, int64_t n, uint64_t inf, unsigned long long *key, int *changed, int inner) {
   int ch = 0;
+  for (int it = 0; it < inner; ++it)
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t u = src[e], v = dst[e];
     const WT wt = w[e];
@@ -122,23 +128,29 @@ __global__ void fill_edges(const int32_t *__restrict__ W, int64_t n, int64_t ld,
   int bad = 0;
   for (int64_t i = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; i < n; i += warps) {
     int64_t pos = off[i];
-    for (int64_t j0 = 0; j0 < n; j0 += 32) {
-      const int64_t j = j0 + lane;
-      int32_t x = 0;
-      bool keep = false;
-      if (j < n) {
-        x = W[i * ld + j];
-        keep = (j != i && x < 1073741823);
+    constexpr int U = 8;  // loads in flight: one at a time the row's scan is a chain of memory latencies
+    for (int64_t j0 = 0; j0 < n; j0 += 32 * U) {
+      int32_t xs[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t j = j0 + 32 * u + lane;
+        xs[u] = j < n ? W[i * ld + j] : 1073741823;
       }
-      const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
-      if (keep) {
-        const int64_t p = pos + __popc(bal & ((1u << lane) - 1u));
-        src[p] = (int32_t)i;
-        dst[p] = (int32_t)j;
-        w[p] = x;
-        if (W[j * ld + i] != x) bad = 1;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t j = j0 + 32 * u + lane;
+        const int32_t x = xs[u];
+        const bool keep = j < n && j != i && x < 1073741823;
+        const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
+        if (keep) {
+          const int64_t p = pos + __popc(bal & ((1u << lane) - 1u));
+          src[p] = (int32_t)i;
+          dst[p] = (int32_t)j;
+          w[p] = x;
+          if (W[j * ld + i] != x) bad = 1;
+        }
+        pos += __popc(bal);
       }
-      pos += __popc(bal);
     }
   }
   if (bad) *asym = 1;
@@ -163,7 +175,8 @@ cudaError_t run_bf(const int32_t *src, const int32_t *dst, const WT *w, int64_t 
   *bound = 0;
   *ok = 1;
   if (n <= 0) return cudaSuccess;
-  constexpr int kMaxGroup = 64;  // sweeps between two host checks, at most
+  constexpr int kMaxGroup = 16;  // launches between two host checks, at most
+  constexpr int kInner = 8;      // sweeps per launch
   DevBuf keyb(s), aux(s);
   cudaError_t e = keyb.alloc((size_t)n * sizeof(unsigned long long));
   if (e != cudaSuccess) return e;
@@ -179,15 +192,16 @@ cudaError_t run_bf(const int32_t *src, const int32_t *dst, const WT *w, int64_t 
   const unsigned ge = (unsigned)(eb < 1 ? 1 : (eb > 152 * 8 ? 152 * 8 : eb));
   // At most n + 1 sweeps are needed (each sweep fixes one more hop of every
   // shortest-path tree); a sweep that changes nothing means the keys are final.
-  // Sweeps run in groups between host checks, each sweep with its own flag;
-  // the groups double (4, 8, ..., 64) so that deep graphs need few round trips
-  // while shallow ones stop after a few sweeps.
+  // Launches of kInner sweeps run in groups between host checks, each launch with
+  // its own flag; the groups double (2, 4, ..., 16) so that deep graphs need few
+  // round trips while shallow ones stop after a few sweeps.
   bool converged = false;
   int h_flags[kMaxGroup];
-  for (int64_t done = 0, group = 4; !converged && done <= n + 1; done += group, group = std::min<int64_t>(2 * group, kMaxGroup)) {
+  for (int64_t done = 0, group = 2; !converged && done <= n + 1;
+       done += kInner * group, group = std::min<int64_t>(2 * group, kMaxGroup)) {
     e = cudaMemsetAsync(changed, 0, (size_t)group * sizeof(int), s);
     if (e != cudaSuccess) return e;
-    for (int r = 0; r < group; ++r) bf_sweep<WT><<<ge, 256, 0, s>>>(src, dst, w, m, n, inf, key, changed + r);
+    for (int r = 0; r < group; ++r) bf_sweep<WT><<<ge, 256, 0, s>>>(src, dst, w, m, n, inf, key, changed + r, kInner);
     *launches += group;
     e = cudaMemcpyAsync(h_flags, changed, (size_t)group * sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return e;

@@ -36,6 +36,7 @@
 #include "fw_device.cuh"
 #include "fw_launch.h"
 #include "fw_panels.cuh"
+#include "fw_passes.cuh"
 #include "fw_tasks.cuh"
 #include "tma.cuh"
 
@@ -242,48 +243,6 @@ __global__ void __launch_bounds__(P1_THREADS) fw_phase1_sym(typename Op::elem *_
   pdl_trigger();
   pdl_wait();
   phase1_body<Op, BK, P1_THREADS, false>(D, L, n, p0, colT, ldT, s, threadIdx.x, rowP);
-}
-
-// ---------------------------------------------------------------- symmetry
-// D[r][c] = D[c][r] for every r > c (the lower triangle from the upper), by
-// 32 x 32 blocks through shared memory; block (R, C) with R >= C.
-template <class Op>
-__global__ void mirror_kernel(typename Op::elem *__restrict__ D, int64_t n, int64_t ld, const int *sym_flag) {
-  __shared__ typename Op::elem tile[32][33];
-  if (sym_flag && *sym_flag != 0) return;  // the device found D not symmetric: the general path ran
-  const int64_t R = blockIdx.y, Cb = blockIdx.x;
-  if (R < Cb) return;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  // read block (Cb, R) of the upper triangle: rows Cb*32.., columns R*32..
-  for (int k = ty; k < 32; k += 8) {
-    const int64_t r = Cb * 32 + k, c = R * 32 + tx;
-    if (r < n && c < n) tile[k][tx] = D[r * ld + c];
-  }
-  __syncthreads();
-  for (int k = ty; k < 32; k += 8) {
-    const int64_t r = R * 32 + k, c = Cb * 32 + tx;  // target (r, c) = source (c, r)
-    if (r < n && c < n && r > c) D[r * ld + c] = tile[tx][k];
-  }
-}
-
-// flag |= 1 when some D[r][c] != D[c][r] (compared bitwise), same blocking.
-template <class Op>
-__global__ void symmetry_check_kernel(const typename Op::elem *__restrict__ D, int64_t n, int64_t ld, int *flag) {
-  __shared__ typename Op::elem tile[32][33];
-  const int64_t R = blockIdx.y, Cb = blockIdx.x;
-  if (R < Cb) return;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int k = ty; k < 32; k += 8) {
-    const int64_t r = Cb * 32 + k, c = R * 32 + tx;
-    if (r < n && c < n) tile[k][tx] = D[r * ld + c];
-  }
-  __syncthreads();
-  int bad = 0;
-  for (int k = ty; k < 32; k += 8) {
-    const int64_t r = R * 32 + k, c = Cb * 32 + tx;
-    if (r < n && c < n && elem_bits<Op>(D[r * ld + c]) != elem_bits<Op>(tile[tx][k])) bad = 1;
-  }
-  if (__syncthreads_or(bad) && tx == 0 && ty == 0) atomicOr(flag, 1);
 }
 
 // ---------------------------------------------------------------- Phase 3
@@ -1929,74 +1888,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   if (abort_flag && tid == 0) atomicOr(err, 4);
 }
 
-// ---------------------------------------------------------------- ingest / checks
-// Copies W to D (when they differ) and checks the input: diagonal 0, weights
-// >= 0, finite weights < INF.  status |= 1 (invalid) or 2 (range).
-// fp32: a -0.0 is written as +0.0 (also in place), so that every stored
-// distance is a non-negative float whose bit pattern orders like the value
-// under a signed int32 compare -- the Phase-3 tiles leave by an int32 TMA
-// min-reduction on those bits.
-template <class Op>
-__global__ void ingest_kernel(const typename Op::elem *__restrict__ W, typename Op::elem *__restrict__ D, int64_t n,
-                              int64_t ld, int copy, int *status) {
-  int bad = 0;
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-      typename Op::elem e = W[i * ld + j];
-      if constexpr (Op::DTYPE == 2) {
-        if (!(e >= 0.0f)) bad |= 1;              // negative or NaN
-        if (i == j && e != 0.0f) bad |= 1;
-        if (__float_as_uint(e) == 0x80000000u) {  // -0.0
-          e = 0.0f;
-          if (!copy) D[i * ld + j] = e;
-        }
-      } else if constexpr (Op::DTYPE == 1) {
-        if (e > Op::inf_elem()) bad |= 2;
-        if (i == j && e != 0) bad |= 1;
-      } else {
-        if (e < 0) bad |= 1;
-        if (e > Op::inf_elem()) bad |= 2;
-        if (i == j && e != 0) bad |= 1;
-      }
-      if (copy) D[i * ld + j] = e;
-    }
-  }
-  if (bad) atomicOr(status, bad);
-}
-
-template <class T>
-__global__ void copy_kernel(const T *__restrict__ s, int64_t lds, T *__restrict__ d, int64_t ldd, int64_t n) {
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-      d[i * ldd + j] = s[i * lds + j];
-}
-
-__global__ void pack_kernel(const int32_t *__restrict__ s, int64_t lds, uint16_t *__restrict__ d, int64_t ldd,
-                            int64_t n) {
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-      const int32_t v = s[i * lds + j];
-      d[i * ldd + j] = (uint16_t)(v >= 0x7FFF ? 0x7FFF : v);
-    }
-}
-
-__global__ void unpack_kernel(const uint16_t *__restrict__ s, int64_t lds, int32_t *__restrict__ d, int64_t ldd,
-                              int64_t n) {
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-      const uint16_t v = s[i * lds + j];
-      d[i * ldd + j] = v >= 0x7FFF ? 1073741823 : (int32_t)v;
-    }
-}
-
-// D = INF off the diagonal, 0 on it (n x n region of D).
-template <class Op>
-__global__ void fill_inf_kernel(typename Op::elem *__restrict__ D, int64_t n, int64_t ld) {
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-      D[i * ld + j] = (i == j) ? (typename Op::elem)0 : Op::inf_elem();
-}
-
+// ---------------------------------------------------------------- edge lists
 // Minimum of a 16-bit element by a 16-bit compare-and-swap loop.
 __device__ __forceinline__ void atomic_min_u16(uint16_t *p, uint16_t v) {
   unsigned short *a = reinterpret_cast<unsigned short *>(p);
@@ -2070,10 +1962,8 @@ __global__ void synth_kernel(typename Op::elem *__restrict__ D, int64_t n, int64
 
 // ---------------------------------------------------------------- upper-triangular storage
 // Every stored element (r, c) of the layout (rows [0, T S), columns
-// [S floor(r / S), T S)): from the dense W when r, c < n (W == nullptr: 0 on
-// the diagonal, INF elsewhere), INF in the padding.  With W, the input is
-// checked as in ingest_kernel (status |= 1 invalid, 2 range); fp32 -0.0 is
-// stored as +0.0.
+// [S floor(r / S), T S)) from the dense W, INF in the padding.  The input is
+// checked (status |= 1 invalid, 2 range); fp32 -0.0 is stored as +0.0.
 template <class Op>
 __global__ void tri_fill_kernel(const typename Op::elem *__restrict__ W, int64_t ldw, typename Op::elem *__restrict__ D,
                                 Layout L, int64_t n, int *status) {
@@ -2087,22 +1977,18 @@ __global__ void tri_fill_kernel(const typename Op::elem *__restrict__ W, int64_t
          c += (int64_t)gridDim.x * blockDim.x) {
       E e = Op::inf_elem();
       if (r < n && c < n) {
-        if (!W) {
-          e = r == c ? (E)0 : Op::inf_elem();
+        e = W[r * ldw + c];
+        if constexpr (Op::DTYPE == 2) {
+          if (!(e >= 0.0f)) bad |= 1;
+          if (r == c && e != 0.0f) bad |= 1;
+          if (e == 0.0f) e = 0.0f;
+        } else if constexpr (Op::DTYPE == 1) {
+          if (e > Op::inf_elem()) bad |= 2;
+          if (r == c && e != 0) bad |= 1;
         } else {
-          e = W[r * ldw + c];
-          if constexpr (Op::DTYPE == 2) {
-            if (!(e >= 0.0f)) bad |= 1;
-            if (r == c && e != 0.0f) bad |= 1;
-            if (e == 0.0f) e = 0.0f;
-          } else if constexpr (Op::DTYPE == 1) {
-            if (e > Op::inf_elem()) bad |= 2;
-            if (r == c && e != 0) bad |= 1;
-          } else {
-            if (e < 0) bad |= 1;
-            if (e > Op::inf_elem()) bad |= 2;
-            if (r == c && e != 0) bad |= 1;
-          }
+          if (e < 0) bad |= 1;
+          if (e > Op::inf_elem()) bad |= 2;
+          if (r == c && e != 0) bad |= 1;
         }
       }
       D[o + c] = e;
@@ -2140,20 +2026,6 @@ __global__ void tri_scatter_edges_kernel(const int32_t *__restrict__ src, const 
     }
   }
   if (bad) atomicOr(status, bad);
-}
-
-// Dense out[r][c] for the stored elements with r, c < n (the lower triangle
-// outside the diagonal super-tiles is filled afterwards by mirror_kernel).
-template <class Op>
-__global__ void tri_to_dense_kernel(const typename Op::elem *__restrict__ D, Layout L, int64_t n,
-                                    typename Op::elem *__restrict__ out, int64_t ldo) {
-  for (int64_t r = blockIdx.y; r < n; r += gridDim.y) {
-    const int64_t c_first = (r >> L.sh) << L.sh;
-    const int64_t o = L.off(r, c_first) - c_first;  // D[o + c] is element (r, c) for stored c
-    for (int64_t c = c_first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-         c += (int64_t)gridDim.x * blockDim.x)
-      out[r * ldo + c] = D[o + c];
-  }
 }
 
 // out[i][c] = D(rows[i], c) for c < n: the stored element, or its mirror
@@ -2249,6 +2121,21 @@ static void launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
   cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);  // errors surface in cudaGetLastError
 }
 
+static bool aligned16(const void *p, int64_t ld, size_t esz) {
+  return (reinterpret_cast<uintptr_t>(p) % 16 == 0) && ((ld * (int64_t)esz) % 16 == 0);
+}
+
+template <class Op>
+static cudaError_t output_pass(const typename Op::elem *M, Layout LM, typename Op::elem *D, int64_t ldd, int64_t n,
+                               bool sym, const int *sym_flag, cudaStream_t s, int64_t *launches) {
+  constexpr size_t es = sizeof(typename Op::elem);
+  output_pairs_kernel<Op><<<(unsigned)block_pairs(n), 256, 0, s>>>(M, LM, aligned16(M, LM.ld, es), D, ldd,
+                                                                  aligned16(D, ldd, es), M != D ? 1 : 0, n, sym ? 1 : 0,
+                                                                  sym_flag);
+  if (launches) *launches += 1;
+  return cudaGetLastError();
+}
+
 // Words per panel chunk of the per-round path.  Measured with 16 / 32 words (ms
 // per solve): int32 n = 2048 0.532 / 0.577, n = 25000 377.0 / 377.2, packed
 // 16-bit n = 4096 1.695 / 1.813, n = 16384 63.7 / 64.0.
@@ -2258,7 +2145,7 @@ template <class Op, int BK>
 static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64_t ldT, bool vec, int variant,
                                cudaStream_t s, int64_t *launches, PhaseTimer *tm, int *wait_err, bool sym,
                                void *rowPv, const int *sym_flag, const int *gate, uint32_t dep_spins,
-                               int grid_cap) {
+                               int grid_cap, void *out, int64_t out_ld) {
   const bool use_tma = variant != 0;
   const int sms = grid_cap > 0 ? std::min(sm_count(), grid_cap) : sm_count();
   using Elem = typename Op::elem;
@@ -2574,16 +2461,12 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
       else tm->after(2, s, work[sym ? 1 : 0]);
     }
   }
-  if ((sym || dev_sym) && q > 1 && !tri) {  // the lower triangle from the upper (not stored when tri)
-    const dim3 gm((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32));
-    mirror_kernel<Op><<<gm, dim3(32, 8), 0, s>>>(D, n, ld, dev_sym ? sym_flag : nullptr);
-    if (launches) *launches += 1;
+  if (out || ((sym || dev_sym) && q > 1 && !tri)) {  // the lower triangle from the upper (not stored when tri)
+    e = output_pass<Op>(D, L, out ? static_cast<E *>(out) : D, out ? out_ld : ld, n, sym && q > 1,
+                        dev_sym && q > 1 ? sym_flag : nullptr, s, launches);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
-}
-
-static bool aligned16(const void *p, int64_t ld, size_t esz) {
-  return (reinterpret_cast<uintptr_t>(p) % 16 == 0) && ((ld * (int64_t)esz) % 16 == 0);
 }
 
 template <class Op>
@@ -2592,13 +2475,13 @@ static cudaError_t rounds_bk(const RoundConfig &cfg, void *D, Layout L, int64_t 
   const bool vec = aligned16(D, L.ld, sizeof(typename Op::elem));
   if (cfg.bk == 32)
     return rounds_impl<Op, 32>(D, L, n, colT, ldT, vec, cfg.p3, s, launches, tm, wait_err, cfg.sym, cfg.rowP,
-                               cfg.sym_flag, cfg.gate, cfg.dep_spins, cfg.grid_cap);
+                               cfg.sym_flag, cfg.gate, cfg.dep_spins, cfg.grid_cap, cfg.out, cfg.out_ld);
   if (cfg.bk == 64)
     return rounds_impl<Op, 64>(D, L, n, colT, ldT, vec, cfg.p3, s, launches, tm, wait_err, cfg.sym, cfg.rowP,
-                               cfg.sym_flag, cfg.gate, cfg.dep_spins, cfg.grid_cap);
+                               cfg.sym_flag, cfg.gate, cfg.dep_spins, cfg.grid_cap, cfg.out, cfg.out_ld);
   if (cfg.bk == 128)
     return rounds_impl<Op, 128>(D, L, n, colT, ldT, vec, cfg.p3, s, launches, tm, wait_err, cfg.sym, cfg.rowP,
-                                cfg.sym_flag, cfg.gate, cfg.dep_spins, cfg.grid_cap);
+                                cfg.sym_flag, cfg.gate, cfg.dep_spins, cfg.grid_cap, cfg.out, cfg.out_ld);
   return cudaErrorInvalidValue;
 }
 
@@ -2612,16 +2495,30 @@ bool device_sym(int dtype, const void *D, int64_t ld, int64_t n, const RoundConf
   return (cfg.p3 == 3 || cfg.p3 == 4) && cfg.bk == 64 && n > 1 && aligned16(D, ld, es);
 }
 
-cudaError_t launch_symmetry_check(int dtype, const void *D, int64_t n, int64_t ld, int *flag, cudaStream_t s) {
+template <class Op>
+static cudaError_t input_pass(const void *W, int64_t ldw, void *M, int64_t ldm, int64_t n, int *status, int *asym,
+                              cudaStream_t s) {
+  using E = typename Op::elem;
+  input_pairs_kernel<Op><<<(unsigned)block_pairs(n), 256, 0, s>>>(
+      static_cast<const E *>(W), ldw, aligned16(W, ldw, sizeof(E)), static_cast<E *>(M), ldm,
+      aligned16(M, ldm, sizeof(E)), W != M ? 1 : 0, n, status, asym);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_input(int dtype, const void *W, int64_t ldw, void *M, int64_t ldm, int64_t n, int *status, int *asym,
+                         cudaStream_t s, int64_t *launches) {
   if (n <= 0) return cudaSuccess;
-  const dim3 g((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32));
+  if (launches) *launches += 1;
   switch (dtype) {
-    case 0: symmetry_check_kernel<OpI32><<<g, dim3(32, 8), 0, s>>>(static_cast<const int32_t *>(D), n, ld, flag); break;
-    case 1: symmetry_check_kernel<OpU16><<<g, dim3(32, 8), 0, s>>>(static_cast<const uint16_t *>(D), n, ld, flag); break;
-    case 2: symmetry_check_kernel<OpF32><<<g, dim3(32, 8), 0, s>>>(static_cast<const float *>(D), n, ld, flag); break;
+    case 0: return input_pass<OpI32>(W, ldw, M, ldm, n, status, asym, s);
+    case 1: return input_pass<OpU16>(W, ldw, M, ldm, n, status, asym, s);
+    case 2: return input_pass<OpF32>(W, ldw, M, ldm, n, status, asym, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+}
+
+cudaError_t launch_symmetry_check(int dtype, const void *D, int64_t n, int64_t ld, int *flag, cudaStream_t s) {
+  return launch_input(dtype, D, ld, const_cast<void *>(D), ld, n, nullptr, flag, s, nullptr);
 }
 
 cudaError_t launch_rounds(int dtype, void *D, int64_t ld, int64_t n, void *colT, int64_t ldT, cudaStream_t s,
@@ -2655,14 +2552,24 @@ cudaError_t launch_rounds_tri(int dtype, void *T, int64_t n, void *colT, int64_t
   }
 }
 
+// grid of 16-byte accesses along the rows, several rows a thread
+template <class Op>
+static dim3 fill_grid(int64_t rows, int64_t cols) {
+  return dim3((unsigned)((cols + 1024 * Op::EPW - 1) / (1024 * Op::EPW)), grid_rows((rows + 3) / 4));
+}
+
 template <class Op>
 static cudaError_t tri_fill_impl(const void *W, int64_t ldw, void *T, int64_t n, int *status, cudaStream_t s,
                                  int64_t *launches) {
   using E = typename Op::elem;
   const Layout L = tri_layout(n, Op::EPW, nullptr);
   const int64_t rows = (int64_t)L.T << L.sh;
-  tri_fill_kernel<Op><<<dim3(grid_cols(rows, 256), grid_rows(rows)), 256, 0, s>>>(static_cast<const E *>(W), ldw,
-                                                                                  static_cast<E *>(T), L, n, status);
+  if (W)
+    tri_fill_kernel<Op><<<dim3(grid_cols(rows, 256), grid_rows(rows)), 256, 0, s>>>(
+        static_cast<const E *>(W), ldw, static_cast<E *>(T), L, n, status);
+  else
+    fill_inf_kernel<Op><<<fill_grid<Op>(rows, rows), 256, 0, s>>>(static_cast<E *>(T), L, rows, rows, n,
+                                                                  aligned16(T, L.ld, sizeof(E)));
   if (launches) *launches += 1;
   return cudaGetLastError();
 }
@@ -2721,12 +2628,7 @@ static cudaError_t tri_out_impl(const void *T, int64_t n, void *D, int64_t ld, c
     if (launches) *launches += 1;
     return cudaGetLastError();
   }
-  tri_to_dense_kernel<Op><<<dim3(grid_cols(n, 256), grid_rows(n)), 256, 0, s>>>(static_cast<const E *>(T), L, n,
-                                                                              static_cast<E *>(D), ld);
-  const dim3 gm((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32));
-  mirror_kernel<Op><<<gm, dim3(32, 8), 0, s>>>(static_cast<E *>(D), n, ld, nullptr);
-  if (launches) *launches += 2;
-  return cudaGetLastError();
+  return output_pass<Op>(static_cast<const E *>(T), L, static_cast<E *>(D), ld, n, true, nullptr, s, launches);
 }
 
 cudaError_t launch_tri_to_dense(int dtype, const void *T, int64_t n, void *D, int64_t ld, cudaStream_t s,
@@ -2751,37 +2653,9 @@ cudaError_t launch_tri_rows(int dtype, const void *T, int64_t n, const int64_t *
   }
 }
 
-template <class Op>
-static cudaError_t ingest_impl(const void *W, void *D, int64_t n, int64_t ld, int *status, cudaStream_t s,
-                               int64_t *launches) {
-  using E = typename Op::elem;
-  dim3 g(grid_cols(n, 256), grid_rows(n));
-  ingest_kernel<Op><<<g, 256, 0, s>>>(static_cast<const E *>(W), static_cast<E *>(D), n, ld, W != D ? 1 : 0, status);
-  if (launches) *launches += 1;
-  return cudaGetLastError();
-}
-
 cudaError_t launch_ingest(int dtype, const void *W, void *D, int64_t n, int64_t ld, int *status, cudaStream_t s,
                           int64_t *launches) {
-  if (n <= 0) return cudaSuccess;
-  switch (dtype) {
-    case 0: return ingest_impl<OpI32>(W, D, n, ld, status, s, launches);
-    case 1: return ingest_impl<OpU16>(W, D, n, ld, status, s, launches);
-    case 2: return ingest_impl<OpF32>(W, D, n, ld, status, s, launches);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_copy(int dtype, const void *src, int64_t lds, void *dst, int64_t ldd, int64_t n, cudaStream_t s,
-                        int64_t *launches) {
-  if (n <= 0) return cudaSuccess;
-  const dim3 g(grid_cols(n, 256), grid_rows(n));
-  if (dtype == 1)
-    copy_kernel<<<g, 256, 0, s>>>(static_cast<const uint16_t *>(src), lds, static_cast<uint16_t *>(dst), ldd, n);
-  else
-    copy_kernel<<<g, 256, 0, s>>>(static_cast<const uint32_t *>(src), lds, static_cast<uint32_t *>(dst), ldd, n);
-  if (launches) *launches += 1;
-  return cudaGetLastError();
+  return launch_input(dtype, W, ld, D, ld, n, status, nullptr, s, launches);
 }
 
 cudaError_t launch_synth(int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s) {
@@ -2796,11 +2670,12 @@ cudaError_t launch_synth(int dtype, void *D, int64_t n, int64_t ld, cudaStream_t
   return cudaGetLastError();
 }
 
+static dim3 pack_grid(int64_t n) { return dim3((unsigned)((n + 2047) / 2048), grid_rows((n + 1) / 2)); }
+
 cudaError_t launch_pack(const int32_t *src, int64_t lds, uint16_t *dst, int64_t ldd, int64_t n, cudaStream_t s,
                         int64_t *launches) {
   if (n <= 0) return cudaSuccess;
-  dim3 g(grid_cols(n, 256), grid_rows(n));
-  pack_kernel<<<g, 256, 0, s>>>(src, lds, dst, ldd, n);
+  pack_kernel<<<pack_grid(n), 256, 0, s>>>(src, lds, aligned16(src, lds, 4), dst, ldd, aligned16(dst, ldd, 2), n);
   if (launches) *launches += 1;
   return cudaGetLastError();
 }
@@ -2808,8 +2683,7 @@ cudaError_t launch_pack(const int32_t *src, int64_t lds, uint16_t *dst, int64_t 
 cudaError_t launch_unpack(const uint16_t *src, int64_t lds, int32_t *dst, int64_t ldd, int64_t n, cudaStream_t s,
                           int64_t *launches) {
   if (n <= 0) return cudaSuccess;
-  dim3 g(grid_cols(n, 256), grid_rows(n));
-  unpack_kernel<<<g, 256, 0, s>>>(src, lds, dst, ldd, n);
+  unpack_kernel<<<pack_grid(n), 256, 0, s>>>(src, lds, aligned16(src, lds, 2), dst, ldd, aligned16(dst, ldd, 4), n);
   if (launches) *launches += 1;
   return cudaGetLastError();
 }
@@ -2818,8 +2692,8 @@ template <class Op>
 static cudaError_t densify_impl(const int32_t *src, const int32_t *dst, const void *w, int64_t m, void *D, int64_t n,
                                 int64_t ld, int *status, cudaStream_t s, int64_t *launches) {
   using E = typename Op::elem;
-  dim3 g(grid_cols(n, 256), grid_rows(n));
-  fill_inf_kernel<Op><<<g, 256, 0, s>>>(static_cast<E *>(D), n, ld);
+  fill_inf_kernel<Op><<<fill_grid<Op>(n, n), 256, 0, s>>>(static_cast<E *>(D), Layout(ld), n, n, n,
+                                                          aligned16(D, ld, sizeof(E)));
   if (m > 0) {
     int64_t blocks = (m + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;

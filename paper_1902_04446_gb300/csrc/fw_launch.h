@@ -48,6 +48,8 @@ struct RoundConfig {
   const int *sym_flag = nullptr;
   const int *gate = nullptr;  // kernel 4 only: round 0's Phase 1 also waits for *gate >= 1
   uint32_t dep_spins = 0;     // kernel 4 only: limit of each wait on another work item (0 = default)
+  void *out = nullptr;        // where the result goes (leading dimension out_ld) when not into D
+  int64_t out_ld = 0;
   int grid_cap = 0;           // persistent Phase-3 kernels: at most this many CTAs (0 = one per SM), so that
                               // solves on other streams can run on the remaining SMs
 };
@@ -169,9 +171,10 @@ cudaError_t launch_tri_rows(int dtype, const void *T, int64_t n, const int64_t *
 // Copies W to D when they differ and checks the input (status |= 1 invalid, 2 range).
 cudaError_t launch_ingest(int dtype, const void *W, void *D, int64_t n, int64_t ld, int *status, cudaStream_t s,
                           int64_t *launches);
-// dst <- src, n x n of the given element type, separate leading dimensions.
-cudaError_t launch_copy(int dtype, const void *src, int64_t lds, void *dst, int64_t ldd, int64_t n, cudaStream_t s,
-                        int64_t *launches);
+// The same with separate leading dimensions, and *asym |= 1 when W is not
+// symmetric (bitwise); status and asym nullable.
+cudaError_t launch_input(int dtype, const void *W, int64_t ldw, void *M, int64_t ldm, int64_t n, int *status, int *asym,
+                         cudaStream_t s, int64_t *launches);
 // Fills D with a synthetic symmetric graph (autotuner input).
 cudaError_t launch_synth(int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s);
 cudaError_t launch_pack(const int32_t *src, int64_t lds, uint16_t *dst, int64_t ldd, int64_t n, cudaStream_t s,
