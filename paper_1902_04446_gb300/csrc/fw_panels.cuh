@@ -101,16 +101,23 @@ __device__ __noinline__ void next_diag(const typename Op::elem *__restrict__ D, 
     // all loads first: the panels' 64 x 64 parts and this thread's part of the
     // block.  Rows and columns past the matrix read as INF.
     uint4 ta[4], tb[BIT];
+    const uint32_t *pa = colT + (int64_t)(tid / 16) * ldT + q0 + (tid % 16) * 4;  // panel rows are aligned words
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      ta[k] = load_chunk<OpI32, true>(reinterpret_cast<const int32_t *>(colT), ldT, 64, ldT, (tid + k * 256) / 16,
-                                      q0 + (tid % 16) * 4, true);
+    for (int k = 0; k < 4; ++k) ta[k] = ld16<true>(pa + (int64_t)k * 16 * ldT);
+    if ((symB || vec) && q0 + 64 <= n) {
+      // no branch between the loads: with one each they are a chain of latencies
+      const typename Op::elem *pb = (symB ? symB : D + L.off(p0, 0)) + q0 + (tid % (64 / E4)) * E4;
+      const int64_t row = symB ? ldT : L.ld;
 #pragma unroll
-    for (int k = 0; k < BIT; ++k) {
-      const int t = (tid + k * 256) / (64 / E4);
-      const int64_t x = q0 + (tid % (64 / E4)) * E4;
-      tb[k] = symB ? load_chunk<Op, true>(symB, ldT, 64, n, t, x, true)
-                   : load_chunk<Op, true>(D, L, n, n, p0 + t, x, vec != 0);
+      for (int k = 0; k < BIT; ++k) tb[k] = ld16<true>(pb + (int64_t)((tid + k * 256) / (64 / E4)) * row);
+    } else {
+#pragma unroll
+      for (int k = 0; k < BIT; ++k) {
+        const int t = (tid + k * 256) / (64 / E4);
+        const int64_t x = q0 + (tid % (64 / E4)) * E4;
+        tb[k] = symB ? load_chunk<Op, true>(symB, ldT, 64, n, t, x, true)
+                     : load_chunk<Op, true>(D, L, n, n, p0 + t, x, vec != 0);
+      }
     }
     load_block<Op, 64, true>(D, L, n, q0, v, tid);
 #pragma unroll
@@ -245,15 +252,19 @@ __device__ __forceinline__ void panel_chunk(typename Op::elem *__restrict__ D, L
   uint4 va[AIT], vs[SIT];
 #pragma unroll
   for (int k = 0; k < AIT; ++k) va[k] = __ldcg(reinterpret_cast<const uint4 *>(A) + tid + k * NT);
+  const bool whole = vec && x0 + XE <= n && p0 + 64 <= n;  // no branch between the loads then
 #pragma unroll
   for (int k = 0; k < SIT; ++k) {
     if (!col) {
       const int idx = tid + k * NT;
-      vs[k] = load_chunk<Op, true>(D, L, n, n, p0 + idx / (XW / 4), x0 + (idx % (XW / 4)) * E4, vec);
+      const int64_t r = p0 + idx / (XW / 4), c = x0 + (idx % (XW / 4)) * E4;
+      if (whole) vs[k] = ld16<true>(D + L.off(r, c));
+      else vs[k] = load_chunk<Op, true>(D, L, n, n, r, c, vec);
     } else {
       int x, t;
       col_piece(k, x, t);
-      vs[k] = load_chunk<Op, true>(D, L, n, n, x0 + x, p0 + t, vec);
+      if (whole) vs[k] = ld16<true>(D + L.off(x0 + x, p0 + t));
+      else vs[k] = load_chunk<Op, true>(D, L, n, n, x0 + x, p0 + t, vec);
     }
   }
 #pragma unroll

@@ -134,27 +134,47 @@ __device__ __forceinline__ void close_block(P1Smem<Op, BK> &sm, typename Op::sca
 }
 
 // Thread (by, bx)'s part of the BK x BK diagonal block at p0 (INF outside the
-// matrix): one 16-byte load per row where the addresses allow it.
+// matrix): one access per row, and no branch between them, for a block inside a
+// matrix with 16-byte rows.
 template <class Op, int BK, bool CG>
 __device__ __forceinline__ void load_block(const typename Op::elem *__restrict__ D, Layout L, int64_t n, int64_t p0,
                                            typename Op::scalar (&v)[BK / 16][BK / 16], int tid) {
+  using E = typename Op::elem;
   constexpr int PT = BK / 16;
   const int64_t r0 = p0 + (tid / 16) * PT, c0 = p0 + (tid % 16) * PT;
+  const E *base = D + L.off(p0, p0);
+  if constexpr (PT == 4) {
+    if (p0 + BK <= n && ((reinterpret_cast<uintptr_t>(base) | (uint64_t)L.ld * sizeof(E)) & 15) == 0) {
+      const E *q = base + (r0 - p0) * L.ld + (c0 - p0);
+      if constexpr (Op::EPW == 1) {
+        uint4 w[4];
 #pragma unroll
-  for (int r = 0; r < PT; ++r) {
-    const typename Op::elem *q = D + L.off(r0 + r, c0);
-    if (Op::EPW == 1 && PT == 4 && r0 + r < n && c0 + 4 <= n && (reinterpret_cast<uintptr_t>(q) & 15) == 0) {
-      const uint4 w = ld16<CG>(q);
-      v[r][0] = Op::to_s(bits_elem<Op>(w.x));
-      v[r][1] = Op::to_s(bits_elem<Op>(w.y));
-      v[r][PT - 2] = Op::to_s(bits_elem<Op>(w.z));
-      v[r][PT - 1] = Op::to_s(bits_elem<Op>(w.w));
-    } else {
+        for (int r = 0; r < 4; ++r) w[r] = ld16<CG>(q + r * L.ld);
 #pragma unroll
-      for (int c = 0; c < PT; ++c)
-        v[r][c] = Op::to_s((r0 + r < n && c0 + c < n) ? ld_elem<CG>(q + c) : Op::inf_elem());
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) v[r][c] = Op::to_s(bits_elem<Op>(chunk_get<Op>(w[r], c)));
+      } else {
+        uint2 w[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) w[r] = CG ? __ldcg(reinterpret_cast<const uint2 *>(q + r * L.ld))
+                                              : __ldg(reinterpret_cast<const uint2 *>(q + r * L.ld));
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          v[r][0] = Op::to_s((E)(w[r].x & 0xFFFFu));
+          v[r][1] = Op::to_s((E)(w[r].x >> 16));
+          v[r][2] = Op::to_s((E)(w[r].y & 0xFFFFu));
+          v[r][3] = Op::to_s((E)(w[r].y >> 16));
+        }
+      }
+      return;
     }
   }
+#pragma unroll
+  for (int r = 0; r < PT; ++r)
+#pragma unroll
+    for (int c = 0; c < PT; ++c)
+      v[r][c] = Op::to_s((r0 + r < n && c0 + c < n) ? ld_elem<CG>(D + L.off(r0 + r, c0 + c)) : Op::inf_elem());
 }
 
 // PT consecutive words from PT scalars (an aligned 8- or 16-byte store).
