@@ -523,6 +523,23 @@ __device__ __forceinline__ void load_acc(const typename Op::elem *M, Layout L, i
                                          int64_t row0, int64_t col0, bool vec, uint32_t (&acc)[8][TN], int ty,
                                          int tx) {
   using Map = TileMap<BM, BNW, TN>;
+  if (vec && row0 >= 0 && row0 + BM <= nrows && col0 + (int64_t)BNW * Op::EPW <= ncols) {
+    // a whole tile: no branch between the loads (with one each they are a chain
+    // of memory latencies)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const typename Op::elem *p = M + L.off(row0 + Map::row(ty, r), col0);
+#pragma unroll
+      for (int h = 0; h < Map::NH; ++h) {
+        const uint4 v = ld16<CG>(p + (int64_t)Map::wcol(tx, h) * Op::EPW);
+        acc[r][4 * h + 0] = v.x;
+        acc[r][4 * h + 1] = v.y;
+        acc[r][4 * h + 2] = v.z;
+        acc[r][4 * h + 3] = v.w;
+      }
+    }
+    return;
+  }
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
 #pragma unroll
@@ -577,7 +594,8 @@ __device__ __forceinline__ void store_acc(typename Op::elem *M, Layout L, int64_
 
 // The loaders below issue all of a thread's global loads before the first
 // shared-memory store (compile-time trip counts, fully unrolled in batches of
-// up to 8), so their latencies overlap instead of adding up.
+// up to 8, and for a part that lies inside the matrix no branch between them),
+// so their latencies overlap instead of adding up.
 
 // As[t][i] = colT[t][i0 + i] for t < BK, i < BM (colT rows are aligned words).
 template <int BM, int BK, int NT, bool CG = false>
@@ -610,14 +628,23 @@ __device__ __forceinline__ void load_Bs_rows(uint32_t *Bs, const typename Op::el
   constexpr int CH = BK * BNW / 4;
   static_assert(CH % NT == 0, "chunk count");
   constexpr int IT = CH / NT, BATCH = IT < 8 ? IT : 8;
+  const bool whole = vec && r0 >= 0 && r0 + BK <= nrows && c0 + (int64_t)BNW * Op::EPW <= ncols;
 #pragma unroll
   for (int k0 = 0; k0 < IT; k0 += BATCH) {
     uint4 v[BATCH];
+    if (whole) {
 #pragma unroll
-    for (int k = 0; k < BATCH; ++k) {
-      const int c = tid + (k0 + k) * NT;
-      v[k] = load_chunk<Op, CG>(M, L, nrows, ncols, r0 + c / (BNW / 4), c0 + (int64_t)((c % (BNW / 4)) * 4) * Op::EPW,
-                                vec);
+      for (int k = 0; k < BATCH; ++k) {
+        const int c = tid + (k0 + k) * NT;
+        v[k] = ld16<CG>(M + L.off(r0 + c / (BNW / 4), c0 + (int64_t)((c % (BNW / 4)) * 4) * Op::EPW));
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) {
+        const int c = tid + (k0 + k) * NT;
+        v[k] = load_chunk<Op, CG>(M, L, nrows, ncols, r0 + c / (BNW / 4),
+                                  c0 + (int64_t)((c % (BNW / 4)) * 4) * Op::EPW, vec);
+      }
     }
 #pragma unroll
     for (int k = 0; k < BATCH; ++k) {
@@ -638,13 +665,22 @@ __device__ __forceinline__ void load_As_transposed(uint32_t *As, const typename 
   constexpr int CH = BM * (BK / E);
   static_assert(CH % NT == 0, "chunk count");
   constexpr int IT = CH / NT, BATCH = IT < 8 ? IT : 8;
+  const bool whole = vec && i0 >= 0 && i0 + BM <= nrows && c0 + BK <= ncols;
 #pragma unroll
   for (int k0 = 0; k0 < IT; k0 += BATCH) {
     uint4 v[BATCH];
+    if (whole) {
 #pragma unroll
-    for (int k = 0; k < BATCH; ++k) {
-      const int c = tid + (k0 + k) * NT;
-      v[k] = load_chunk<Op, CG>(M, L, nrows, ncols, i0 + c % BM, c0 + (c / BM) * E, vec);
+      for (int k = 0; k < BATCH; ++k) {
+        const int c = tid + (k0 + k) * NT;
+        v[k] = ld16<CG>(M + L.off(i0 + c % BM, c0 + (c / BM) * E));
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) {
+        const int c = tid + (k0 + k) * NT;
+        v[k] = load_chunk<Op, CG>(M, L, nrows, ncols, i0 + c % BM, c0 + (c / BM) * E, vec);
+      }
     }
 #pragma unroll
     for (int k = 0; k < BATCH; ++k) {

@@ -389,7 +389,11 @@ __device__ __forceinline__ void p3_task(typename Op::elem *__restrict__ D, Layou
   load_acc<Op, BM, BNW, CG>(D, L, n, n, row0, col0, vec, acc, ty, tx);
   __syncthreads();
   tile_minplus<Op, BM, BNW, BK>(As, Bs, acc, ty, tx);
-  store_acc<Op, BM, BNW>(D, L, n, n, row0, col0, p0, p1, p0, p1, vec, acc, ty, tx);
+  if (vec && row0 + BM <= n && col0 + BNW * Op::EPW <= n && (row0 + BM <= p0 || row0 >= p1) &&
+      (col0 + BNW * Op::EPW <= p0 || col0 >= p1))
+    store_acc_interior<Op, BM, BNW>(D, L, row0, col0, acc, ty, tx);
+  else
+    store_acc<Op, BM, BNW>(D, L, n, n, row0, col0, p0, p1, p0, p1, vec, acc, ty, tx);
 }
 
 }  // namespace apsp
