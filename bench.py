@@ -50,7 +50,10 @@ import gen  # noqa: E402
 
 METRIC = "APSP GRelax/s (n³/s) int32 vs packed-int16; serving p50/p99 ms and solves/s"
 UNIT = "GRelax/s"
-ADDMIN_LANES_PER_CLK_PER_SM = 64  # add-min lane-ops per clock per SM: 64 INT32 lanes per SM, as apsp_addmin_peak measures
+ADDMIN_LANES_PER_CLK_PER_SM = 64  # ALU lane-ops per clock per SM: 64 lanes per SM, as apsp_addmin_peak measures
+# The integer tiles' loop takes 0.75 ALU instructions per 32-bit-word relaxation: half of its outputs take two
+# add-mins per two k-steps, half one three-input minimum of two sums formed on the FMA pipe.
+RELAX_PER_CLK_PER_SM = ADDMIN_LANES_PER_CLK_PER_SM / 0.75
 WORKLOAD_TEXT = {
     "gmm16k": "n=16384 symmetric k=10 kNN graph over a 10-D 8-component Gaussian mixture (seed 1), "
               "int32 weights max(1, rint(50 d)), dense INF-padded adjacency matrix",
@@ -133,7 +136,7 @@ class ClockSampler:
 def source_hash():
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1902_04446_gb300", "csrc")
-    for f in ("fw_kernels.cu", "fw_device.cuh", "fw_tasks.cuh", "tma.cuh", "fw_launch.h"):
+    for f in ("fw_kernels.cu", "fw_device.cuh", "fw_tasks.cuh", "fw_panels.cuh", "tma.cuh", "fw_launch.h"):
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -385,7 +388,7 @@ def serving_replay(torch, apsp, device, nreq, **cfg):
         torch.cuda.synchronize()
     sec = e0.elapsed_time(e1) / 1e3
     props = torch.cuda.get_device_properties(device)
-    peak = ADDMIN_LANES_PER_CLK_PER_SM * props.multi_processor_count * 2070e6
+    peak = RELAX_PER_CLK_PER_SM * props.multi_processor_count * 2070e6
     # relaxations the kernel performs: every round of every graph updates its whole tile grid (128 x 128 tiles,
     # round width 64, general mode)
     done = 0.0
@@ -546,7 +549,7 @@ def run_gpu(args):
         pass
     sm_max_mhz = float(peaks.get("sm_max_mhz", 2070.0))
     live = addmin_peaks(apsp, device)
-    peak = ADDMIN_LANES_PER_CLK_PER_SM * sms * sm_max_mhz * 1e6 / 1e9  # GRelax/s, int32 (u16x2: twice)
+    peak = RELAX_PER_CLK_PER_SM * sms * sm_max_mhz * 1e6 / 1e9  # GRelax/s, int32 (u16x2: twice)
 
     g = load_graph(args.workload)
     n = g.n
@@ -564,7 +567,7 @@ def run_gpu(args):
     # roofline of the dominant kernel (Phase 3), from the live event timings
     achieved = phase3_rate(prof)
     phase_ms = {f"phase{p}": round(prof[p][1] / args.steps, 3) for p in (1, 2, 3)}
-    if h.tuned_config("int32", n)[1] == 4:
+    if prof[3][0] <= max(1, args.steps):  # one Phase-3 launch per solve
         kname, kkey = ("fw_solve_ws<int32> (every round in one launch: Phase-3 tiles with each round's Phase 1 and "
                        "Phase 2 as tasks)"), "fw_solve_ws"
         work = ("relaxations performed in the launch: Phase 3 (in symmetric mode only the tiles touching the upper "
@@ -576,16 +579,16 @@ def run_gpu(args):
     roofline = {"bound": "alu", "kernel": kname,
                 "achieved": achieved, "peak": peak, "unit": UNIT, "work": work,
                 "frac": (achieved / peak) if achieved else None,
-                "peak_basis": f"{ADDMIN_LANES_PER_CLK_PER_SM} add-min lanes/clk/SM (the SM's INT32 lanes; measured "
-                              f"live: {live.get('int32', {}).get('relax_per_clk_per_sm', float('nan')):.1f}) x "
-                              f"{sms} SMs x {sm_max_mhz:.0f} MHz (max SM clock)",
+                "peak_basis": f"{RELAX_PER_CLK_PER_SM:.1f} relaxations/clk/SM ({ADDMIN_LANES_PER_CLK_PER_SM} ALU lanes at 0.75 "
+                              f"ALU instructions per relaxation; the add-min alone measured live: "
+                              f"{live.get('int32', {}).get('relax_per_clk_per_sm', float('nan')):.1f}) x {sms} SMs x {sm_max_mhz:.0f} MHz (max SM clock)",
                 "traffic": ncu_traffic(f"{kkey}_int32_{args.workload}"),
                 "traffic_unit": "DRAM bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
                 "phase_ms_per_step": phase_ms,
                 "phase3_launches_per_step": prof[3][0] // max(1, args.steps),
                 "phase3_share_of_step": prof[3][1] / ms if ms else None}
     if clocks and achieved:
-        roofline["frac_at_median_clock"] = achieved / (ADDMIN_LANES_PER_CLK_PER_SM * sms * clocks["sm_mhz"] / 1e3)
+        roofline["frac_at_median_clock"] = achieved / (RELAX_PER_CLK_PER_SM * sms * clocks["sm_mhz"] / 1e3)
 
     out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
            "ms_per_step": ms_max / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -715,8 +718,7 @@ def extras_gmm16k(torch, apsp, h, args, dist, device, peak, live, sms, sm_max_mh
     af = phase3_rate(proff)
     f_rpc = live.get("fp32", {}).get("relax_per_clk_per_sm")
     peak_f = f_rpc * sms * sm_max_mhz / 1e3 if f_rpc else None
-    kf = "fw_solve_ws<fp32> (every round in one launch)" if h.tuned_config("fp32", n)[1] == 4 else \
-        "fw_phase3_ws<fp32> (one launch per round)"
+    kf = "fw_phase3_ws<fp32> (one launch per round)"
     out["fp32"] = {"workload": "gmm16k_f32: the gmm16k points, raw Euclidean distances as fp32 weights",
                    "value": vf, "unit": UNIT, "ms_per_step": msf / args.steps, "gpu_launches": int(lf),
                    "roofline": {"bound": "alu", "kernel": kf, "achieved": af, "peak": peak_f, "unit": UNIT,
@@ -851,7 +853,7 @@ def run_round_shapes(args):
     names = {1: "one CTA per tile", 2: "TMA, 256 threads", 3: "TMA, 512 threads",
              4: "warp-specialized, one launch per round", 5: "warp-specialized, every round in one launch"}
     epw = 2 if args.dtype == "u16" else 1
-    peak = ADDMIN_LANES_PER_CLK_PER_SM * torch.cuda.get_device_properties(0).multi_processor_count * 2070.0 / 1e3
+    peak = RELAX_PER_CLK_PER_SM * torch.cuda.get_device_properties(0).multi_processor_count * 2070.0 / 1e3
     shapes = [(bk, v) for bk in (32, 64) for v in (1, 2, 3, 4, 5)] + [(128, 1), (128, 4)]
     if args.shapes:
         shapes = [tuple(int(x) for x in sv.split("x")) for sv in args.shapes.split(",")]

@@ -79,6 +79,8 @@ struct Profiler : apsp::PhaseTimer {
   std::vector<Pair> pairs;       // recorded, not yet read
   std::vector<cudaEvent_t> pool; // free events
   std::vector<int *> flags;      // free pinned flag slots
+  std::vector<int *> used;       // slots that recorded pairs refer to
+  int *cur = nullptr;            // the current solve's slot
   cudaEvent_t get() {
     if (!pool.empty()) {
       cudaEvent_t e = pool.back();
@@ -101,23 +103,25 @@ struct Profiler : apsp::PhaseTimer {
     pending = nullptr;
   }
   void after_choice(int phase, cudaStream_t s, double relax_sym, double relax_gen, const int *dflag) override {
-    int *f = nullptr;
-    if (!flags.empty()) {
-      f = flags.back();
-      flags.pop_back();
-    } else if (cudaHostAlloc(&f, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
-      f = nullptr;
-      cudaGetLastError();
-    }
-    if (f && cudaMemcpyAsync(f, dflag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) {
-      flags.push_back(f);
-      f = nullptr;
+    if (!cur) {  // one copy of the flag per solve, whatever its number of launches
+      if (!flags.empty()) {
+        cur = flags.back();
+        flags.pop_back();
+      } else if (cudaHostAlloc(&cur, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+        cur = nullptr;
+        cudaGetLastError();
+      }
+      if (cur) {
+        used.push_back(cur);
+        if (cudaMemcpyAsync(cur, dflag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess) *cur = 1;
+      }
     }
     cudaEvent_t b = get();  // after the flag copy: the pair's end event covers it
     cudaEventRecord(b, s);
-    pairs.push_back({pending, b, phase, relax_sym, relax_gen, f});
+    pairs.push_back({pending, b, phase, relax_sym, relax_gen, cur});
     pending = nullptr;
   }
+  void new_solve() override { cur = nullptr; }
   void read(int64_t *launches, double *ms, double *relax) {
     for (int p = 0; p < 3; ++p) {
       if (launches) launches[p] = 0;
@@ -131,20 +135,22 @@ struct Profiler : apsp::PhaseTimer {
       if (launches) launches[q.phase] += 1;
       if (ms) ms[q.phase] += t;
       if (relax) relax[q.phase] += (q.flag && *q.flag != 0) ? q.relax_alt : q.relax;
-      if (q.flag) flags.push_back(q.flag);
       pool.push_back(q.a);
       pool.push_back(q.b);
     }
     pairs.clear();
+    flags.insert(flags.end(), used.begin(), used.end());
+    used.clear();
+    cur = nullptr;
   }
   ~Profiler() {
     for (Pair &q : pairs) {
       cudaEventDestroy(q.a);
       cudaEventDestroy(q.b);
-      if (q.flag) cudaFreeHost(q.flag);
     }
     for (cudaEvent_t e : pool) cudaEventDestroy(e);
     for (int *f : flags) cudaFreeHost(f);
+    for (int *f : used) cudaFreeHost(f);
   }
 };
 
@@ -165,6 +171,8 @@ struct apsp_handle {
   size_t rowP_bytes = 0;
   void *mpT = nullptr;  // min-plus product: A^T (32-bit words)
   size_t mpT_bytes = 0;
+  void *mpBC = nullptr;  // min-plus product: copies of B and C with 16-byte rows
+  size_t mpBC_bytes = 0;
   int *d_status = nullptr;
   int *h_status = nullptr;  // pinned
   std::string last_error;
@@ -274,8 +282,8 @@ bool needs_aligned_copy(const void *D, int64_t ld, int64_t n, int dtype, const a
 }
 
 // The copy stays with the handle, so it is kept to an eighth of the device's memory.
-bool aligned_copy_fits(apsp_handle *h, size_t bytes) {
-  if (h->wsD && h->wsD_bytes >= bytes) return true;
+bool aligned_copy_fits(const void *have, size_t have_bytes, size_t bytes) {
+  if (have && have_bytes >= bytes) return true;
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
     cudaGetLastError();
@@ -304,7 +312,7 @@ void *round_matrix(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, co
   int64_t ldc = 0;
   if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc)) {
     const size_t bytes = (size_t)n * ldc * (dtype == APSP_U16 ? 2 : 4);
-    if (aligned_copy_fits(h, bytes)) {
+    if (aligned_copy_fits(h->wsD, h->wsD_bytes, bytes)) {
       if (ensure(&h->wsD, &h->wsD_bytes, bytes) == cudaSuccess) {
         *ldm = ldc;
         return h->wsD;
@@ -568,6 +576,7 @@ apsp_status apsp_destroy(apsp_handle *h) {
   if (h->wsD) cudaFree(h->wsD);
   if (h->rowP) cudaFree(h->rowP);
   if (h->mpT) cudaFree(h->mpT);
+  if (h->mpBC) cudaFree(h->mpBC);
   if (h->d_status) cudaFree(h->d_status);
   if (h->h_status) cudaFreeHost(h->h_status);
   delete h;
@@ -694,6 +703,13 @@ apsp_status apsp_int16_bound(apsp_handle *h, const int32_t *W, int64_t n, int64_
   return APSP_OK;
 }
 
+// Relaxations from which a product on B and C without 16-byte rows runs on copies
+// of them.  Measured, us without / with copies (m, k, n): int32 257, 260, 301
+// (2.0e7) 81 / 81, 401, 600, 501 137 / 114, 128, 1000, 131 199 / 157, 2000, 3000,
+// 3001 1355 / 1134; packed 16-bit 3000, 1000, 2001 354 / 303; fp32 3000, 1777,
+// 5001 2108 / 1532.
+constexpr double kCopyProduct = 1.6e7;
+
 // The product into C with the library's A^T workspace (the warp-specialized
 // kernel) when it can be had, else the one-CTA-per-tile kernel.  h->mu held.
 static cudaError_t minplus_locked(apsp_handle *h, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb,
@@ -704,9 +720,32 @@ static cudaError_t minplus_locked(apsp_handle *h, int dtype, const void *A, int6
     if (ensure(&h->mpT, &h->mpT_bytes, need) == cudaSuccess) scr = h->mpT;
     else cudaGetLastError();  // out of memory: the kernel without workspace
   }
+  // B and C without 16-byte rows: the TMA-fed kernel on copies of them, where
+  // the product is large enough to pay for the two copies in and the one out
+  const int64_t es = dtype == APSP_U16 ? 2 : 4;
+  auto rows16 = [es](const void *p, int64_t ld) {
+    return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld * es % 16 == 0;
+  };
   int64_t l = 0;
-  cudaError_t e = apsp::launch_minplus(dtype, A, lda, B, ldb, C, ldc, m, k, n, s, &l, scr, scr ? h->mpT_bytes : 0,
-                                       h->d_status);
+  cudaError_t e = cudaSuccess;
+  if (scr && k > 0 && !(rows16(B, ldb) && rows16(C, ldc)) && (double)m * n * k >= kCopyProduct) {
+    const int64_t ldn = round_up(n, 16 / es);
+    const size_t bytes = (size_t)(k + m) * ldn * es;
+    if (aligned_copy_fits(h->mpBC, h->mpBC_bytes, bytes)) {
+      if (ensure(&h->mpBC, &h->mpBC_bytes, bytes) == cudaSuccess) {
+        char *Bc = static_cast<char *>(h->mpBC), *Cc = Bc + (size_t)k * ldn * es;
+        e = apsp::launch_copy_rect(dtype, B, ldb, Bc, ldn, k, n, s, &l);
+        if (e == cudaSuccess) e = apsp::launch_copy_rect(dtype, C, ldc, Cc, ldn, m, n, s, &l);
+        if (e == cudaSuccess)
+          e = apsp::launch_minplus(dtype, A, lda, Bc, ldn, Cc, ldn, m, k, n, s, &l, scr, h->mpT_bytes, h->d_status);
+        if (e == cudaSuccess) e = apsp::launch_copy_rect(dtype, Cc, ldn, C, ldc, m, n, s, &l);
+        h->launches += l;
+        return e;
+      }
+      cudaGetLastError();  // out of memory: the kernel for any alignment
+    }
+  }
+  e = apsp::launch_minplus(dtype, A, lda, B, ldb, C, ldc, m, k, n, s, &l, scr, scr ? h->mpT_bytes : 0, h->d_status);
   h->launches += l;
   return e;
 }

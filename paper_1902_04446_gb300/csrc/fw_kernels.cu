@@ -2146,6 +2146,7 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
                                cudaStream_t s, int64_t *launches, PhaseTimer *tm, int *wait_err, bool sym,
                                void *rowPv, const int *sym_flag, const int *gate, uint32_t dep_spins,
                                int grid_cap, void *out, int64_t out_ld) {
+  if (tm) tm->new_solve();
   const bool use_tma = variant != 0;
   const int sms = grid_cap > 0 ? std::min(sm_count(), grid_cap) : sm_count();
   using Elem = typename Op::elem;
@@ -2656,6 +2657,21 @@ cudaError_t launch_tri_rows(int dtype, const void *T, int64_t n, const int64_t *
 cudaError_t launch_ingest(int dtype, const void *W, void *D, int64_t n, int64_t ld, int *status, cudaStream_t s,
                           int64_t *launches) {
   return launch_input(dtype, W, ld, D, ld, n, status, nullptr, s, launches);
+}
+
+cudaError_t launch_copy_rect(int dtype, const void *src, int64_t lds, void *dst, int64_t ldd, int64_t rows,
+                             int64_t cols, cudaStream_t s, int64_t *launches) {
+  if (rows <= 0 || cols <= 0) return cudaSuccess;
+  if (launches) *launches += 1;
+  if (dtype == 1)
+    copy_rect_kernel<OpU16><<<fill_grid<OpU16>(rows, cols), 256, 0, s>>>(
+        static_cast<const uint16_t *>(src), lds, aligned16(src, lds, 2), static_cast<uint16_t *>(dst), ldd,
+        aligned16(dst, ldd, 2), rows, cols);
+  else  // 32-bit elements of either type
+    copy_rect_kernel<OpI32><<<fill_grid<OpI32>(rows, cols), 256, 0, s>>>(
+        static_cast<const int32_t *>(src), lds, aligned16(src, lds, 4), static_cast<int32_t *>(dst), ldd,
+        aligned16(dst, ldd, 4), rows, cols);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_synth(int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s) {

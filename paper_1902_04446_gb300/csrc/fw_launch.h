@@ -17,6 +17,7 @@ struct PhaseTimer {
     (void)dflag;
     after(phase, s, relax_gen);
   }
+  virtual void new_solve() {}  // a solve's launches begin
   virtual ~PhaseTimer() {}
 };
 
@@ -175,6 +176,9 @@ cudaError_t launch_ingest(int dtype, const void *W, void *D, int64_t n, int64_t 
 // symmetric (bitwise); status and asym nullable.
 cudaError_t launch_input(int dtype, const void *W, int64_t ldw, void *M, int64_t ldm, int64_t n, int *status, int *asym,
                          cudaStream_t s, int64_t *launches);
+// dst <- src, rows x cols of the given element type.
+cudaError_t launch_copy_rect(int dtype, const void *src, int64_t lds, void *dst, int64_t ldd, int64_t rows,
+                             int64_t cols, cudaStream_t s, int64_t *launches);
 // Fills D with a synthetic symmetric graph (autotuner input).
 cudaError_t launch_synth(int dtype, void *D, int64_t n, int64_t ld, cudaStream_t s);
 cudaError_t launch_pack(const int32_t *src, int64_t lds, uint16_t *dst, int64_t ldd, int64_t n, cudaStream_t s,

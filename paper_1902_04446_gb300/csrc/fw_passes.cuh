@@ -163,6 +163,17 @@ __global__ void __launch_bounds__(256) output_pairs_kernel(const typename Op::el
   }
 }
 
+// dst <- src, rows x cols, 16 bytes a thread and row.
+template <class Op>
+__global__ void __launch_bounds__(256) copy_rect_kernel(const typename Op::elem *__restrict__ s, int64_t lds, int vs,
+                                                        typename Op::elem *__restrict__ d, int64_t ldd, int vd,
+                                                        int64_t rows, int64_t cols) {
+  const int64_t j = ((int64_t)blockIdx.x * 256 + threadIdx.x) * (4 * Op::EPW);
+  if (j >= cols) return;
+  for (int64_t i = blockIdx.y; i < rows; i += gridDim.y)
+    store_chunk<Op>(d, ldd, i, j, load_chunk<Op>(s, lds, rows, cols, i, j, vs != 0), row_mask<Op>(j, cols), vd != 0);
+}
+
 // int32 -> packed 16-bit (saturated to INF16) and back, 8 elements a thread.
 static __global__ void __launch_bounds__(256) pack_kernel(const int32_t *__restrict__ s, int64_t lds, int vs,
                                                    uint16_t *__restrict__ d, int64_t ldd, int vd, int64_t n) {

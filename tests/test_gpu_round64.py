@@ -118,3 +118,23 @@ def test_input_pass_checks_every_block(lib, n):
         V[n - 1, n - 1] = 2
         h.solve_t("int32", torch.from_numpy(V).cuda())
         assert h.last_status() == 1
+
+
+@pytest.mark.parametrize("dtype", ["int32", "u16", "fp32"])
+@pytest.mark.parametrize("m,k,n", [(257, 260, 301), (301, 203, 333), (128, 1000, 129)])
+def test_minplus_unaligned_rows(lib, dtype, m, k, n):
+    """Products whose B and C have no 16-byte rows, above the size from which they run on copies."""
+    rng = np.random.default_rng(m * n)
+    inf = 0x7FFF if dtype == "u16" else INF
+    mats = []
+    for shape in ((m, k), (k, n), (m, n)):
+        x = rng.integers(0, 2000, size=shape)
+        x[rng.random(shape) < 0.2] = inf
+        mats.append(x)
+    E = oracle.minplus(*mats)
+    A, B, C = (torch.from_numpy(np.where(x >= inf, np.inf, x) if dtype == "fp32" else x).to(TD[dtype]).cuda()
+               for x in mats)
+    with lib.Handle(device=0) as h:
+        h.minplus(A, B, C)
+    got = C.cpu().numpy().astype(np.float64)
+    np.testing.assert_array_equal(np.where(got >= inf, inf, got).astype(np.int64), np.minimum(E, inf))
