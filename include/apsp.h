@@ -397,9 +397,11 @@ apsp_status apsp_noalloc_status(void *stream);
 /* ---- the add-min step itself (measurement support) ----------------------- */
 /* The relaxation c = min(c, a + b) is the min-plus step of Table 1 (MatProd
  * followed by MatMin); Phase 3 is bound by how many of them the SMs issue per
- * clock.  apsp_addmin_peak measures that rate on `device` for the add-min form
- * the library's Phase-3 tiles use for `dtype` (APSP_I32: __viaddmin_s32;
- * APSP_U16: __viaddmin_u16x2, two relaxations per 32-bit lane-op; APSP_F32:
+ * clock.  apsp_addmin_peak measures that rate on `device` for the add-min
+ * instruction of `dtype` (APSP_I32: __viaddmin_s32; APSP_U16:
+ * __viaddmin_u16x2, two relaxations per 32-bit lane-op -- the integer tiles
+ * take it for half of their outputs and form the other half's sums on the FMA
+ * pipe, so they may exceed this rate; APSP_F32, the tiles' own form:
  * two k-steps at a time, a packed pair add for two neighbouring columns and
  * one three-input minimum for each output's two sums): independent chains in
  * registers, one full wave of 4 CTAs x 256 threads per SM.

@@ -12,6 +12,9 @@
 //            contiguous rows.
 //   Phase 3  fw_phase3: D_IJ = min(D_IJ, D_Ik (x) D_kJ) for every block outside
 //            row k and column k (Table 1 MatProd + MatMin, Alg. 4 "offcol").
+// Those are the kernels of round widths 32 and 128; at width 64 a round is two
+// launches, fw_panels and a Phase 3 that also closes the next round's diagonal
+// block (fw_panels.cuh).
 // The product with a closed D_kk equals the in-place sweep over t of the
 // original algorithm: the shortest path from i in block k to j that uses
 // intermediate vertices of block k ends with one step from its last block-k
@@ -2306,6 +2309,7 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
   };
   // Widths 32 and 128: Phase 1 and Phase 2 of round k as their own launches.
   auto panels = [&](int64_t k, uint32_t *cT, Elem *rP) {
+    if constexpr (BK != 64) {
     int64_t p0, p1;
     span(k, p0, p1);
     const double w = (double)(p1 - p0), rest = (double)(n - (p1 - p0));
@@ -2344,6 +2348,7 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
       }
     }
     if (tm) tm->after(1, s, sym ? rest * w * w : 2.0 * rest * w * w);
+    }
   };
   // relaxations of round k's Phase 3 actually performed: the processed tiles' share of (n - w)^2 w
   auto p3_work = [&](int64_t k) {
