@@ -94,7 +94,8 @@ typedef struct {
                             only the upper triangle): Phase 3 updates only the tiles touching the upper
                             triangle and the lower triangle is mirrored at the end -- same result, about
                             half the relaxations.  0 = use it when a device check finds W symmetric
-                            (one stream synchronization per solve), 1 = the caller guarantees W is
+                            (the kernels read its answer on the device; round widths other than 64 and
+                            the other Phase-3 kernels synchronize the stream once per solve), 1 = the caller guarantees W is
                             symmetric, 2 = never.  Edge-list solves are symmetric by construction. */
   int64_t serving_large_n; /* serving: a request with n >= this runs alone in its own group on the per-round
                               kernels; smaller ones share the batched persistent kernel (0 = default 1536),
@@ -123,6 +124,9 @@ apsp_status apsp_destroy(apsp_handle *h);
  * dtype.  W and D are device pointers with the same leading dimension ld;
  * W == D (in place) is allowed.  Asynchronous on `stream`, except that
  * APSP_AUTO synchronizes the stream once to read the 16-bit bound.
+ * Matrices without 16-byte rows (base or ld * element size not a multiple of 16)
+ * are solved in a copy that the handle keeps, up to an eighth of the device's
+ * memory; larger ones, or when it cannot be had, by a slower kernel in place.
  * Input checks that need the data (negative weight, non-zero diagonal,
  * finite weight >= INF) run on the device; read their result with
  * apsp_last_status().  Errors returned directly: APSP_E_INVALID (null pointer,
@@ -166,7 +170,9 @@ apsp_status apsp_int16_bound(apsp_handle *h, const int32_t *W, int64_t n, int64_
  * `stream`: the rounds of every graph (Alg. 3/4 phases) are cut into tasks
  * that resident CTAs pull from a device work queue in dependency order, so
  * rounds of different graphs overlap on the device.  W[i], D[i] are device
- * matrices (n[i] rows of ld[i] elements, W[i] == D[i] allowed).  Asynchronous;
+ * matrices (n[i] rows of ld[i] elements, W[i] == D[i] allowed).  A symmetric
+ * graph updates only its upper tiles; one without 16-byte rows is solved in a
+ * copy in the handle's workspace.  Asynchronous;
  * apsp_last_status() reports the input checks of all graphs and
  * APSP_E_TIMEOUT if a bounded device wait gave up.  Errors: APSP_E_INVALID,
  * APSP_E_NOMEM (workspace), APSP_E_CUDA. */
@@ -186,11 +192,12 @@ apsp_status apsp_check_bounded_wait(apsp_handle *h, int64_t spin_limit);
 /* ---- building blocks (Table 1) ------------------------------------------ */
 /* C = min(C, A (x) B): the min-plus product ("MatProd") followed by the
  * element-wise minimum ("MatMin").  A is m x k (lda), B is k x n (ldb), C is
- * m x n (ldc), all device, row-major, of the given dtype (APSP_I32, APSP_U16 or
- * APSP_F32).  C must not overlap A or B.  Uses a handle-owned workspace of
+ * m x n (ldc), all device, row-major, of the given dtype (APSP_I32, APSP_U16 with
+ * values <= APSP_INF_U16, or APSP_F32).  C must not overlap A or B.  Uses a handle-owned workspace of
  * about 4*m*k bytes (A transposed) for the TMA-fed kernel when it can be
- * allocated and B and C are 16-byte addressable; otherwise a kernel without
- * workspace.  Asynchronous on `stream`; a device wait that gave up is reported
+ * allocated and B and C are 16-byte addressable or can be copied (products of
+ * 1.6e7 relaxations and more; the copies stay with the handle, up to an eighth of
+ * the device's memory); otherwise a kernel without workspace.  Asynchronous on `stream`; a device wait that gave up is reported
  * by apsp_last_status (bit 4).  Errors: APSP_E_INVALID, APSP_E_CUDA. */
 apsp_status apsp_minplus(apsp_handle *h, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb,
                          void *C, int64_t ldc, int64_t m, int64_t k, int64_t n, void *stream);
@@ -435,7 +442,9 @@ int64_t apsp_launch_count(apsp_handle *h);
  * the recorded events and writes, for phases 0, 1, 2 (= Phase 1, 2, 3), the
  * number of timed launches, their summed device time in ms, and their summed
  * algorithmic relaxation counts (Phase 1: w^3, Phase 2: 2 (n-w) w^2, Phase 3:
- * (n-w)^2 w for a round of width w); then it clears the record.  Any of the
+ * (n-w)^2 w for a round of width w; with 64-wide rounds and the
+ * warp-specialized kernel only round 0 has a Phase-1 launch, the later diagonal
+ * blocks are closed inside Phase 3); then it clears the record.  Any of the
  * output arrays may be NULL. */
 apsp_status apsp_profile(apsp_handle *h, int enable);
 apsp_status apsp_profile_read(apsp_handle *h, int64_t launches[3], double ms[3], double relaxations[3]);

@@ -1,6 +1,7 @@
 // Phase bodies of one round of blocked Floyd-Warshall (the paper's Sec. 4.4/4.5,
-// Alg. 3 and 4), as device functions shared by the per-round kernels
-// (fw_kernels.cu) and the batched persistent kernel (batch.cu).
+// Alg. 3 and 4), as device functions shared by the per-round kernels and the
+// single launch (fw_kernels.cu), the 64-wide rounds (fw_panels.cuh) and the
+// batched persistent kernel (batch.cu).
 //
 // Round k covers vertices [p0, p1) = [k*BK, min(n, (k+1)*BK)); w = p1 - p0.
 //   phase1_body   Floyd-Warshall closure of D_kk (Table 1 FloydWarshall); also
