@@ -32,26 +32,30 @@ __global__ void init_keys(unsigned long long *key, int64_t n) {
 }
 
 // `inner` sweeps over the edges, each thread over its own without waiting for
-// the others: keys only fall, and a launch in which no thread lowered any key
-// has checked every edge against the final keys, so any order gives the same
-// result.  A sweep of its own launch costs 5 us at 120 thousand edges, most of
-// it launch latency; inside a launch it is one round trip to L2.
+// the others.  Keys only fall, so any order reaches the same fixed point, and a
+// launch in which no thread lowered any key has checked every edge against the
+// final keys.  What a launch is sure to settle is one hop, as one sweep does:
+// the threads may run one after another, each sweep before the next thread's
+// first.  Usually they run together and settle about a hop a sweep.  A sweep of
+// its own launch costs 5 us at 120 thousand edges, most of it launch latency;
+// inside a launch it is one round trip to L2.
 template <typename WT>
 __global__ void bf_sweep(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, const WT *__restrict__ w,
                          int64_t m, int64_t n, uint64_t inf, unsigned long long *key, int *changed, int inner) {
   int ch = 0;
-  for (int it = 0; it < inner; ++it)
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t u = src[e], v = dst[e];
-    const WT wt = w[e];
-    if (u < 0 || u >= n || v < 0 || v >= n || u == v) continue;
-    if ((int64_t)wt < 0 || (uint64_t)wt >= inf) continue;
-    const unsigned long long ku = *((volatile unsigned long long *)&key[u]);
-    const unsigned long long kv = *((volatile unsigned long long *)&key[v]);
-    const unsigned long long cu = relax_key(ku, (unsigned long long)wt);
-    if (cu < kv) { atomicMin(&key[v], cu); ch = 1; }
-    const unsigned long long cv = relax_key(kv, (unsigned long long)wt);
-    if (cv < ku) { atomicMin(&key[u], cv); ch = 1; }
+  for (int it = 0; it < inner; ++it) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+      const int64_t u = src[e], v = dst[e];
+      const WT wt = w[e];
+      if (u < 0 || u >= n || v < 0 || v >= n || u == v) continue;
+      if ((int64_t)wt < 0 || (uint64_t)wt >= inf) continue;
+      const unsigned long long ku = *((volatile unsigned long long *)&key[u]);
+      const unsigned long long kv = *((volatile unsigned long long *)&key[v]);
+      const unsigned long long cu = relax_key(ku, (unsigned long long)wt);
+      if (cu < kv) { atomicMin(&key[v], cu); ch = 1; }
+      const unsigned long long cv = relax_key(kv, (unsigned long long)wt);
+      if (cv < ku) { atomicMin(&key[u], cv); ch = 1; }
+    }
   }
   if (ch) *changed = 1;
 }
@@ -184,21 +188,23 @@ cudaError_t run_bf(const int32_t *src, const int32_t *dst, const WT *w, int64_t 
   if (e != cudaSuccess) return e;
   unsigned long long *key = static_cast<unsigned long long *>(keyb.p);
   unsigned long long *mx = static_cast<unsigned long long *>(aux.p);
-  int *changed = reinterpret_cast<int *>(static_cast<char *>(aux.p) + 64);  // one flag per sweep of a group
+  int *changed = reinterpret_cast<int *>(static_cast<char *>(aux.p) + 64);  // one flag per launch of a group
   const unsigned gb = (unsigned)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
   init_keys<<<gb, 256, 0, s>>>(key, n);
   *launches += 1;
   const int64_t eb = (m + 255) / 256;
   const unsigned ge = (unsigned)(eb < 1 ? 1 : (eb > 152 * 8 ? 152 * 8 : eb));
-  // At most n + 1 sweeps are needed (each sweep fixes one more hop of every
-  // shortest-path tree); a sweep that changes nothing means the keys are final.
-  // Launches of kInner sweeps run in groups between host checks, each launch with
-  // its own flag; the groups double (2, 4, ..., 16) so that deep graphs need few
-  // round trips while shallow ones stop after a few sweeps.
+  // Each launch settles one more hop of every shortest-path tree (at most n - 1),
+  // and a launch that changes nothing means the keys are final, so n launches
+  // are always enough; counted by their kInner sweeps they were not (a path of
+  // 2030 vertices needs 255 launches even at a hop a sweep).  Launches run in
+  // groups between host checks, each launch with its own flag; the groups double
+  // (2, 4, ..., 16) so that deep graphs need few round trips while shallow ones
+  // stop after a few sweeps.
   bool converged = false;
   int h_flags[kMaxGroup];
-  for (int64_t done = 0, group = 2; !converged && done <= n + 1;
-       done += kInner * group, group = std::min<int64_t>(2 * group, kMaxGroup)) {
+  for (int64_t done = 0, group = 2; !converged && done <= n;
+       done += group, group = std::min<int64_t>(2 * group, kMaxGroup)) {
     e = cudaMemsetAsync(changed, 0, (size_t)group * sizeof(int), s);
     if (e != cudaSuccess) return e;
     for (int r = 0; r < group; ++r) bf_sweep<WT><<<ge, 256, 0, s>>>(src, dst, w, m, n, inf, key, changed + r, kInner);
