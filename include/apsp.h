@@ -192,8 +192,10 @@ apsp_status apsp_check_bounded_wait(apsp_handle *h, int64_t spin_limit);
 /* ---- building blocks (Table 1) ------------------------------------------ */
 /* C = min(C, A (x) B): the min-plus product ("MatProd") followed by the
  * element-wise minimum ("MatMin").  A is m x k (lda), B is k x n (ldb), C is
- * m x n (ldc), all device, row-major, of the given dtype (APSP_I32, APSP_U16 with
- * values <= APSP_INF_U16, or APSP_F32).  C must not overlap A or B.  Uses a handle-owned workspace of
+ * m x n (ldc), all device, row-major, of the given dtype (APSP_I32, APSP_U16 or
+ * APSP_F32).  A packed 16-bit sum above 0xFFFF wraps in its own element; products
+ * of 1e9 relaxations and more look at A and B first and run faster when no
+ * element is above APSP_INF_U16.  C must not overlap A or B.  Uses a handle-owned workspace of
  * about 4*m*k bytes (A transposed) for the TMA-fed kernel when it can be
  * allocated and B and C are 16-byte addressable or can be copied (products of
  * 1.6e7 relaxations and more; the copies stay with the handle, up to an eighth of

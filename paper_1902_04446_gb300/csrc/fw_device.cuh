@@ -312,9 +312,9 @@ template <bool PREFETCH_, int UNROLL_, bool COLS_, int MIX_>
 struct KLoop {
   static constexpr bool PREFETCH = PREFETCH_, COLS = COLS_;
   static constexpr int UNROLL = UNROLL_, MIX = MIX_;
-  static_assert(MIX >= 0 && MIX <= 3, "mix pattern");
+  static_assert(MIX >= 0 && MIX <= 4, "mix pattern");
   __host__ __device__ static constexpr bool fma_form(int r, int c) {
-    return (MIX == 0 ? (r + c) & 1 : MIX == 1 ? (c >> 1) & 1 : MIX == 2 ? r & 1 : c & 1) != 0;
+    return (MIX == 0 ? (r + c) & 1 : MIX == 1 ? (c >> 1) & 1 : MIX == 2 ? r & 1 : MIX == 3 ? c & 1 : 0) != 0;
   }
 };
 // Kernels with at most 128 registers a thread (Phase 2, one CTA per tile, batched).
@@ -475,8 +475,11 @@ struct RegsU32 {
 // issue port two cycles.  Measured with operands in shared memory and no
 // epilogue (relaxations per clock per SM, 32-bit words): no output in the FMA
 // form 63.2, a quarter 67, half 70 - 73, three quarters 65, all 53.
-// Packed 16-bit words add as plain 32-bit integers: every stored value is
-// <= 0x7FFF, so the low lane's sum never carries into the high lane.
+// In the FMA form packed 16-bit words add as plain 32-bit integers: right where
+// every value is <= 0x7FFF, as a solve's input check sees to, since the low
+// lane's sum then never carries into the high lane.  The min-plus product takes
+// values unchecked, so its packed loops keep to the add-min (MIX 4), whose lanes
+// wrap apart.
 template <class Op, int BM, int BNW, int BK, int TN = 8, class KL = KLoopSmall>
 __device__ __forceinline__ void tile_minplus(const uint32_t *__restrict__ As, const uint32_t *__restrict__ Bs,
                                              uint32_t (&acc)[8][TN], int ty, int tx, int ksteps = BK) {

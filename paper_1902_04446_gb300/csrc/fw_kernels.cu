@@ -521,18 +521,24 @@ struct P3Loop {
   using Round = typename std::conditional<BK == 128, KLoop<true, 1, true, 1>, KLoop<false, 1, false, 1>>::type;
   using Solve = KLoop<true, 2, true, 0>;
   using Product = KLoop<true, 2, true, 0>;
+  using AnyProduct = Product;       // a product whose operands may hold any value
+  using PlainProduct = KLoopSmall;  // minplus_kernel
 };
 template <int BK>
 struct P3Loop<OpU16, BK> {
   using Round = KLoop<true, 1, false, 2>;
   using Solve = KLoop<false, 1, false, 1>;
-  using Product = KLoop<false, 1, false, 3>;
+  using Product = KLoop<false, 1, false, 3>;     // operands <= 0x7FFF
+  using AnyProduct = KLoop<false, 8, false, 4>;  // no FMA form (see tile_minplus)
+  using PlainProduct = AnyProduct;
 };
 template <int BK>
 struct P3Loop<OpF32, BK> {
   using Round = KLoop<true, 1, true, 0>;
   using Solve = KLoop<false, 2, true, 0>;
   using Product = KLoop<false, 4, true, 1>;
+  using AnyProduct = Product;
+  using PlainProduct = KLoopSmall;
 };
 
 // What a Phase-3 launch is told besides its tiles.
@@ -1688,7 +1694,7 @@ __global__ void __launch_bounds__(256, 2) minplus_kernel(const typename Op::elem
     load_As_transposed<Op, Cfg::BM, BK, Cfg::THREADS>(As, A, lda, m, k, row0, t0, veca, tid);
     load_Bs_rows<Op, Cfg::BNW, BK, Cfg::THREADS>(Bs, B, ldb, k, nn, t0, col0, vecb, tid);
     __syncthreads();
-    tile_minplus<Op, Cfg::BM, Cfg::BNW, BK>(As, Bs, acc, ty, tx);
+    tile_minplus<Op, Cfg::BM, Cfg::BNW, BK, 8, typename P3Loop<Op, BK>::PlainProduct>(As, Bs, acc, ty, tx);
     __syncthreads();
   }
   store_acc<Op, Cfg::BM, Cfg::BNW>(Cm, ldc, m, nn, row0, col0, 0, 0, 0, 0, vecc, acc, ty, tx);
@@ -1715,6 +1721,33 @@ __global__ void transpose_dup_kernel(const typename Op::elem *__restrict__ A, in
   }
 }
 
+// *wide |= 1 when an element of the packed 16-bit A (m x k) or B (k x nn) is
+// above 0x7FFF; blockIdx.z picks the matrix, 16 bytes a thread and row.
+static __global__ void __launch_bounds__(256) wide_operand_kernel(const uint16_t *__restrict__ A, int64_t lda, int veca,
+                                                                  const uint16_t *__restrict__ B, int64_t ldb, int vecb,
+                                                                  int64_t m, int64_t k, int64_t nn, int *wide) {
+  const bool second = blockIdx.z != 0;
+  const uint16_t *M = second ? B : A;
+  const int64_t ld = second ? ldb : lda, rows = second ? k : m, cols = second ? nn : k;
+  const bool vec = (second ? vecb : veca) != 0;
+  const int64_t j = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 8;
+  uint32_t any = 0;
+  if (j < cols)
+    for (int64_t i = blockIdx.y; i < rows; i += gridDim.y) {
+      const uint4 v = load_chunk<OpU16>(M, ld, rows, cols, i, j, vec);  // INF past the matrix
+      any |= v.x | v.y | v.z | v.w;
+    }
+  if (__syncthreads_or((any & 0x80008000u) != 0) && threadIdx.x == 0) atomicOr(wide, 1);
+}
+
+// Relaxations from which a packed 16-bit product looks at its operands first and
+// takes the mixed loop when they are all <= 0x7FFF, the add-min loop otherwise.
+// Both kernels are launched and one of them returns at once, so nothing waits
+// for the answer on the host.  The look, the flag's reset and the empty launch
+// cost about 10 us: n = m = k = 1024 144 us by the add-min loop alone, 140 with
+// them, 4096 2183 / 1946 us.
+constexpr double kWideCheck = 1e9;
+
 // C = min(C, A (x) B) for general shapes, warp-specialized like fw_phase3_ws:
 // 8 consumer warps own 8 x 8 words of a 128 x 128-word output tile and walk
 // its k in chunks of 64 (one work slot per chunk; the accumulators start at INF
@@ -1722,12 +1755,13 @@ __global__ void transpose_dup_kernel(const typename Op::elem *__restrict__ A, in
 // applies the tile after its last chunk: TMA min-reduction for int32 (the map
 // ends at ncols rounded down to 4 elements, the tail merged by its owners),
 // merge with a TMA-loaded C and TMA store (interior) or masked stores (edge)
-// otherwise.  Static contiguous tile ranges per CTA; bounded waits.
-template <class Op, bool RED>
+// otherwise.  Static contiguous tile ranges per CTA; bounded waits.  gate
+// (nullable): the launch does nothing unless *gate == run_if.
+template <class Op, bool RED, class KL>
 __global__ void __launch_bounds__(P3W_THREADS, 1)
     fw_minplus_ws(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                   const __grid_constant__ CUtensorMap mapC, typename Op::elem *__restrict__ C, int64_t ldc, int64_t m,
-                  int64_t ncols, int nk, int tiles_x, int tiles_total, int *err) {
+                  int64_t ncols, int nk, int tiles_x, int tiles_total, int *err, const int *gate, int run_if) {
   constexpr int BK = 64, BM = 128, BNW = 128, TN = 8;
   using Map = TileMap<BM, BNW, TN>;
   constexpr int NCW = Map::THREADS / 32;
@@ -1743,7 +1777,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   const int per = tiles_total / (int)gridDim.x, extra = tiles_total % (int)gridDim.x;
   const int t_begin = (int)blockIdx.x * per + min((int)blockIdx.x, extra);
   const int t_end = t_begin + per + ((int)blockIdx.x < extra ? 1 : 0);
-  if (t_begin >= t_end) return;
+  if (t_begin >= t_end || (gate && *gate != run_if)) return;
   const long long n_slots = (long long)(t_end - t_begin) * nk;
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -1839,7 +1873,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
         if (lane == 0) abort_flag = 1;
         break;
       }
-      tile_minplus<Op, BM, BNW, BK, TN, typename P3Loop<Op, BK>::Product>(stA(s), stB(s), acc, ty, tx);
+      tile_minplus<Op, BM, BNW, BK, TN, KL>(stA(s), stB(s), acc, ty, tx);
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty_ab[s]);
       if (c != nk - 1) continue;
@@ -2782,23 +2816,39 @@ static cudaError_t minplus_ws_impl(const void *A, int64_t lda, const void *B, in
       !make_map(&mB, dt, B, (uint64_t)nn, (uint64_t)k, (uint64_t)ldb * es, 128 * Op::EPW, 64) ||
       !make_map(&mC, dt, Cm, cx, (uint64_t)m, (uint64_t)ldc * es, 128 * Op::EPW, 128))
     return cudaErrorNotSupported;
-  cudaError_t e = cudaFuncSetAttribute(fw_minplus_ws<Op, RED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       P3T<64>::SMEM);
-  if (e != cudaSuccess) return e;
-  const dim3 gt((unsigned)(ldat / 32), (unsigned)(k_pad / 32));
-  transpose_dup_kernel<Op><<<gt, dim3(32, 8), 0, s>>>(static_cast<const E *>(A), lda, m, k, AT, ldat, k_pad);
   const int tiles_x = (int)((nn + 128 * Op::EPW - 1) / (128 * Op::EPW));
   const int tiles_total = tiles_x * (int)((m + 127) / 128);
   const int grid = std::min(sm_count(), tiles_total);
-  fw_minplus_ws<Op, RED><<<grid, P3W_THREADS, P3T<64>::SMEM, s>>>(mA, mB, mC, static_cast<E *>(Cm), ldc, m, nn,
-                                                                   (int)(k_pad / 64), tiles_x, tiles_total, err);
-  if (launches) *launches += 2;
-  return cudaGetLastError();
+  auto go = [&](auto kernel, const int *gate, int run_if) {
+    const cudaError_t ea = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P3T<64>::SMEM);
+    if (ea != cudaSuccess) return ea;
+    kernel<<<grid, P3W_THREADS, P3T<64>::SMEM, s>>>(mA, mB, mC, static_cast<E *>(Cm), ldc, m, nn, (int)(k_pad / 64),
+                                                    tiles_x, tiles_total, err, gate, run_if);
+    if (launches) *launches += 1;
+    return cudaGetLastError();
+  };
+  const dim3 gt((unsigned)(ldat / 32), (unsigned)(k_pad / 32));
+  transpose_dup_kernel<Op><<<gt, dim3(32, 8), 0, s>>>(static_cast<const E *>(A), lda, m, k, AT, ldat, k_pad);
+  if (launches) *launches += 1;
+  if constexpr (Op::DTYPE == 1) {
+    if ((double)m * (double)k * (double)nn >= kWideCheck) {
+      int *wide = reinterpret_cast<int *>(AT + k_pad * ldat);
+      cudaError_t e = cudaMemsetAsync(wide, 0, sizeof(int), s);
+      if (e != cudaSuccess) return e;
+      const dim3 gw((unsigned)((std::max(k, nn) + 2047) / 2048), grid_rows((std::max(m, k) + 7) / 8), 2);
+      wide_operand_kernel<<<gw, 256, 0, s>>>(static_cast<const E *>(A), lda, aligned16(A, lda, es),
+                                             static_cast<const E *>(B), ldb, aligned16(B, ldb, es), m, k, nn, wide);
+      if (launches) *launches += 1;
+      e = go(fw_minplus_ws<Op, RED, typename P3Loop<Op, 64>::Product>, wide, 0);
+      return e != cudaSuccess ? e : go(fw_minplus_ws<Op, RED, typename P3Loop<Op, 64>::AnyProduct>, wide, 1);
+    }
+  }
+  return go(fw_minplus_ws<Op, RED, typename P3Loop<Op, 64>::AnyProduct>, nullptr, 0);
 }
 
 size_t minplus_scratch_bytes(int64_t m, int64_t k) {
   if (m <= 0 || k <= 0) return 0;
-  return (size_t)((k + 63) / 64 * 64) * (size_t)((m + 255) / 256 * 256) * 4;
+  return (size_t)((k + 63) / 64 * 64) * (size_t)((m + 255) / 256 * 256) * 4 + 256;  // A^T, then the wide-operand flag
 }
 
 cudaError_t launch_minplus(int dtype, const void *A, int64_t lda, const void *B, int64_t ldb, void *Cm, int64_t ldc,
