@@ -126,7 +126,8 @@ apsp_status apsp_destroy(apsp_handle *h);
  * APSP_AUTO synchronizes the stream once to read the 16-bit bound.
  * Matrices without 16-byte rows (base or ld * element size not a multiple of 16)
  * are solved in a copy that the handle keeps, up to an eighth of the device's
- * memory; larger ones, or when it cannot be had, by a slower kernel in place.
+ * memory; larger ones, or when it cannot be had (under stream capture: when the
+ * handle has none of that size yet), by a slower kernel in place.
  * Input checks that need the data (negative weight, non-zero diagonal,
  * finite weight >= INF) run on the device; read their result with
  * apsp_last_status().  Errors returned directly: APSP_E_INVALID (null pointer,

@@ -282,8 +282,15 @@ bool needs_aligned_copy(const void *D, int64_t ld, int64_t n, int dtype, const a
 }
 
 // The copy stays with the handle, so it is kept to an eighth of the device's memory.
-bool aligned_copy_fits(const void *have, size_t have_bytes, size_t bytes) {
+// Under stream capture only a copy that is there already is used: an allocation
+// would end the capture, and the kernel without a copy allocates nothing.
+bool aligned_copy_fits(const void *have, size_t have_bytes, size_t bytes, cudaStream_t s) {
   if (have && have_bytes >= bytes) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
     cudaGetLastError();
@@ -308,11 +315,11 @@ apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, in
 // The matrix the rounds of D run on: D, or the handle's copy with 16-byte rows;
 // *ldm its leading dimension.
 void *round_matrix(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, const apsp::RoundConfig &rc,
-                   int64_t *ldm) {
+                   cudaStream_t s, int64_t *ldm) {
   int64_t ldc = 0;
   if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc)) {
     const size_t bytes = (size_t)n * ldc * (dtype == APSP_U16 ? 2 : 4);
-    if (aligned_copy_fits(h->wsD, h->wsD_bytes, bytes)) {
+    if (aligned_copy_fits(h->wsD, h->wsD_bytes, bytes, s)) {
       if (ensure(&h->wsD, &h->wsD_bytes, bytes) == cudaSuccess) {
         *ldm = ldc;
         return h->wsD;
@@ -330,7 +337,7 @@ apsp_status run_rounds_locked(apsp_handle *h, int dtype, void *D, int64_t n, int
                               bool known_sym = false) {
   apsp::RoundConfig rc = run_config(h, dtype, n);
   int64_t ldm = ld, l = 0;
-  void *M = round_matrix(h, dtype, D, n, ld, rc, &ldm);
+  void *M = round_matrix(h, dtype, D, n, ld, rc, s, &ldm);
   if (M != D) {
     const cudaError_t e = apsp::launch_input(dtype, D, ld, M, ldm, n, nullptr, nullptr, s, &l);
     h->launches += l;
@@ -349,7 +356,7 @@ apsp_status solve_dense_locked(apsp_handle *h, int dtype, const void *W, int64_t
                                cudaStream_t s) {
   apsp::RoundConfig rc = run_config(h, dtype, n);
   int64_t ldm = ld, l = 0;
-  void *M = round_matrix(h, dtype, D, n, ld, rc, &ldm);
+  void *M = round_matrix(h, dtype, D, n, ld, rc, s, &ldm);
   if (M != D) {
     rc.out = D;
     rc.out_ld = ld;
@@ -731,7 +738,7 @@ static cudaError_t minplus_locked(apsp_handle *h, int dtype, const void *A, int6
   if (scr && k > 0 && !(rows16(B, ldb) && rows16(C, ldc)) && (double)m * n * k >= kCopyProduct) {
     const int64_t ldn = round_up(n, 16 / es);
     const size_t bytes = (size_t)(k + m) * ldn * es;
-    if (aligned_copy_fits(h->mpBC, h->mpBC_bytes, bytes)) {
+    if (aligned_copy_fits(h->mpBC, h->mpBC_bytes, bytes, s)) {
       if (ensure(&h->mpBC, &h->mpBC_bytes, bytes) == cudaSuccess) {
         char *Bc = static_cast<char *>(h->mpBC), *Cc = Bc + (size_t)k * ldn * es;
         e = apsp::launch_copy_rect(dtype, B, ldb, Bc, ldn, k, n, s, &l);

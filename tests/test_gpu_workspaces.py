@@ -1,0 +1,63 @@
+"""The copies with 16-byte rows that unaligned matrices and products run on (GPU): calls under stream capture."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.test_gpu_round64 import back, graph, to_dev
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def capture(fn):
+    g = torch.cuda.CUDAGraph()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=side):
+        fn()
+    return g
+
+
+# a handle that is warm for the size, but has no copy of it yet, can be captured: nothing may be allocated then
+# (symmetric 0 without a copy reads the symmetry check back on the host, which no capture allows)
+@pytest.mark.parametrize("dtype", ["int32", "u16", "fp32"])
+@pytest.mark.parametrize("symmetric,warm", [(1, "aligned"), (2, "aligned"), (0, "unaligned"), (1, "unaligned"),
+                                            (2, "unaligned")])
+def test_unaligned_solve_under_capture(lib, dtype, symmetric, warm):
+    n = 301
+    _, _, _, W = graph(n, n)
+    E = oracle.fw(W.astype(np.int64))
+    Wa, Wu = to_dev(W, dtype, 304), to_dev(W, dtype, n)
+    D = torch.full_like(Wu, 5)
+    with lib.Handle(device=0, symmetric=symmetric) as h:
+        if warm == "aligned":
+            h.solve_t(dtype, Wa, torch.empty_like(Wa))
+        else:
+            h.solve_t(dtype, Wu, D)
+        D.fill_(5)
+        g = capture(lambda: h.solve_t(dtype, Wu, D))
+        for _ in range(2):
+            D.fill_(5)
+            g.replay()
+            torch.cuda.synchronize()
+            assert h.last_status() == 0
+            np.testing.assert_array_equal(back(D, n, dtype), E)
+        del g
+
+
+def test_unaligned_product_under_capture(lib):
+    m, k, n = 400, 300, 401
+    rng = np.random.default_rng(3)
+    A, B, C = (rng.integers(0, 5000, size=s) for s in ((m, k), (k, n), (m, n)))
+    Ad, Bd, Cd = (torch.from_numpy(x.astype(np.int32)).cuda() for x in (A, B, C))
+    with lib.Handle(device=0) as h:
+        big = [torch.zeros((512, 512), dtype=torch.int32, device="cuda") for _ in range(3)]
+        h.minplus(*big)  # warm: the workspace for A transposed
+        torch.cuda.synchronize()
+        g = capture(lambda: h.minplus(Ad, Bd, Cd))
+        g.replay()
+        torch.cuda.synchronize()
+        assert h.last_status() == 0
+        np.testing.assert_array_equal(Cd.cpu().numpy(), oracle.minplus(A, B, C))
+        del g
