@@ -318,9 +318,12 @@ void *round_matrix(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, co
                    cudaStream_t s, int64_t *ldm) {
   int64_t ldc = 0;
   if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc)) {
-    const size_t bytes = (size_t)n * ldc * (dtype == APSP_U16 ? 2 : 4);
+    // allocated in steps of 256 vertices, as the panel buffer is: growing sizes
+    // do not each synchronize the device to replace it
+    const size_t es = dtype == APSP_U16 ? 2 : 4, bytes = (size_t)n * ldc * es;
     if (aligned_copy_fits(h->wsD, h->wsD_bytes, bytes, s)) {
-      if (ensure(&h->wsD, &h->wsD_bytes, bytes) == cudaSuccess) {
+      const size_t step = (size_t)panel_ld(n) * panel_ld(n) * es;
+      if (ensure(&h->wsD, &h->wsD_bytes, h->wsD_bytes >= bytes ? bytes : step) == cudaSuccess) {
         *ldm = ldc;
         return h->wsD;
       }

@@ -1,4 +1,5 @@
-"""The copies with 16-byte rows that unaligned matrices and products run on (GPU): calls under stream capture."""
+"""The copies with 16-byte rows that unaligned matrices and products run on (GPU): calls under stream capture
+and sequences of growing sizes."""
 import numpy as np
 import pytest
 
@@ -61,3 +62,20 @@ def test_unaligned_product_under_capture(lib):
         assert h.last_status() == 0
         np.testing.assert_array_equal(Cd.cpu().numpy(), oracle.minplus(A, B, C))
         del g
+
+
+def test_growing_unaligned_sizes_reuse_the_copy(lib):
+    """Sizes that share the panel buffer (steps of 256 vertices) share the copy too: a reallocation would
+    synchronize the device in a call that is asynchronous."""
+    buf = torch.empty(2559 * 2559, dtype=torch.int32, device="cuda")
+    with lib.Handle(device=0, symmetric=2) as h:
+        free = None
+        for n in (2305, 2401, 2503, 2559):
+            W = buf[:n * n].view(n, n)
+            W.fill_(7).fill_diagonal_(0)
+            h.solve_t("int32", W, W)
+            torch.cuda.synchronize()
+            now = torch.cuda.mem_get_info()[0]
+            free = now if free is None else free
+            assert now == free, n
+            assert h.last_status() == 0 and int(W.max()) == 7 and int(W[n - 1, 0]) == 7
