@@ -158,7 +158,9 @@ struct Profiler : apsp::PhaseTimer {
 
 struct apsp_handle {
   apsp_config cfg{};
-  std::mutex mu;  // serializes solve-path workspace use and last_error
+  // serializes solve-path workspace use and last_error; recursive, since a call
+  // that holds it also records its error text (set_err)
+  std::recursive_mutex mu;
   void *colT = nullptr;
   size_t colT_bytes = 0;
   void *ws16 = nullptr;
@@ -201,7 +203,7 @@ thread_local std::string tls_error;
 
 apsp_status set_err(apsp_handle *h, apsp_status st, const std::string &msg) {
   if (h) {
-    std::lock_guard<std::mutex> g(h->mu);
+    std::lock_guard<std::recursive_mutex> g(h->mu);
     h->last_error = msg;
   }
   return st;
@@ -600,7 +602,7 @@ apsp_status apsp_solve_t(apsp_handle *h, int dtype, const void *W, int64_t n, in
   if (n > (int64_t(1) << 31) - 1) return set_err(h, APSP_E_INVALID, "n too large");
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   return solve_locked(h, dtype, W, n, ld, D, static_cast<cudaStream_t>(stream));
 }
 
@@ -618,7 +620,7 @@ apsp_status apsp_solve_edges(apsp_handle *h, int dtype, const int32_t *src, cons
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   e = cudaMemsetAsync(h->d_status, 0, sizeof(int), s);
   if (e != cudaSuccess) {
     h->last_error = std::string("status reset: ") + cudaGetErrorString(e);
@@ -677,7 +679,7 @@ apsp_status apsp_last_status(apsp_handle *h, void *stream) {
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   e = cudaMemcpyAsync(h->h_status, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
@@ -769,7 +771,7 @@ apsp_status apsp_minplus(apsp_handle *h, int dtype, const void *A, int64_t lda, 
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   if ((e = cudaMemsetAsync(h->d_status, 0, sizeof(int), s)) != cudaSuccess) return cuda_fail(h, e, "status reset");
   e = minplus_locked(h, dtype, A, lda, B, ldb, C, ldc, m, k, n, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "minplus");
@@ -785,7 +787,7 @@ apsp_status apsp_solve_squaring(apsp_handle *h, int dtype, const void *W, int64_
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   if ((e = cudaMemsetAsync(h->d_status, 0, sizeof(int), s)) != cudaSuccess) return cuda_fail(h, e, "status reset");
   if (n == 0) return APSP_OK;
   int64_t l = 0;
@@ -822,7 +824,7 @@ apsp_status apsp_tri_from_dense(apsp_handle *h, int dtype, const void *W, int64_
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   if ((e = cudaMemsetAsync(h->d_status, 0, sizeof(int), s)) != cudaSuccess) return cuda_fail(h, e, "status reset");
   int64_t l = 0;
   e = apsp::launch_tri_fill(dtype, W, ldw, T, n, h->d_status, s, &l);
@@ -840,7 +842,7 @@ apsp_status apsp_tri_from_edges(apsp_handle *h, int dtype, const int32_t *src, c
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   if ((e = cudaMemsetAsync(h->d_status, 0, sizeof(int), s)) != cudaSuccess) return cuda_fail(h, e, "status reset");
   if (n == 0) return APSP_OK;
   int64_t l = 0;
@@ -871,7 +873,7 @@ apsp_status apsp_solve_tri(apsp_handle *h, int dtype, void *T, int64_t n, void *
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   if (n == 0) return APSP_OK;
   const int64_t ldT = panel_ld(n);
   apsp::RoundConfig rc = config_for(h, dtype, n);
@@ -987,7 +989,7 @@ apsp_status apsp_solve_batch(apsp_handle *h, int64_t count, const int32_t *const
       return set_err(h, APSP_E_INVALID, "bad graph " + std::to_string(i) + " in batch");
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   std::vector<const int32_t *> Wv(W, W + count);
   std::vector<int64_t> nv(n, n + count), ldv(ld, ld + count);
   std::vector<int32_t *> Dv(D, D + count);
@@ -998,7 +1000,7 @@ apsp_status apsp_check_bounded_wait(apsp_handle *h, int64_t spin_limit) {
   if (!h || spin_limit <= 0) return APSP_E_INVALID;
   cudaError_t e = cudaSetDevice(h->cfg.device);
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaSetDevice");
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   // two checks: the batched kernel on a 96-node path (two rounds), and every
   // round of a 320-node path in one persistent launch (five rounds)
   const int64_t n = 96, n1 = 320, ldT = 512;
@@ -1152,7 +1154,7 @@ apsp_status apsp_autotune(apsp_handle *h, int dtype, int64_t n_max, const char *
   if ((e = cudaGetDeviceProperties(&prop, h->cfg.device)) != cudaSuccess) return cuda_fail(h, e, "properties");
   const std::string gpu = prop.name;
   std::vector<TuneEntry> cache = read_cache(cache_path);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   const int64_t top = bucket_of(n_max);
   const size_t es = dtype == APSP_U16 ? 2 : 4;
   bool wrote = false;
@@ -1224,7 +1226,7 @@ apsp_status apsp_autotune(apsp_handle *h, int dtype, int64_t n_max, const char *
 
 apsp_status apsp_tuned_config(apsp_handle *h, int dtype, int64_t n, int *block_k, int *tma) {
   if (!h || !block_k || !tma || !valid_dtype(dtype) || n < 0) return APSP_E_INVALID;
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   const apsp::RoundConfig c = config_for(h, dtype, n);
   *block_k = c.bk;
   *tma = c.p3;
@@ -1250,7 +1252,7 @@ const char *apsp_strerror(apsp_status s) {
 
 const char *apsp_last_error(apsp_handle *h) {
   if (!h) return "null handle";
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   tls_error = h->last_error;
   return tls_error.c_str();
 }
@@ -1260,7 +1262,7 @@ int64_t apsp_launch_count(apsp_handle *h) { return h ? h->launches.load() : 0; }
 apsp_status apsp_profile(apsp_handle *h, int enable) {
   if (!h) return APSP_E_INVALID;
   cudaSetDevice(h->cfg.device);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   if (enable && !h->prof) h->prof.reset(new Profiler());
   if (!enable && h->prof) {
     cudaDeviceSynchronize();
@@ -1272,7 +1274,7 @@ apsp_status apsp_profile(apsp_handle *h, int enable) {
 apsp_status apsp_profile_read(apsp_handle *h, int64_t launches[3], double ms[3], double relaxations[3]) {
   if (!h) return APSP_E_INVALID;
   cudaSetDevice(h->cfg.device);
-  std::lock_guard<std::mutex> g(h->mu);
+  std::lock_guard<std::recursive_mutex> g(h->mu);
   if (!h->prof) {
     for (int p = 0; p < 3; ++p) {
       if (launches) launches[p] = 0;
