@@ -445,7 +445,8 @@ int64_t apsp_launch_count(apsp_handle *h);
  * the recorded events and writes, for phases 0, 1, 2 (= Phase 1, 2, 3), the
  * number of timed launches, their summed device time in ms, and their summed
  * algorithmic relaxation counts (Phase 1: w^3, Phase 2: 2 (n-w) w^2, Phase 3:
- * (n-w)^2 w for a round of width w; with 64-wide rounds and the
+ * (n-w)^2 w for a round of width w; in symmetric mode half of Phase 2's and the
+ * processed tiles' share of Phase 3's; with 64-wide rounds and the
  * warp-specialized kernel only round 0 has a Phase-1 launch, the later diagonal
  * blocks are closed inside Phase 3); then it clears the record.  Any of the
  * output arrays may be NULL. */

@@ -2339,7 +2339,8 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
                  dev_sym ? sym_flag : (const int *)nullptr);
     }
     if (launches) *launches += 1;
-    if (tm) tm->after(1, s, sym ? rest * w * w : 2.0 * rest * w * w);
+    if (tm && dev_sym) tm->after_choice(1, s, rest * w * w, 2.0 * rest * w * w, sym_flag);
+    else if (tm) tm->after(1, s, sym ? rest * w * w : 2.0 * rest * w * w);
   };
   // Widths 32 and 128: Phase 1 and Phase 2 of round k as their own launches.
   auto panels = [&](int64_t k, uint32_t *cT, Elem *rP) {
