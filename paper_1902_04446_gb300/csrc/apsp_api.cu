@@ -62,6 +62,7 @@ struct Request {
   bool admitted = false;
   bool finished = false;
   bool alone = false;     // runs in its own group on the per-round kernels
+  bool copy = false;      // solved in a copy with 16-byte rows (request_copy_bytes)
   apsp_status err = APSP_OK;
   void *D = nullptr;
   std::shared_ptr<Group> group;
@@ -1306,7 +1307,12 @@ constexpr int kMaxGroupsInFlight = 16;
 constexpr int64_t kLargeN = 1536;
 int64_t large_n(const apsp_handle *h) { return h->cfg.serving_large_n > 0 ? h->cfg.serving_large_n : kLargeN; }
 
-int64_t panel_bytes(int64_t n) { return 64 * apsp::batch_panel_ld(n) * 4 + 256; }
+// Bytes of a request's panels in the batched kernel, the closed diagonal block
+// with them, and the least that a request is accepted for: its matrix and panel
+// rows.  One that fits with nothing else in flight runs, if need be in place
+// (no copy) and with that block (32 KB) past the budget.
+int64_t panel_bytes(int64_t n) { return apsp::batch_panel_bytes(n) + 256; }
+int64_t least_bytes(int64_t n) { return n * n * 4 + panel_bytes(n) - (int64_t)apsp::kDiagBufBytes; }
 
 // Bytes of the copy with 16-byte rows that a request is solved in: a result has
 // rows of n elements, so n % 4 != 0 needs one.  0 where the rows are aligned, or
@@ -1484,7 +1490,7 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
     apsp::RoundConfig rc = large_round_config(h, APSP_I32, rn);
     void *M = rs[0]->D;  // the matrix the rounds run on: the request's, or a copy with 16-byte rows
     int64_t ldm = rn;
-    const bool copy = needs_aligned_copy(rs[0]->D, rn, rn, APSP_I32, rc, &ldm) && request_copy_bytes(h, rn) > 0;
+    const bool copy = needs_aligned_copy(rs[0]->D, rn, rn, APSP_I32, rc, &ldm) && rs[0]->copy;
     if (!copy) ldm = rn;
     const size_t pb = (apsp::panel_buffer_bytes(rn, ldT, rc.p3 == 4) + 255) & ~size_t(255);
     if (cudaMallocAsync(&g->ws, pb + (copy ? (size_t)rn * ldm * 4 : 0), s) != cudaSuccess) {
@@ -1526,7 +1532,7 @@ apsp_status admit_group_steps(apsp_handle *h, const std::vector<Request *> &rs, 
   for (size_t i = 0; i < rs.size(); ++i) {
     const int64_t rn = rs[i]->req.n;
     int32_t *Di = static_cast<int32_t *>(rs[i]->D);
-    if (rn > 0) in.push_back(apsp::BatchInput{Di, Di, rn, rn, rn, g->status + i, request_copy_bytes(h, rn) > 0});
+    if (rn > 0) in.push_back(apsp::BatchInput{Di, Di, rn, rn, rn, g->status + i, rs[i]->copy});
   }
   apsp::BatchPlan plan;
   if (cudaMallocAsync(&g->ws, std::max<size_t>(plan.build(in, nullptr), 256), s) != cudaSuccess) {
@@ -1564,13 +1570,21 @@ void worker_loop(apsp_handle *h) {
         const bool big = r->req.n >= large_n(h);
         bool large = lone || big;
         if (large && !rs.empty()) break;  // a large request starts its own group
-        const int64_t base = r->bytes + panel_bytes(r->req.n) + request_copy_bytes(h, r->req.n);
-        int64_t b = base + (large ? large_extra_bytes(h, r->req) : 0);
+        // the per-round kernels keep the diagonal block in their own panel buffer
+        const int64_t least = least_bytes(r->req.n), copy = request_copy_bytes(h, r->req.n);
+        const int64_t extra = large ? large_extra_bytes(h, r->req) : 0;
+        int64_t b = least + copy + (large ? extra : (int64_t)apsp::kDiagBufBytes);
+        r->copy = copy > 0;
         if (large && !big && h->used + add + b > h->budget) {
           large = false;  // no room for the per-round workspace: the batched kernel after all
-          b = base;
+          b = least + copy + (int64_t)apsp::kDiagBufBytes;
         }
-        if (h->used + add + b > h->budget) break;  // wait for memory to free up
+        if (h->used + add + b > h->budget) {
+          // wait for memory to free up, unless nothing in flight can free any
+          if (!rs.empty() || !h->groups.empty() || h->used + least + (large ? extra : 0) > h->budget) break;
+          r->copy = false;
+          b -= copy;
+        }
         h->queue.pop_front();
         r->alone = large;
         r->transient = b - r->bytes;
@@ -1636,7 +1650,7 @@ apsp_status apsp_submit(apsp_handle *h, const apsp_request *r, uint64_t *ticket)
   std::unique_lock<std::mutex> g(h->smu);
   start_worker(h);
   const int64_t bytes = r->n * r->n * 4;
-  if (bytes + panel_bytes(r->n) > h->budget) return APSP_E_NOMEM;
+  if (least_bytes(r->n) > h->budget) return APSP_E_NOMEM;
   if ((int64_t)h->queue.size() >= h->cfg.queue_depth) return APSP_E_BUSY;
   std::unique_ptr<Request> q(new Request());
   q->ticket = h->next_ticket++;

@@ -299,8 +299,6 @@ size_t pad256(size_t b) { return (b + 255) / 256 * 256; }
 
 }  // namespace
 
-int64_t batch_panel_ld(int64_t n) { return ((n > 0 ? n : 1) + 255) / 256 * 256; }
-
 size_t BatchPlan::build(const std::vector<BatchInput> &in, char *base) {
   graphs.clear();
   segs.clear();
@@ -377,7 +375,7 @@ size_t BatchPlan::build(const std::vector<BatchInput> &in, char *base) {
   for (size_t i = 0; i < graphs.size(); ++i) {
     BatchGraph &g = graphs[i];
     g.colT = reinterpret_cast<uint32_t *>(base + off);
-    off += pad256((size_t)64 * g.ldT * 4 + sizeof(DiagBuf));
+    off += pad256((size_t)batch_panel_bytes(g.n));
     g.M = g.D;
     if (g.ld != g.ldd || (in[i].copy && reinterpret_cast<uintptr_t>(g.D) % 16 != 0)) {
       g.M = reinterpret_cast<int32_t *>(base + off);

@@ -6,6 +6,8 @@
 
 #include <cuda_runtime.h>
 
+#include "fw_launch.h"
+
 namespace apsp {
 
 // Default bound on every dependency wait of the batched kernel (polls with a
@@ -54,7 +56,9 @@ struct BatchPlan {
 };
 
 // Panel-buffer leading dimension for a graph of n vertices (words per row; 64 rows).
-int64_t batch_panel_ld(int64_t n);
+inline int64_t batch_panel_ld(int64_t n) { return ((n > 0 ? n : 1) + 255) / 256 * 256; }
+// Bytes of the panel buffer and the closed diagonal block (DiagBuf) behind it.
+inline int64_t batch_panel_bytes(int64_t n) { return 64 * batch_panel_ld(n) * 4 + (int64_t)kDiagBufBytes; }
 // Bytes of the copy with 16-byte rows of an n x n int32 matrix.
 inline int64_t batch_copy_bytes(int64_t n) { return n * ((n + 3) / 4 * 4) * 4 + 256; }
 
