@@ -355,10 +355,11 @@ apsp_status apsp_cancel(apsp_handle *h, uint64_t ticket);
  * when present, and new results are written back.  Synchronizes the device. */
 apsp_status apsp_autotune(apsp_handle *h, int dtype, int64_t n_max, const char *cache_path);
 
-/* The round shape the handle uses for (dtype, n): *block_k and *tma, the
+/* The round shape that apsp_config, apsp_autotune or, without either, the
+ * default table by n and dtype gives for (dtype, n): *block_k and *tma, the
  * Phase-3 kernel numbered as apsp_config.phase3_variant minus one (0 = one
  * CTA per tile, 1-3 = the persistent TMA kernels launched per round, 4 = every
- * round in one launch).  A 4 that neither apsp_config nor apsp_autotune chose
+ * round in one launch).  Solves run this shape, but a 4 from the default table
  * runs as 3 where that was measured faster: int32 below n = 7680 and from 14336,
  * packed 16-bit below 9216 and from 32768, fp32 at every n. */
 apsp_status apsp_tuned_config(apsp_handle *h, int dtype, int64_t n, int *block_k, int *tma);

@@ -61,29 +61,24 @@ bool single_launch(int dtype, const void *D, int64_t ld, int64_t n, const RoundC
 // decided on the device, by the single launch or by the warp-specialized kernel
 // at width 64.
 bool device_sym(int dtype, const void *D, int64_t ld, int64_t n, const RoundConfig &cfg);
-// The default Phase-3 kernel for (n, dtype) when nothing was tuned: every round
-// in one launch for mid-size n, one launch per round below and above (timed per
-// n and dtype on GB300, the per-round kernels with programmatic dependent
-// launch).  Below the lower cut a round is at most a few waves of tiles and the
-// per-round launches are cheaper than the single launch's item scheduling;
-// above the upper cut the per-round launches' fixed cost per round is small
-// against the single launch's cost per tile.  Measured (symmetric mode, ms per
-// solve, one launch per round / single launch): int32 n = 5120 6.52 / 6.89,
-// 6144 9.89 / 8.62, 16384 128.4 / 125.6, 32768 954 / 975; packed 16-bit
-// n = 5120 5.48 / 6.23, 6144 8.05 / 7.66, 65536 3922 / 3983 (its rounds have
-// half the tiles); fp32 n = 5120 6.39 / 6.82, 6144 9.60 / 8.55.
+// The default table of Phase-3 kernels by (n, dtype), as apsp_tuned_config
+// answers it when nothing was tuned: every round in one launch for mid-size n,
+// one launch per round below and above.  Solves follow it through solve_phase3,
+// below, which holds the measurements.
 inline int default_phase3(int64_t n, int dtype) {
   const int64_t hi = dtype == 1 ? 49152 : 24576;
   return n >= 6144 && n < hi ? 4 : 3;
 }
-// The default round width for (n, dtype): 128 where large n runs one launch
-// per round in packed 16-bit or fp32 (each tile then takes 128 k-steps in two
-// stages and stores its C block half as often), else 64.  Measured (symmetric
-// mode, ms per solve, width 64 / 128): fp32 n = 65536 7177 / 6967, packed
-// 16-bit n = 65536 3931 / 3910, n = 32768 528 / 519; int32 n = 65536 7486 /
-// 7550 (its k-loop runs slower in the two-stage kernel than the epilogue
-// saves), and every element type at small n, where the 128-wide Phase 1 on
-// one SM is on the critical path (int32 n = 4096 4.07 / 5.24).
+// The default round width for (n, dtype): 128 where the table runs large n in
+// packed 16-bit or fp32 one launch per round (each tile then takes 128 k-steps in
+// two stages and stores its C block half as often), else 64.  Measured (symmetric
+// mode, one launch per round, ms per solve, width 64 / 128): packed 16-bit
+// n = 24576 201 / 204, 32768 464 / 455, 49152 1510 / 1473, 65536 3512 / 3431;
+// fp32 n = 16384 104.2 / 109.3, 24576 340 / 344, 32768 799 / 791, 65536 6295 /
+// 6129; int32 n = 65536 6450 / 6568 (its k-loop runs slower in the two-stage
+// kernel than the epilogue saves), and every element type at small n, where the
+// 128-wide Phase 1 on one SM is on the critical path (int32 n = 4096 2.46 /
+// 4.86).  So the line is right within about 2 % on either side of it.
 inline int default_round_width(int64_t n, int dtype) {
   return dtype != 0 && default_phase3(n, dtype) == 3 && n >= 6144 ? 128 : 64;
 }
@@ -97,10 +92,11 @@ inline int default_round_width(int64_t n, int dtype) {
 // gains, for the integer types, where a round is a few dozen waves of tiles, by
 // starting a round's tiles before the previous round's last wave has ended.
 // Measured (symmetric mode, ms per solve, per round / single launch): int32
-// n = 6144 7.07 / 7.98, 7168 10.9 / 10.9, 8192 15.4 / 14.7, 12288 47.8 / 47.4,
-// 16384 108.7 / 109.5; packed 16-bit n = 6144 4.52 / 7.03, 8192 10.1 / 11.6,
-// 10240 18.1 / 17.1, 24576 205.0 / 201.1, 49152 1498 / 1534; fp32 n = 6144
-// 6.92 / 8.06, 8192 15.1 / 15.5, 16384 105.7 / 113.9.
+// n = 6144 6.70 / 7.80, 7168 10.3 / 10.6, 7680 13.0 / 12.1, 8192 14.8 / 14.3,
+// 12288 46.2 / 46.6, 16384 107.0 / 108.1, 24576 350 / 358; packed 16-bit n = 6144
+// 4.13 / 6.68, 8192 8.9 / 11.2, 9216 12.3 / 13.4, 10240 16.6 / 16.3, 16384 62.9 /
+// 61.7, 24576 201.4 / 199.4, 32768 463.6 / 464.2, 49152 1510 / 1539; fp32
+// n = 6144 6.60 / 7.81, 8192 14.6 / 15.0, 16384 104.2 / 112.3.
 inline int solve_phase3(int64_t n, int dtype) {
   if (default_phase3(n, dtype) != 4) return 3;
   if (dtype == 0) return n >= 7680 && n < 14336 ? 4 : 3;

@@ -302,7 +302,8 @@ class Handle:
             b <<= 1
 
     def tuned_config(self, dtype, n: int):
-        """apsp_tuned_config: (Bk, tma) the handle uses for (dtype, n)."""
+        """apsp_tuned_config: (Bk, tma) of the configuration, the autotuner or the default table for (dtype, n); a
+        solve runs a default tma of 4 as 3 where that is faster (include/apsp.h)."""
         bk, tma = ctypes.c_int(), ctypes.c_int()
         self._check(_L().apsp_tuned_config(self._h, dtype_code(dtype), n, ctypes.byref(bk), ctypes.byref(tma)),
                     "apsp_tuned_config")
