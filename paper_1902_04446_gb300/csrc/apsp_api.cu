@@ -941,7 +941,8 @@ apsp_status batch_locked(apsp_handle *h, const std::vector<const int32_t *> &W, 
   int64_t copies = 0;
   for (size_t i = 0; i < n.size(); ++i) {
     if (n[i] == 0) continue;
-    const bool unaligned = reinterpret_cast<uintptr_t>(D[i]) % 16 != 0 || ld[i] % 4 != 0;
+    // a graph of one round reads and writes its matrix once: a copy would not pay
+    const bool unaligned = n[i] > 64 && (reinterpret_cast<uintptr_t>(D[i]) % 16 != 0 || ld[i] % 4 != 0);
     if (unaligned) copies += apsp::batch_copy_bytes(n[i]);
     in.push_back(apsp::BatchInput{W[i], D[i], n[i], ld[i], ld[i], h->d_status, unaligned});
   }
