@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(TileMap<128, 128, TN>::THREADS, 1)
   __shared__ __align__(8) uint64_t bar_ab[2];
   __shared__ __align__(8) uint64_t bar_c;
   __shared__ int abort_flag;
-  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
+  uint8_t *base = align_smem(smem_raw);
   // stage s: A at base + s * STAGE, B right after it; C after both stages
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * P3T_STAGE_BYTES); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * P3T_STAGE_BYTES) + BK * BM; };
@@ -532,6 +532,10 @@ struct P3Loop<OpU16, BK> {
   using AnyProduct = KLoop<false, 8, false, 4>;  // no FMA form (see tile_minplus)
   using PlainProduct = AnyProduct;
 };
+// fp32 products: of 15 schedules timed these are the fastest although they spill
+// (fw_minplus_ws 44 bytes a thread at 168 registers, 4096 cubed 3289 us, the
+// fastest without spills, KLoop<false, 1, false, 1>, 3312; minplus_kernel 480
+// bytes at 128 registers, 200 x 200 x 201 58 us, the others 58 - 69).
 template <int BK>
 struct P3Loop<OpF32, BK> {
   using Round = KLoop<true, 1, true, 0>;
@@ -698,7 +702,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_ab[2], empty_ab[2], full_c, cdone, cfree;
   __shared__ int abort_flag;
-  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
+  uint8_t *base = align_smem(smem_raw);
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE) + KS * BM; };
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
@@ -1193,7 +1197,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   __shared__ __align__(8) uint64_t full_ab[2], empty_ab[2], full_c, cdone, cfree;
   __shared__ int slot_kind[2], slot_info[2], slot_round[2];
   __shared__ int abort_flag;
-  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
+  uint8_t *base = align_smem(smem_raw);
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE) + BK * BM; };
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
@@ -1769,7 +1773,7 @@ __global__ void __launch_bounds__(P3W_THREADS, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_ab[2], empty_ab[2], full_c, cdone, cfree;
   __shared__ int abort_flag;
-  uint8_t *base = smem_raw + ((0u - smem_addr(smem_raw)) & 1023u);
+  uint8_t *base = align_smem(smem_raw);
   auto stA = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE); };
   auto stB = [&](int s) { return reinterpret_cast<uint32_t *>(base + s * STAGE) + BK * BM; };
   uint32_t *Cs = reinterpret_cast<uint32_t *>(base + 2 * STAGE);
@@ -2345,44 +2349,44 @@ static cudaError_t rounds_impl(void *Dv, Layout L, int64_t n, void *colTv, int64
   // Widths 32 and 128: Phase 1 and Phase 2 of round k as their own launches.
   auto panels = [&](int64_t k, uint32_t *cT, Elem *rP) {
     if constexpr (BK != 64) {
-    int64_t p0, p1;
-    span(k, p0, p1);
-    const double w = (double)(p1 - p0), rest = (double)(n - (p1 - p0));
-    if (tm) tm->before(0, s);
-    if constexpr (BK > 64)
-      launch_pdl(fw_phase1_w128<Op>, dim3(1), dim3(P1W_THREADS), sizeof(P1WSmem<Op>), s, D, L, n, p0, cT, ldT,
-                 sym ? rP : nullptr);
-    else if (sym && rP)
-      launch_pdl(fw_phase1_sym<Op, BK>, dim3(1), dim3(P1_THREADS), 0, s, D, L, n, p0, cT, ldT, rP);
-    else
-      launch_pdl(fw_phase1<Op, BK>, dim3(1), dim3(P1_THREADS), 0, s, D, L, n, p0, cT, ldT);
-    if (launches) *launches += 1;
-    if (tm) tm->after(0, s, w * w * w);
-    if (q == 1) return;
-    if (tm) tm->before(1, s);
-    SymPanel<Op> sp{rP, (p0 / (128 * Op::EPW)) * (128 * Op::EPW) + 128 * Op::EPW};
-    int r_first = 0, r_count = nrow, c_count = ncol;
-    if (sym) {  // row chunks that reach columns >= p1; column chunks with rows < p0
-      r_first = (int)(p1 / (C2::ROW_BNW * Op::EPW));
-      r_count = std::max(0, nrow - r_first);
-      c_count = (int)((p0 + C2::COL_BM - 1) / C2::COL_BM);
-    }
-    if (r_count + c_count > 0) {
-      launch_pdl(fw_phase2<Op, BK>, dim3(r_count + c_count), dim3(C2::THREADS), (size_t)C2::SMEM, s, D, L, n, p0, p1, cT,
-                 ldT, r_count, vec ? 1 : 0, r_first, sym ? 1 : 0, sp);
+      int64_t p0, p1;
+      span(k, p0, p1);
+      const double w = (double)(p1 - p0), rest = (double)(n - (p1 - p0));
+      if (tm) tm->before(0, s);
+      if constexpr (BK > 64)
+        launch_pdl(fw_phase1_w128<Op>, dim3(1), dim3(P1W_THREADS), sizeof(P1WSmem<Op>), s, D, L, n, p0, cT, ldT,
+                   sym ? rP : nullptr);
+      else if (sym && rP)
+        launch_pdl(fw_phase1_sym<Op, BK>, dim3(1), dim3(P1_THREADS), 0, s, D, L, n, p0, cT, ldT, rP);
+      else
+        launch_pdl(fw_phase1<Op, BK>, dim3(1), dim3(P1_THREADS), 0, s, D, L, n, p0, cT, ldT);
       if (launches) *launches += 1;
-    }
-    if (sym && p0 > 0) {
-      const int64_t band_start = (p0 / (128 * Op::EPW)) * (128 * Op::EPW);
-      const int64_t xs = rP ? p0 : p0 - band_start;  // elements to visit per row
-      const unsigned gx = (unsigned)std::min<int64_t>((xs + 255) / 256, 64);
-      if (xs > 0) {
-        launch_pdl(panel_finalize<Op>, dim3(gx, BK), dim3(256), 0, s, D, L, n, p0, (const uint32_t *)cT, ldT, rP,
-                   band_start);
+      if (tm) tm->after(0, s, w * w * w);
+      if (q == 1) return;
+      if (tm) tm->before(1, s);
+      SymPanel<Op> sp{rP, (p0 / (128 * Op::EPW)) * (128 * Op::EPW) + 128 * Op::EPW};
+      int r_first = 0, r_count = nrow, c_count = ncol;
+      if (sym) {  // row chunks that reach columns >= p1; column chunks with rows < p0
+        r_first = (int)(p1 / (C2::ROW_BNW * Op::EPW));
+        r_count = std::max(0, nrow - r_first);
+        c_count = (int)((p0 + C2::COL_BM - 1) / C2::COL_BM);
+      }
+      if (r_count + c_count > 0) {
+        launch_pdl(fw_phase2<Op, BK>, dim3(r_count + c_count), dim3(C2::THREADS), (size_t)C2::SMEM, s, D, L, n, p0,
+                   p1, cT, ldT, r_count, vec ? 1 : 0, r_first, sym ? 1 : 0, sp);
         if (launches) *launches += 1;
       }
-    }
-    if (tm) tm->after(1, s, sym ? rest * w * w : 2.0 * rest * w * w);
+      if (sym && p0 > 0) {
+        const int64_t band_start = (p0 / (128 * Op::EPW)) * (128 * Op::EPW);
+        const int64_t xs = rP ? p0 : p0 - band_start;  // elements to visit per row
+        const unsigned gx = (unsigned)std::min<int64_t>((xs + 255) / 256, 64);
+        if (xs > 0) {
+          launch_pdl(panel_finalize<Op>, dim3(gx, BK), dim3(256), 0, s, D, L, n, p0, (const uint32_t *)cT, ldT, rP,
+                     band_start);
+          if (launches) *launches += 1;
+        }
+      }
+      if (tm) tm->after(1, s, sym ? rest * w * w : 2.0 * rest * w * w);
     }
   };
   // relaxations of round k's Phase 3 actually performed: the processed tiles' share of (n - w)^2 w

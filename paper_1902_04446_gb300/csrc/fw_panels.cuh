@@ -6,8 +6,9 @@
 // by the chain diagonal closure -> panels -> tiles: at n = 2048 38 us, of which
 // the tiles' add-mins need 7.  Here a round is two launches:
 //   fw_panels   relaxes every chunk of the panels with the closed diagonal
-//               block (16 words wide, so that a small n still fills the GPU), and publishes them: D, colT, and in symmetric mode the
-//               element panel and the band elements below the diagonal;
+//               block (16 words wide, so that a small n still fills the GPU),
+//               and publishes them: D, colT, and in symmetric mode the element
+//               panel and the band elements below the diagonal;
 //   Phase 3     whose first CTA, before its tiles, applies this round's update
 //               to the next diagonal block and closes it (next_diag), into a
 //               side buffer that the next fw_panels reads and copies into D.
