@@ -126,8 +126,8 @@ apsp_status apsp_destroy(apsp_handle *h);
  * APSP_AUTO synchronizes the stream once to read the 16-bit bound.
  * Matrices without 16-byte rows (base or ld * element size not a multiple of 16)
  * are solved in a copy that the handle keeps, up to an eighth of the device's
- * memory; larger ones, or when it cannot be had (under stream capture: when the
- * handle has none of that size yet), by a slower kernel in place.
+ * memory; larger ones, when it cannot be had, and under stream capture, by a
+ * slower kernel in place.
  * Input checks that need the data (negative weight, non-zero diagonal,
  * finite weight >= INF) run on the device; read their result with
  * apsp_last_status().  Errors returned directly: APSP_E_INVALID (null pointer,
@@ -200,7 +200,8 @@ apsp_status apsp_check_bounded_wait(apsp_handle *h, int64_t spin_limit);
  * about 4*m*k bytes (A transposed) for the TMA-fed kernel when it can be
  * allocated and B and C are 16-byte addressable or can be copied (products of
  * 1.6e7 relaxations and more; the copies stay with the handle, up to an eighth of
- * the device's memory); otherwise a kernel without workspace.  Asynchronous on `stream`; a device wait that gave up is reported
+ * the device's memory; none under stream capture); otherwise a kernel without
+ * workspace.  Asynchronous on `stream`; a device wait that gave up is reported
  * by apsp_last_status (bit 4).  Errors: APSP_E_INVALID, APSP_E_CUDA. */
 apsp_status apsp_minplus(apsp_handle *h, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb,
                          void *C, int64_t ldc, int64_t m, int64_t k, int64_t n, void *stream);

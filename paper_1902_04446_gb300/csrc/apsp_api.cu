@@ -284,16 +284,19 @@ bool needs_aligned_copy(const void *D, int64_t ld, int64_t n, int dtype, const a
   return n > 64 && rc.p3 != 0 && (reinterpret_cast<uintptr_t>(D) % 16 != 0 || ld * es % 16 != 0);
 }
 
-// The copy stays with the handle, so it is kept to an eighth of the device's memory.
-// Under stream capture only a copy that is there already is used: an allocation
-// would end the capture, and the kernel without a copy allocates nothing.
-bool aligned_copy_fits(const void *have, size_t have_bytes, size_t bytes, cudaStream_t s) {
-  if (have && have_bytes >= bytes) return true;
+// Calls under stream capture use no copies: allocating one would end the capture,
+// and a captured graph would keep the pointer of one that a later, larger call
+// replaces.  The kernels without copies run then.
+bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+// The copy stays with the handle, so it is kept to an eighth of the device's memory.
+bool aligned_copy_fits(const void *have, size_t have_bytes, size_t bytes) {
+  if (have && have_bytes >= bytes) return true;
   size_t fr = 0, tot = 0;
   if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
     cudaGetLastError();
@@ -320,11 +323,11 @@ apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, in
 void *round_matrix(apsp_handle *h, int dtype, void *D, int64_t n, int64_t ld, const apsp::RoundConfig &rc,
                    cudaStream_t s, int64_t *ldm) {
   int64_t ldc = 0;
-  if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc)) {
+  if (needs_aligned_copy(D, ld, n, dtype, rc, &ldc) && !capturing(s)) {
     // allocated in steps of 256 vertices, as the panel buffer is: growing sizes
     // do not each synchronize the device to replace it
     const size_t es = dtype == APSP_U16 ? 2 : 4, bytes = (size_t)n * ldc * es;
-    if (aligned_copy_fits(h->wsD, h->wsD_bytes, bytes, s)) {
+    if (aligned_copy_fits(h->wsD, h->wsD_bytes, bytes)) {
       const size_t step = (size_t)panel_ld(n) * panel_ld(n) * es;
       if (ensure(&h->wsD, &h->wsD_bytes, h->wsD_bytes >= bytes ? bytes : step) == cudaSuccess) {
         *ldm = ldc;
@@ -396,6 +399,10 @@ apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, in
     h->last_error = std::string("panel workspace: ") + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? APSP_E_NOMEM : APSP_E_CUDA;
   }
+  // captured in place of a solve in a copy: no answer can be read back, so the
+  // general mode, exact for any W
+  int64_t copy_ld = 0;
+  const bool in_place_capture = needs_aligned_copy(D, ld, n, dtype, rc, &copy_ld) && capturing(s);
   if (h->cfg.symmetric == 1 || (h->cfg.symmetric == 0 && known_sym)) {
     rc.sym = true;
   } else if (h->cfg.symmetric == 0 && n > 1 && apsp::device_sym(dtype, D, ld, n, rc)) {
@@ -408,7 +415,7 @@ apsp_status run_rounds_aligned(apsp_handle *h, int dtype, void *D, int64_t n, in
       return APSP_E_CUDA;
     }
     rc.sym_flag = flag;
-  } else if (h->cfg.symmetric == 0 && n > 1) {
+  } else if (h->cfg.symmetric == 0 && n > 1 && !in_place_capture) {
     // device check of W == W^T; the answer is read back before the rounds are enqueued
     int *flag = h->d_status + 1;
     e = check_symmetry(h, dtype, D, n, ld, flag_ready, s);
@@ -741,10 +748,11 @@ static cudaError_t minplus_locked(apsp_handle *h, int dtype, const void *A, int6
   };
   int64_t l = 0;
   cudaError_t e = cudaSuccess;
-  if (scr && k > 0 && !(rows16(B, ldb) && rows16(C, ldc)) && (double)m * n * k >= kCopyProduct) {
+  if (scr && k > 0 && !(rows16(B, ldb) && rows16(C, ldc)) && (double)m * n * k >= kCopyProduct &&
+      !capturing(s)) {
     const int64_t ldn = round_up(n, 16 / es);
     const size_t bytes = (size_t)(k + m) * ldn * es;
-    if (aligned_copy_fits(h->mpBC, h->mpBC_bytes, bytes, s)) {
+    if (aligned_copy_fits(h->mpBC, h->mpBC_bytes, bytes)) {
       if (ensure(&h->mpBC, &h->mpBC_bytes, bytes) == cudaSuccess) {
         char *Bc = static_cast<char *>(h->mpBC), *Cc = Bc + (size_t)k * ldn * es;
         e = apsp::launch_copy_rect(dtype, B, ldb, Bc, ldn, k, n, s, &l);

@@ -20,11 +20,10 @@ def capture(fn):
     return g
 
 
-# a handle that is warm for the size, but has no copy of it yet, can be captured: nothing may be allocated then
-# (symmetric 0 without a copy reads the symmetry check back on the host, which no capture allows)
+# a handle that is warm for the size can be captured: nothing may be allocated then
 @pytest.mark.parametrize("dtype", ["int32", "u16", "fp32"])
-@pytest.mark.parametrize("symmetric,warm", [(1, "aligned"), (2, "aligned"), (0, "unaligned"), (1, "unaligned"),
-                                            (2, "unaligned")])
+@pytest.mark.parametrize("symmetric,warm", [(0, "aligned"), (1, "aligned"), (2, "aligned"), (0, "unaligned"),
+                                            (1, "unaligned"), (2, "unaligned")])
 def test_unaligned_solve_under_capture(lib, dtype, symmetric, warm):
     n = 301
     _, _, _, W = graph(n, n)
@@ -44,6 +43,30 @@ def test_unaligned_solve_under_capture(lib, dtype, symmetric, warm):
             torch.cuda.synchronize()
             assert h.last_status() == 0
             np.testing.assert_array_equal(back(D, n, dtype), E)
+        del g
+
+
+@pytest.mark.parametrize("wider", [False, True])
+def test_captured_solve_outlives_the_copy_of_its_size(lib, wider):
+    """A larger unaligned solve (more vertices, or wider elements) replaces the handle's copy; a graph captured
+    before still replays right."""
+    n, m = 301, 900
+    _, _, _, W = graph(n, n)
+    E = oracle.fw(W.astype(np.int64))
+    Wu, Wm = to_dev(W, "u16", n), graph(m, m)[3]
+    D = torch.full_like(Wu, 5)
+    with lib.Handle(device=0) as h:
+        Wa = to_dev(Wm, "int32", m)  # rows of 16 bytes
+        h.solve_t("int32", Wa, torch.empty_like(Wa))  # the panel buffer for m vertices, no copy
+        h.solve_t("u16", Wu, D)
+        g = capture(lambda: h.solve_t("u16", Wu, D))
+        Wb = to_dev(W, "int32", n) if wider else to_dev(Wm, "int32", m + 1)
+        h.solve_t("int32", Wb, torch.empty_like(Wb))
+        D.fill_(5)
+        g.replay()
+        torch.cuda.synchronize()
+        assert h.last_status() == 0
+        np.testing.assert_array_equal(back(D, n, "u16"), E)
         del g
 
 
