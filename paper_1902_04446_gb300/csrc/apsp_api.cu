@@ -174,8 +174,9 @@ struct apsp_handle {
   size_t rowP_bytes = 0;
   void *mpT = nullptr;  // min-plus product: A^T (32-bit words)
   size_t mpT_bytes = 0;
-  void *mpBC = nullptr;  // min-plus product: copies of B and C with 16-byte rows
+  void *mpBC = nullptr;  // min-plus product: A^T and copies of B and C with 16-byte rows
   size_t mpBC_bytes = 0;
+  cudaEvent_t mpBC_done = nullptr;  // after the last product that used mpBC
   int *d_status = nullptr;
   int *h_status = nullptr;  // pinned
   std::string last_error;
@@ -597,6 +598,7 @@ apsp_status apsp_destroy(apsp_handle *h) {
   if (h->rowP) cudaFree(h->rowP);
   if (h->mpT) cudaFree(h->mpT);
   if (h->mpBC) cudaFree(h->mpBC);
+  if (h->mpBC_done) cudaEventDestroy(h->mpBC_done);
   if (h->d_status) cudaFree(h->d_status);
   if (h->h_status) cudaFreeHost(h->h_status);
   delete h;
@@ -730,43 +732,62 @@ apsp_status apsp_int16_bound(apsp_handle *h, const int32_t *W, int64_t n, int64_
 // 5001 2108 / 1532.
 constexpr double kCopyProduct = 1.6e7;
 
-// The product into C with the library's A^T workspace (the warp-specialized
-// kernel) when it can be had, else the one-CTA-per-tile kernel.  h->mu held.
+// A product on copies of B and C with 16-byte rows, *ran = whether they could be
+// had.  Products on such B and C need no workspace otherwise and may run on
+// several streams at once, so this one keeps its A^T beside the copies and waits
+// for the last product that used them.  h->mu held.
+static cudaError_t minplus_on_copies(apsp_handle *h, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb,
+                                     void *C, int64_t ldc, int64_t m, int64_t k, int64_t n, cudaStream_t s, bool *ran) {
+  const int64_t es = dtype == APSP_U16 ? 2 : 4, ldn = round_up(n, 16 / es);
+  const size_t need = (apsp::minplus_scratch_bytes(m, k) + 255) / 256 * 256, bytes = need + (size_t)(k + m) * ldn * es;
+  // in steps of 256 rows and columns, so that growing sizes do not each replace it
+  const size_t step = need + (size_t)(round_up(k, 256) + round_up(m, 256)) * round_up(n, 256) * es;
+  *ran = false;
+  if (!aligned_copy_fits(h->mpBC, h->mpBC_bytes, bytes)) return cudaSuccess;
+  if (ensure(&h->mpBC, &h->mpBC_bytes, h->mpBC_bytes >= bytes ? bytes : step) != cudaSuccess ||
+      (!h->mpBC_done && cudaEventCreateWithFlags(&h->mpBC_done, cudaEventDisableTiming) != cudaSuccess)) {
+    cudaGetLastError();  // out of memory: the kernel for any alignment
+    return cudaSuccess;
+  }
+  *ran = true;
+  char *Bc = static_cast<char *>(h->mpBC) + need, *Cc = Bc + (size_t)k * ldn * es;
+  int64_t l = 0;
+  cudaError_t e = cudaStreamWaitEvent(s, h->mpBC_done, 0);
+  if (e == cudaSuccess) e = apsp::launch_copy_rect(dtype, B, ldb, Bc, ldn, k, n, s, &l);
+  if (e == cudaSuccess) e = apsp::launch_copy_rect(dtype, C, ldc, Cc, ldn, m, n, s, &l);
+  if (e == cudaSuccess)
+    e = apsp::launch_minplus(dtype, A, lda, Bc, ldn, Cc, ldn, m, k, n, s, &l, h->mpBC, need, h->d_status);
+  if (e == cudaSuccess) e = apsp::launch_copy_rect(dtype, Cc, ldn, C, ldc, m, n, s, &l);
+  const cudaError_t er = cudaEventRecord(h->mpBC_done, s);
+  h->launches += l;
+  return e != cudaSuccess ? e : er;
+}
+
+// The product into C: the warp-specialized kernel with the handle's A^T workspace
+// when it can be had, else the one-CTA-per-tile kernel; for B and C without 16-byte
+// rows the former on copies where the product is large enough to pay for them.
+// h->mu held.
 static cudaError_t minplus_locked(apsp_handle *h, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb,
                                   void *C, int64_t ldc, int64_t m, int64_t k, int64_t n, cudaStream_t s) {
-  const size_t need = apsp::minplus_scratch_bytes(m, k);
+  const int64_t es = dtype == APSP_U16 ? 2 : 4;
+  auto rows16 = [es](const void *p, int64_t ld) {
+    return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld * es % 16 == 0;
+  };
+  const bool aligned = rows16(B, ldb) && rows16(C, ldc);
+  if (!aligned && k > 0 && (double)m * n * k >= kCopyProduct && !capturing(s)) {
+    bool ran = false;
+    const cudaError_t e = minplus_on_copies(h, dtype, A, lda, B, ldb, C, ldc, m, k, n, s, &ran);
+    if (e != cudaSuccess || ran) return e;
+  }
+  const size_t need = aligned ? apsp::minplus_scratch_bytes(m, k) : 0;
   void *scr = nullptr;
   if (need > 0) {
     if (ensure(&h->mpT, &h->mpT_bytes, need) == cudaSuccess) scr = h->mpT;
     else cudaGetLastError();  // out of memory: the kernel without workspace
   }
-  // B and C without 16-byte rows: the TMA-fed kernel on copies of them, where
-  // the product is large enough to pay for the two copies in and the one out
-  const int64_t es = dtype == APSP_U16 ? 2 : 4;
-  auto rows16 = [es](const void *p, int64_t ld) {
-    return reinterpret_cast<uintptr_t>(p) % 16 == 0 && ld * es % 16 == 0;
-  };
   int64_t l = 0;
-  cudaError_t e = cudaSuccess;
-  if (scr && k > 0 && !(rows16(B, ldb) && rows16(C, ldc)) && (double)m * n * k >= kCopyProduct &&
-      !capturing(s)) {
-    const int64_t ldn = round_up(n, 16 / es);
-    const size_t bytes = (size_t)(k + m) * ldn * es;
-    if (aligned_copy_fits(h->mpBC, h->mpBC_bytes, bytes)) {
-      if (ensure(&h->mpBC, &h->mpBC_bytes, bytes) == cudaSuccess) {
-        char *Bc = static_cast<char *>(h->mpBC), *Cc = Bc + (size_t)k * ldn * es;
-        e = apsp::launch_copy_rect(dtype, B, ldb, Bc, ldn, k, n, s, &l);
-        if (e == cudaSuccess) e = apsp::launch_copy_rect(dtype, C, ldc, Cc, ldn, m, n, s, &l);
-        if (e == cudaSuccess)
-          e = apsp::launch_minplus(dtype, A, lda, Bc, ldn, Cc, ldn, m, k, n, s, &l, scr, h->mpT_bytes, h->d_status);
-        if (e == cudaSuccess) e = apsp::launch_copy_rect(dtype, Cc, ldn, C, ldc, m, n, s, &l);
-        h->launches += l;
-        return e;
-      }
-      cudaGetLastError();  // out of memory: the kernel for any alignment
-    }
-  }
-  e = apsp::launch_minplus(dtype, A, lda, B, ldb, C, ldc, m, k, n, s, &l, scr, scr ? h->mpT_bytes : 0, h->d_status);
+  const cudaError_t e =
+      apsp::launch_minplus(dtype, A, lda, B, ldb, C, ldc, m, k, n, s, &l, scr, scr ? h->mpT_bytes : 0, h->d_status);
   h->launches += l;
   return e;
 }

@@ -1,5 +1,5 @@
-"""The copies with 16-byte rows that unaligned matrices and products run on (GPU): calls under stream capture
-and sequences of growing sizes."""
+"""The copies with 16-byte rows that unaligned matrices and products run on (GPU): calls under stream capture,
+on several streams, and in sequences of growing sizes."""
 import numpy as np
 import pytest
 
@@ -85,6 +85,31 @@ def test_unaligned_product_under_capture(lib):
         assert h.last_status() == 0
         np.testing.assert_array_equal(Cd.cpu().numpy(), oracle.minplus(A, B, C))
         del g
+
+
+@pytest.mark.parametrize("dtype", ["int32", "u16"])
+def test_unaligned_products_on_several_streams(lib, dtype):
+    """Products without 16-byte rows on two streams of one handle, between aligned ones: each is its own."""
+    rng = np.random.default_rng(8)
+    npdt = {"int32": np.int32, "u16": np.int16}[dtype]
+    jobs = []
+    for m, k, n in ((400, 300, 401), (600, 250, 301), (300, 500, 333), (700, 201, 255), (512, 512, 512)):
+        A, B, C = (rng.integers(0, 9000, size=x) for x in ((m, k), (k, n), (m, n)))
+        jobs.append((oracle.minplus(A, B, C), [torch.from_numpy(x.astype(npdt)).cuda() for x in (A, B, C)]))
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    with lib.Handle(device=0) as h:
+        for rep in range(20):
+            outs = []
+            for i, (E, (A, B, C)) in enumerate(jobs[:4]):
+                with torch.cuda.stream(streams[i % 2]):
+                    outs.append((E, h.minplus(A, B, C.clone())))
+            with torch.cuda.stream(streams[0]):  # 16-byte rows: the handle's own A^T
+                E, (A, B, C) = jobs[4]
+                outs.append((E, h.minplus(A, B, C.clone())))
+            torch.cuda.synchronize()
+            for E, D in outs:
+                np.testing.assert_array_equal(D.cpu().numpy().astype(np.int64), E)
 
 
 def test_growing_unaligned_sizes_reuse_the_copy(lib):
